@@ -4,17 +4,19 @@
 //   m = max_v l_v, id = the lowest v with l_v = m,
 //   conf = max_v softmax(l)_v = 1 / sum_v exp(l_v - m).
 // A row is cut into `split` pieces, one CTA each (a thread-block cluster when
-// split > 1). Pieces of at most 2048 vectors (a few rows over many SMs, as
-// in a decode step) take logits_argmax_small_kernel: every thread loads its
-// vectors at once and folds them in one pass. Larger pieces stream: in a CTA
-// one producer warp streams the piece through a ring of
-// 16 KB stages with bulk copies (TMA engine) and eight warps fold each 8-logit
-// vector into a running (max, sum of exp(l - max), argmax): the vector max
-// comes first, so the rare rescale happens once per vector, then one exp per
-// logit. The partial states merge by the log-sum-exp rule (ties: the lower
-// index) across the warps, the CTA and, through distributed shared memory,
-// the cluster. NaN logits never win the argmax and make the sum NaN; a row
-// with nothing above -inf gets id 0 and confidence 0.
+// split > 1). Pieces of at most 4096 vectors of 8 logits (vocabularies up to
+// 262144) are kept in registers: every thread loads its vectors at once and
+// folds them in one pass. Longer pieces stream: in a CTA one producer warp
+// streams the piece through a ring of 16 KB stages with bulk copies (TMA
+// engine) and eight warps fold each 8-logit vector into a running (max, sum
+// of exp(l - max), argmax): the vector max comes first, so the rare rescale
+// happens once per vector, then one exp per logit. The partial states merge
+// by the log-sum-exp rule (ties: the lower index) across the warps, the CTA
+// and, through distributed shared memory, the cluster. NaN logits never win
+// the argmax and make the sum NaN; a row with nothing above -inf gets id 0
+// and confidence 0.
+#include <limits.h>
+
 #include "nld_internal.cuh"
 
 namespace nld {
@@ -213,22 +215,31 @@ __global__ void __launch_bounds__(kLgThreads)
   }
 }
 
-// Small pieces (at most kLsThreads * kLsMaxVecs 8-logit vectors per CTA: a
-// few rows over many SMs, the decode-step case): no ring. Every thread loads
-// all its vectors at once (one memory round trip), folds them in one pass
-// (the max of its logits first, then one exp per logit against it), and
-// the CTA merges the threads' states; the pieces of a row then push their
-// states into rank 0's shared memory with a remote store and a release
-// arrival on rank 0's mbarrier, and rank 0 merges them, so no peer waits
-// for another. Same rules as logits_argmax_kernel (ties to the lower index;
-// NaN never wins and makes the sum NaN; nothing above -inf: id 0, conf 0).
-constexpr int kLsThreads = 256;  // light enough for two CTAs per SM, so every cluster of 8 is resident at once
+// Pieces that fit in a CTA's registers (at most THREADS * kLsMaxVecs 8-logit
+// vectors): no ring. Every thread loads all its vectors at once (one memory
+// round trip); the logits' max is taken on packed bf16 pairs, then one exp
+// per logit against the warp's max; the index of the max is searched only by
+// the warps that hold the CTA's. The pieces of a row push their states into
+// rank 0's shared memory with a remote store and a release arrival on rank
+// 0's mbarrier, and rank 0 merges them, so no peer waits for another. Same
+// rules as logits_argmax_kernel (ties to the lower index; NaN never wins and
+// makes the sum NaN; nothing above -inf: id 0, conf 0).
+// Bound: few rows, the chain load - exps - three merges; many rows,
+// instruction issue (51% of the cycles, 7.4 instructions a logit) and CTAs
+// that hold their slots through the merges, at 16 rows x 131072 3.6 us (a
+// per-logit max and index search: 4.6), at 512 rows 25.9 us = 5.2 TB/s (the
+// streaming kernel, one CTA a row: 34.7, its 512 CTAs being 1.1 waves), at
+// 1024 rows 47 us = 5.7 TB/s (55). Measured and left out: clusters that stay
+// and prefetch the next row's vectors (32 us at 512 rows: one chain per row),
+// clusters that stream several rows through a ring (28.7 us), the exponent as
+// one FMA against an integer reference (28.6 us: paired subtract and multiply
+// take fewer issue slots).
 constexpr int kLsMaxVecs = 8;  // vectors a thread holds in flight
 
 __device__ __forceinline__ void cluster_arrive_relaxed() {
   asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void st_dsmem_f32(uint32_t addr, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
@@ -255,136 +266,206 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
   }
 }
 
-__global__ void __launch_bounds__(kLsThreads)
-    logits_argmax_small_kernel(const __nv_bfloat16* __restrict__ logits, int vocab, long ld, int split,
+// Warp max of values that are never NaN.
+__device__ __forceinline__ float warp_max(float x) {
+  const int b = __float_as_int(x);
+  const int k = __reduce_max_sync(0xffffffffu, b ^ ((b >> 31) & 0x7fffffff));  // signed order of the floats
+  return __int_as_float(k ^ ((k >> 31) & 0x7fffffff));
+}
+
+// Merge the (m, s, i) states of a warp's lanes: the max, the sums rescaled to
+// it, the lowest index holding it; every lane returns the merged state. m is
+// never NaN; a state whose m is -inf has s 0, or NaN if it met a NaN logit.
+__device__ __forceinline__ void lg_warp_merge(float& m, float& s, int& i) {
+  const float mm = warp_max(m);
+  if (m != -INFINITY) s *= ex2((m - mm) * kLog2e);
+  i = static_cast<int>(__reduce_min_sync(0xffffffffu, static_cast<unsigned>(m == mm ? i : INT_MAX)));
+  m = mm;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+}
+
+// 8 logits of a vector as packed bf16 pairs: their max, per half.
+__device__ __forceinline__ uint32_t bf16x2_max(uint32_t a, uint32_t b) {
+  const __nv_bfloat162 r =
+      __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
+  return *reinterpret_cast<const uint32_t*>(&r);  // a NaN operand gives the other one
+}
+__device__ __forceinline__ uint32_t vec_max(uint4 w) { return bf16x2_max(bf16x2_max(w.x, w.y), bf16x2_max(w.z, w.w)); }
+
+constexpr uint32_t kNegInf2 = 0xFF80FF80u;  // two bf16 -inf
+
+// Row vectors v0 + t + j*THREADS < v1 into w, all loads in flight (-inf past
+// v1; rows are readable to a multiple of 8).
+template <int THREADS, int VECS>
+__device__ __forceinline__ void load_logit_vecs(const uint4* row, int v0, int v1, int t, uint4 (&w)[VECS]) {
+#pragma unroll
+  for (int j = 0; j < VECS; ++j) {
+    const int v = v0 + t + j * THREADS;
+    w[j] = v < v1 ? __ldg(row + v) : make_uint4(kNegInf2, kNegInf2, kNegInf2, kNegInf2);
+  }
+}
+
+// -inf past the vocabulary in a last vector that it does not fill. Apart from
+// the loads: a branch on the loaded values would wait for them.
+template <int THREADS, int VECS>
+__device__ __forceinline__ void mask_last_vec(int v0, int v1, int t, int vocab, uint4 (&w)[VECS]) {
+  if (v1 * 8 > vocab && (v1 - 1 - v0 - t) % THREADS == 0) {  // this thread holds the partial last vector
+#pragma unroll
+    for (int j = 0; j < VECS; ++j)
+      if (v0 + t + j * THREADS == v1 - 1) {
+        uint32_t q[4] = {w[j].x, w[j].y, w[j].z, w[j].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int first = (v1 - 1) * 8 + 2 * e;  // the pair's first logit
+          if (first >= vocab) q[e] = kNegInf2;
+          else if (first + 1 == vocab) q[e] = (q[e] & 0xFFFFu) | (kNegInf2 & 0xFFFF0000u);
+        }
+        w[j] = make_uint4(q[0], q[1], q[2], q[3]);
+      }
+  }
+}
+
+// acc += exp(x - m) over the 8 logits of w, m finite: a pair of logits takes
+// two widenings, a paired subtract, multiply and add and two exponentials (4
+// cycles of the MUFU pipe per warp instruction here).
+__device__ __forceinline__ void add_exps(uint4 w, float m, float2& acc) {
+  const uint32_t q[4] = {w.x, w.y, w.z, w.w};
+  const float2 nm = make_float2(-m, -m), l2 = make_float2(kLog2e, kLog2e);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    float2 x;
+    unpack_bf16(q[j], x.x, x.y);
+    x = mul2(add2(x, nm), l2);
+    acc = add2(acc, make_float2(ex2(x.x), ex2(x.y)));
+  }
+}
+
+// Position (from the first vector's start) of the first logit equal to m
+// among vectors w (their per-half maxima in vm), vector j starting at j*STRIDE;
+// some logit is m.
+template <int STRIDE, int VECS>
+__device__ __forceinline__ int first_of_max(const uint4 (&w)[VECS], const uint32_t (&vm)[VECS], float m) {
+  int jb = 0;
+  uint4 wb = w[0];
+  float lo, hi;
+#pragma unroll
+  for (int j = VECS - 1; j >= 0; --j) {
+    unpack_bf16(vm[j], lo, hi);
+    if (lo == m || hi == m) {
+      jb = j;
+      wb = w[j];
+    }
+  }
+  const uint32_t q[4] = {wb.x, wb.y, wb.z, wb.w};
+  int e = 0;
+#pragma unroll
+  for (int j = 3; j >= 0; --j) {
+    unpack_bf16(q[j], lo, hi);
+    if (hi == m) e = 2 * j + 1;
+    if (lo == m) e = 2 * j;
+  }
+  return jb * STRIDE + e;
+}
+
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS)
+    logits_argmax_small_kernel(const __nv_bfloat16* __restrict__ logits, int vocab, long ld, int log2_split, int per,
                                int32_t* __restrict__ ids, float* __restrict__ conf, unsigned int* err) {
-  __shared__ float red[kLsThreads / 32][3];
+  constexpr int kW = THREADS / 32;
+  __shared__ float red_m[kW], red_s[kW];
+  __shared__ int first;          // the lowest index holding this CTA's max
   __shared__ float parts[8][3];  // rank 0: the pieces' (m, s, id)
   __shared__ __align__(8) uint64_t arrived;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = threadIdx.x;
-  const int piece = static_cast<int>(blockIdx.x % split);
-  const long row = static_cast<long>(blockIdx.x / split);
-  const int nvec = vocab >> 3, tail = vocab & 7;
-  const int per = (nvec + split - 1) / split;
+  const int split = 1 << log2_split;
+  const int piece = static_cast<int>(blockIdx.x) & (split - 1);
+  const long row = static_cast<long>(blockIdx.x >> log2_split);
+  const int nvec = (vocab + 7) >> 3;
   const int v0 = min(nvec, piece * per), v1 = min(nvec, v0 + per);
-  if (split > 1) {
-    if (t == 0) {
+  if (t == 0) {
+    first = INT_MAX;
+    if (split > 1) {
       mbar_init(&arrived, static_cast<uint32_t>(split));
       fence_mbar_init();
     }
-    cluster_arrive_relaxed();  // rank 0's barrier is ready once every CTA has arrived (waited below)
   }
-  grid_launch_dependents();  // dependents launch early; they wait on this grid themselves
-  grid_dependency_wait();    // the logits come from the previous kernel
+  if (split > 1) cluster_arrive_relaxed();  // rank 0's barrier is ready once every CTA has arrived (waited below)
+  grid_launch_dependents();                 // dependents launch early; they wait on this grid themselves
+  grid_dependency_wait();                   // the logits come from the previous kernel
   const uint4* grow = reinterpret_cast<const uint4*>(logits + row * ld);
   uint4 w[kLsMaxVecs];
+  load_logit_vecs<THREADS>(grow, v0, v1, t, w);
+  mask_last_vec<THREADS>(v0, v1, t, vocab, w);
+  // the max of this thread's logits (NaN is passed over), then of the warp's
+  uint32_t vm[kLsMaxVecs];
+  uint32_t pm = kNegInf2;
 #pragma unroll
   for (int j = 0; j < kLsMaxVecs; ++j) {
-    const int v = v0 + t + j * kLsThreads;
-    w[j] = v < v1 ? __ldg(grow + v) : make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);  // -inf
+    vm[j] = vec_max(w[j]);
+    pm = bf16x2_max(pm, vm[j]);
   }
-  // max of this thread's logits and the lowest index holding it
-  float m = -INFINITY;
-  int idx = 0;
+  float lo, hi;
+  unpack_bf16(pm, lo, hi);
+  const float mt = fmaxf(lo, hi);
+  const float mw = warp_max(mt);
+  // one exp per logit against the warp's max, so the lanes' sums just add
+  float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  const float mref = mw == -INFINITY ? 0.f : mw;
 #pragma unroll
-  for (int j = 0; j < kLsMaxVecs; ++j) {
-    float x[8];
-    unpack_bf16(w[j].x, x[0], x[1]);
-    unpack_bf16(w[j].y, x[2], x[3]);
-    unpack_bf16(w[j].z, x[4], x[5]);
-    unpack_bf16(w[j].w, x[6], x[7]);
-    const int e0 = (v0 + t + j * kLsThreads) * 8;
+  for (int j = 0; j < kLsMaxVecs; ++j) add_exps(w[j], mref, acc[j & 1]);
+  float s = (acc[0].x + acc[0].y) + (acc[1].x + acc[1].y);
 #pragma unroll
-    for (int e = 0; e < 8; ++e)
-      if (x[e] > m) {  // strictly greater: the first (lowest) index of the max stays; NaN never is
-        m = x[e];
-        idx = e0 + e;
-      }
-  }
-  float s = 0.f;
-#pragma unroll
-  for (int j = 0; j < kLsMaxVecs; ++j) {
-    float x[8];
-    unpack_bf16(w[j].x, x[0], x[1]);
-    unpack_bf16(w[j].y, x[2], x[3]);
-    unpack_bf16(w[j].z, x[4], x[5]);
-    unpack_bf16(w[j].w, x[6], x[7]);
-    if (m != -INFINITY) {
-#pragma unroll
-      for (int e = 0; e < 8; ++e) s += ex2((x[e] - m) * kLog2e);  // padding (-inf) adds 0; a NaN makes s NaN
-    } else {
-#pragma unroll
-      for (int e = 0; e < 8; ++e)
-        if (isnan(x[e])) s = NAN;
-    }
-  }
-  if (piece == split - 1 && t < tail) {  // the last vocab % 8 logits
-    const uint16_t bits = reinterpret_cast<const uint16_t*>(logits + row * ld)[nvec * 8 + t];
-    const float x[1] = {__uint_as_float(static_cast<uint32_t>(bits) << 16)};
-    lg_fold(x, nvec * 8 + t, m, s, idx);
-  }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
-    const float s2 = __shfl_xor_sync(0xffffffffu, s, off);
-    const int i2 = __shfl_xor_sync(0xffffffffu, idx, off);
-    lg_merge(m, s, idx, m2, s2, i2);
-  }
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
   if (lane == 0) {
-    red[warp][0] = m;
-    red[warp][1] = s;
-    red[warp][2] = __int_as_float(idx);
+    red_m[warp] = mw;
+    red_s[warp] = s;
   }
   __syncthreads();
+  // the CTA's max; its first index is searched only by the warps that hold it
+  const float ml = lane < kW ? red_m[lane] : -INFINITY;
+  const float m = warp_max(ml);
+  if (mt == m && m != -INFINITY)
+    atomicMin(&first, (v0 + t) * 8 + first_of_max<THREADS * 8>(w, vm, m));
   if (warp == 0) {
-    constexpr int kW = kLsThreads / 32;
-    m = lane < kW ? red[lane][0] : -INFINITY;
-    s = lane < kW ? red[lane][1] : 0.f;
-    idx = lane < kW ? __float_as_int(red[lane][2]) : 0;
+    s = lane < kW ? red_s[lane] : 0.f;
+    if (ml != -INFINITY) s *= ex2((ml - m) * kLog2e);  // a warp without finite logits has sum 0 or NaN
 #pragma unroll
-    for (int off = kW / 2; off > 0; off >>= 1) {
-      const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
-      const float s2 = __shfl_xor_sync(0xffffffffu, s, off);
-      const int i2 = __shfl_xor_sync(0xffffffffu, idx, off);
-      lg_merge(m, s, idx, m2, s2, i2);
-    }
-    if (split == 1 && lane == 0) {
+    for (int off = kW / 2; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  }
+  __syncthreads();
+  int idx = m == -INFINITY ? 0 : first;
+  if (split == 1) {
+    if (t == 0) {
       ids[row] = idx;
       conf[row] = m == -INFINITY ? 0.f : 1.f / s;
     }
+    return;
   }
-  if (split > 1) {
-    cluster_wait();
-    if (t == 0) {
-      const uint32_t slot = smem_u32(&parts[piece][0]);
-      st_dsmem_f32(dsmem_addr(slot, 0), m);
-      st_dsmem_f32(dsmem_addr(slot + 4, 0), s);
-      st_dsmem_f32(dsmem_addr(slot + 8, 0), __int_as_float(idx));
-      mbar_arrive_remote_release(dsmem_addr(smem_u32(&arrived), 0));
+  cluster_wait();
+  if (t == 0) {
+    const uint32_t slot = dsmem_addr(smem_u32(&parts[piece][0]), 0);
+    st_dsmem_f32(slot, m);
+    st_dsmem_f32(slot + 4, s);
+    st_dsmem_f32(slot + 8, __int_as_float(idx));
+    mbar_arrive_remote_release(dsmem_addr(smem_u32(&arrived), 0));
+  }
+  if (piece == 0 && warp == 0) {
+    bool ok = true;
+    if (lane == 0) ok = mbar_wait_cluster(&arrived, 0, err);
+    ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+    float mr = -INFINITY;
+    s = 0.f;
+    idx = 0;
+    if (ok && lane < split) {
+      mr = parts[lane][0];
+      s = parts[lane][1];
+      idx = __float_as_int(parts[lane][2]);
     }
-    if (cluster_ctarank() == 0 && warp == 0) {
-      bool ok = true;
-      if (lane == 0) ok = mbar_wait_cluster(&arrived, 0, err);
-      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-      m = -INFINITY;
-      s = 0.f;
-      idx = 0;
-      if (ok && lane < split) {
-        m = parts[lane][0];
-        s = parts[lane][1];
-        idx = __float_as_int(parts[lane][2]);
-      }
-#pragma unroll
-      for (int off = 4; off > 0; off >>= 1) {
-        const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
-        const float s2 = __shfl_xor_sync(0xffffffffu, s, off);
-        const int i2 = __shfl_xor_sync(0xffffffffu, idx, off);
-        lg_merge(m, s, idx, m2, s2, i2);
-      }
-      if (lane == 0 && ok) {
-        ids[row] = idx;
-        conf[row] = m == -INFINITY ? 0.f : 1.f / s;
-      }
+    lg_warp_merge(mr, s, idx);
+    if (lane == 0 && ok) {
+      ids[row] = idx;
+      conf[row] = mr == -INFINITY ? 0.f : 1.f / s;
     }
   }
 }
@@ -585,6 +666,7 @@ __global__ void __launch_bounds__(kEnThreads)
 }  // namespace
 
 int logits_split_vectors() { return kLgStageVecs; }
+int logits_piece_limit() { return 512 * kLsMaxVecs; }
 
 cudaError_t launch_ensemble_argmax(const __nv_bfloat16* ar, const __nv_bfloat16* diff, int rows, int vocab, long ld,
                                    int split, float lambda, int32_t* ids, float* conf, cudaStream_t stream) {
@@ -606,10 +688,14 @@ cudaError_t launch_logits_argmax(const __nv_bfloat16* logits, int rows, int voca
     __atomic_store_n(&configured[dev], 1, __ATOMIC_RELEASE);
   }
   const dim3 grid(static_cast<unsigned>(static_cast<long>(rows) * split));
-  const long piece_vecs = ((vocab >> 3) + split - 1) / split;
-  if (piece_vecs <= static_cast<long>(kLsThreads) * kLsMaxVecs)
-    return launch_kernel_cluster(logits_argmax_small_kernel, grid, dim3(kLsThreads), 0, stream, split, logits, vocab,
-                                 ld, split, ids, conf, err);
+  const long piece_vecs = ((static_cast<long>(vocab) + 7) / 8 + split - 1) / split;
+  const int log2_split = __builtin_ctz(static_cast<unsigned>(split));
+  if (piece_vecs <= 256L * kLsMaxVecs)
+    return launch_kernel_cluster(logits_argmax_small_kernel<256>, grid, dim3(256), 0, stream, split, logits, vocab, ld,
+                                 log2_split, static_cast<int>(piece_vecs), ids, conf, err);
+  if (piece_vecs <= 512L * kLsMaxVecs)
+    return launch_kernel_cluster(logits_argmax_small_kernel<512>, grid, dim3(512), 0, stream, split, logits, vocab, ld,
+                                 log2_split, static_cast<int>(piece_vecs), ids, conf, err);
   return launch_kernel_cluster(logits_argmax_kernel, grid, dim3(kLgThreads), kLgSmemBytes, stream, split, logits,
                                vocab, ld, split, ids, conf, err);
 }

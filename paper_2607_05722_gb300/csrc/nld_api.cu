@@ -269,6 +269,28 @@ nld_status_t encode_out_map(CUtensorMap* map, const nld::AttnArgs& a, int D) {
   return r == CUDA_SUCCESS ? NLD_OK : NLD_ERR_CUDA;
 }
 
+// Pieces (CTAs of one cluster, 1..8) per row of the logits kernels. With fewer
+// rows than SMs: enough to fill the SMs once, of at least 1024 vectors of 8
+// logits each. Then, with any number of rows, as many as bring a piece down to
+// `fit` vectors, what the kernels that keep a piece in registers take with
+// their smallest CTAs, where 8 pieces can be kept in registers at all: at 128
+// rows x 131072 pieces of 2048 vectors take 9.3 us, whole rows streamed 21.9;
+// more pieces than that only add merges (512 rows x 32000: 2 pieces 8.9 us, 4
+// pieces 12.2).
+int logits_split(int rows, int vocab, int sms, int fit) {
+  int split = 1;
+  if (rows < sms) {
+    const int by_sms = sms / rows;
+    const int by_len = (vocab / 8) / nld::logits_split_vectors();
+    const int want = by_sms < by_len ? by_sms : by_len;
+    while (split * 2 <= want && split * 2 <= 8) split *= 2;
+  }
+  const long nvec = (static_cast<long>(vocab) + 7) / 8;
+  if (nvec <= 8L * nld::logits_piece_limit())
+    while (split < 8 && nvec > static_cast<long>(split) * fit) split *= 2;
+  return split;
+}
+
 }  // namespace
 
 namespace nld {
@@ -536,15 +558,7 @@ nld_status_t nld_logits_argmax(const void* logits, int rows, int vocab, int ld, 
   int sms = 0;
   nld_status_t st = device_state(&err, &sms);
   if (st != NLD_OK) return st;
-  // Pieces per row: fill the SMs once when there are fewer rows than SMs, at
-  // least one ring stage of vectors a piece, at most one cluster of 8.
-  int split = 1;
-  if (rows < sms) {
-    const int by_sms = sms / rows;
-    const int by_len = (vocab / 8) / nld::logits_split_vectors();
-    const int want = by_sms < by_len ? by_sms : by_len;
-    while (split * 2 <= want && split * 2 <= 8) split *= 2;
-  }
+  const int split = logits_split(rows, vocab, sms, 2048);
   return nld::launch_logits_argmax(static_cast<const __nv_bfloat16*>(logits), rows, vocab, ld, split, ids, conf, err,
                                    stream) == cudaSuccess
              ? NLD_OK

@@ -315,6 +315,27 @@ def test_logits_matches_oracle(orc, rows, vocab, ld):
     check_logits(gpu_logits(bits, vocab), orc.logits_argmax(bits, vocab), f"rows={rows} V={vocab} ld={ld}")
 
 
+@pytest.mark.parametrize("rows,vocab", [(200, 131072), (3, 131073), (3, 262144), (3, 262145), (400, 16384),
+                                        (2, 16385), (160, 40001)])
+def test_logits_register_pieces(orc, rows, vocab):
+    """Sizes at the edges of the register kernels' pieces (2048 and 4096
+    vectors a CTA, then the ring), with logits masked by the lowest bf16
+    value, ties across pieces and a NaN in the last, partial vector."""
+    rng = np.random.default_rng(vocab)
+    ld = (vocab + 7) // 8 * 8
+    x = (rng.standard_normal((rows, ld)) * 3.0).astype(np.float32)
+    x[:, vocab:] = 1e4  # padding past vocab must never count
+    low = W.bf16_bits_to_f32(np.array([0xFF7F], np.uint16))[0]
+    x[0, : vocab - 1] = low                                       # one logit above the masked ones
+    x[1, :vocab] = low                                            # all masked alike: id 0
+    x[-1, vocab // 3] = x[-1, vocab - 1] = 30.0                   # a tie between pieces: the lower index
+    if rows > 3:
+        x[2, vocab - 1] = np.nan
+        x[3, :vocab] += 7e4                                       # large logits: differences of bf16 steps
+    bits = W.f32_to_bf16_bits(x)
+    check_logits(gpu_logits(bits, vocab), orc.logits_argmax(bits, vocab), f"rows={rows} V={vocab}")
+
+
 def gpu_ensemble(a_bits, d_bits, lam, vocab=None):
     rows = a_bits.shape[0]
     ta = torch.from_numpy(np.ascontiguousarray(a_bits).view(np.int16)).view(torch.bfloat16).cuda()
