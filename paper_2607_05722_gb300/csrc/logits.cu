@@ -663,14 +663,224 @@ __global__ void __launch_bounds__(kEnThreads)
   }
 }
 
+// The same for pieces that fit in a CTA's registers (both rows' vectors of a
+// thread, VECS each): the logits are read once. Pass 1 as in
+// logits_argmax_small_kernel; each piece pushes its (max, sum) pairs to every
+// CTA of the cluster (remote stores, release arrivals), so the totals take
+// one hop; pass 2 evaluates p only where it can be the maximum. With
+// ca = lambda / sum_a, cb = (1 - lambda) / sum_b, the largest p is at least
+// c = max(ca, cb), its value at that row's own maximum, so a vector whose
+// terms ca exp(a - max_a) and cb exp(b - max_b) all lie below 0.49 c cannot
+// hold it: two compares of a vector's maxima decide.
+// Bound by the chain load - sums - exchange - best, during which a CTA holds
+// its registers (ncu at 160 row pairs: 41% of issue cycles, waits at CTA
+// barriers first): 160 x 100003 25.1 us (reading both rows twice, with two
+// exponentials a logit each time: 54.6), 16 x 131072 5.5 us (12.7), 512 x
+// 131072 74 us (132).
+template <int THREADS, int VECS>
+__global__ void __launch_bounds__(THREADS, VECS == 4 ? 1024 / THREADS : 1)
+    ensemble_argmax_small_kernel(const __nv_bfloat16* __restrict__ ar, const __nv_bfloat16* __restrict__ diff,
+                                 int vocab, long ld, int log2_split, int per, float lambda, int32_t* __restrict__ ids,
+                                 float* __restrict__ conf, unsigned int* err) {
+  constexpr int kW = THREADS / 32;
+  __shared__ float red[kW][4];       // the warps' m_a, s_a, m_b, s_b, then their (p, index)
+  __shared__ float totals[8][4];     // the pieces' m_a, s_a, m_b, s_b
+  __shared__ float whole[4];         // the row pair's
+  __shared__ float best[8][2];       // rank 0: the pieces' (p, index)
+  __shared__ __align__(8) uint64_t have_totals, have_best;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = threadIdx.x;
+  const int split = 1 << log2_split;
+  const int piece = static_cast<int>(blockIdx.x) & (split - 1);
+  const long row = static_cast<long>(blockIdx.x >> log2_split);
+  const int nvec = (vocab + 7) >> 3;
+  const int v0 = min(nvec, piece * per), v1 = min(nvec, v0 + per);
+  if (split > 1) {
+    if (t == 0) {
+      mbar_init(&have_totals, static_cast<uint32_t>(split));
+      mbar_init(&have_best, static_cast<uint32_t>(split));
+      fence_mbar_init();
+    }
+    cluster_arrive_relaxed();  // the barriers are ready once every CTA has arrived (waited below)
+  }
+  grid_launch_dependents();
+  grid_dependency_wait();  // the logits come from earlier kernels
+  uint4 wa[VECS], wb[VECS];
+  load_logit_vecs<THREADS>(reinterpret_cast<const uint4*>(ar + row * ld), v0, v1, t, wa);
+  load_logit_vecs<THREADS>(reinterpret_cast<const uint4*>(diff + row * ld), v0, v1, t, wb);
+
+  // ---- pass 1: (max, sum) of each row over this piece ----
+  auto fold = [&](uint4(&w)[VECS], float& m, float& s) {
+    mask_last_vec<THREADS>(v0, v1, t, vocab, w);
+    uint32_t pm = kNegInf2;
+#pragma unroll
+    for (int j = 0; j < VECS; ++j) pm = bf16x2_max(pm, vec_max(w[j]));
+    float lo, hi;
+    unpack_bf16(pm, lo, hi);
+    m = warp_max(fmaxf(lo, hi));
+    float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    const float mref = m == -INFINITY ? 0.f : m;
+#pragma unroll
+    for (int j = 0; j < VECS; ++j) add_exps(w[j], mref, acc[j & 1]);
+    s = (acc[0].x + acc[0].y) + (acc[1].x + acc[1].y);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  };
+  // the lanes' states of one row merged: the max, and the sum rescaled to it
+  auto merge = [](float& m, float& s) {
+    const float mm = warp_max(m);
+    if (m != -INFINITY) s *= ex2((m - mm) * kLog2e);
+    m = mm;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  };
+  float ma, sa, mb, sb;
+  fold(wa, ma, sa);
+  fold(wb, mb, sb);
+  if (lane == 0) {
+    red[warp][0] = ma; red[warp][1] = sa; red[warp][2] = mb; red[warp][3] = sb;
+  }
+  __syncthreads();
+  bool ok = true;
+  if (split > 1) cluster_wait();
+  if (warp == 0) {
+    ma = lane < kW ? red[lane][0] : -INFINITY;
+    sa = lane < kW ? red[lane][1] : 0.f;
+    mb = lane < kW ? red[lane][2] : -INFINITY;
+    sb = lane < kW ? red[lane][3] : 0.f;
+    merge(ma, sa);
+    merge(mb, sb);
+    if (split > 1) {
+      if (lane < split) {  // to every CTA of the cluster
+        const uint32_t slot = dsmem_addr(smem_u32(&totals[piece][0]), lane);
+        st_dsmem_f32(slot, ma);
+        st_dsmem_f32(slot + 4, sa);
+        st_dsmem_f32(slot + 8, mb);
+        st_dsmem_f32(slot + 12, sb);
+        mbar_arrive_remote_release(dsmem_addr(smem_u32(&have_totals), lane));
+      }
+      __syncwarp();
+      if (lane == 0) ok = mbar_wait_cluster(&have_totals, 0, err);
+      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+      ma = -INFINITY; sa = 0.f; mb = -INFINITY; sb = 0.f;
+      if (ok && lane < split) {
+        ma = totals[lane][0]; sa = totals[lane][1]; mb = totals[lane][2]; sb = totals[lane][3];
+      }
+      merge(ma, sa);
+      merge(mb, sb);
+    }
+    if (lane == 0) {
+      whole[0] = ma; whole[1] = sa; whole[2] = mb; whole[3] = sb;
+    }
+  }
+  __syncthreads();
+  ma = whole[0]; sa = whole[1]; mb = whole[2]; sb = whole[3];
+  // An empty distribution (max -inf) gets weight 0 and a stand-in max of 0,
+  // so its terms are exp(-inf) * 0 = 0.
+  const float ca = ma == -INFINITY ? 0.f : lambda / sa;
+  const float cb = mb == -INFINITY ? 0.f : (1.f - lambda) / sb;
+  ma = ma == -INFINITY ? 0.f : ma;
+  mb = mb == -INFINITY ? 0.f : mb;
+
+  // ---- pass 2: the lowest-index maximum of p over this piece ----
+  const float c = 0.49f * fmaxf(ca, cb);
+  const float da = lg2(c / ca) * kLn2, db = lg2(c / cb) * kLn2;  // NaN when both rows are empty: every vector is taken
+  float pbest = -1.f;
+  int ibest = 0;
+  unsigned take = 0;
+#pragma unroll
+  for (int j = 0; j < VECS; ++j) {
+    float lo, hi;
+    unpack_bf16(vec_max(wa[j]), lo, hi);
+    const float xa = fmaxf(lo, hi);
+    unpack_bf16(vec_max(wb[j]), lo, hi);
+    const float xb = fmaxf(lo, hi);
+    if (!(xa - ma < da && xb - mb < db)) take |= 1u << j;
+  }
+#pragma unroll 1
+  for (; take != 0; take &= take - 1) {  // few vectors, in index order
+    const int jt = __ffs(take) - 1;
+    uint4 va = wa[0], vb = wb[0];
+#pragma unroll
+    for (int j = 1; j < VECS; ++j)
+      if (j == jt) {
+        va = wa[j];
+        vb = wb[j];
+      }
+    const uint32_t qa[4] = {va.x, va.y, va.z, va.w}, qb[4] = {vb.x, vb.y, vb.z, vb.w};
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const uint32_t ba = qa[e >> 1], bb = qb[e >> 1];
+      const float a = __uint_as_float((e & 1) ? ba & 0xFFFF0000u : ba << 16);
+      const float b = __uint_as_float((e & 1) ? bb & 0xFFFF0000u : bb << 16);
+      const float p = ca * ex2((a - ma) * kLog2e) + cb * ex2((b - mb) * kLog2e);
+      if (p > pbest) {
+        pbest = p;
+        ibest = (v0 + t + jt * THREADS) * 8 + e;
+      }
+    }
+  }
+  // the lanes' best: the largest p, its lowest index
+  auto best_of = [](float& p, int& i) {
+    const float pp = warp_max(p);
+    i = static_cast<int>(__reduce_min_sync(0xffffffffu, static_cast<unsigned>(p == pp ? i : INT_MAX)));
+    p = pp;
+  };
+  best_of(pbest, ibest);
+  if (lane == 0) {
+    red[warp][0] = pbest;
+    red[warp][1] = __int_as_float(ibest);
+  }
+  __syncthreads();
+  if (warp != 0) return;
+  pbest = lane < kW ? red[lane][0] : -1.f;
+  ibest = lane < kW ? __float_as_int(red[lane][1]) : 0;
+  best_of(pbest, ibest);
+  if (split > 1) {
+    if (lane == 0) {
+      const uint32_t slot = dsmem_addr(smem_u32(&best[piece][0]), 0);
+      st_dsmem_f32(slot, pbest);
+      st_dsmem_f32(slot + 4, __int_as_float(ibest));
+      mbar_arrive_remote_release(dsmem_addr(smem_u32(&have_best), 0));
+    }
+    if (piece != 0) return;
+    __syncwarp();
+    bool got = true;
+    if (lane == 0) got = mbar_wait_cluster(&have_best, 0, err);
+    ok = ok && __shfl_sync(0xffffffffu, got ? 1 : 0, 0) != 0;
+    pbest = -1.f;
+    ibest = 0;
+    if (ok && lane < split) {
+      pbest = best[lane][0];
+      ibest = __float_as_int(best[lane][1]);
+    }
+    best_of(pbest, ibest);
+  }
+  if (lane == 0 && ok) {
+    ids[row] = ibest;
+    conf[row] = pbest;
+  }
+}
+
 }  // namespace
 
 int logits_split_vectors() { return kLgStageVecs; }
 int logits_piece_limit() { return 512 * kLsMaxVecs; }
 
 cudaError_t launch_ensemble_argmax(const __nv_bfloat16* ar, const __nv_bfloat16* diff, int rows, int vocab, long ld,
-                                   int split, float lambda, int32_t* ids, float* conf, cudaStream_t stream) {
+                                   int split, float lambda, int32_t* ids, float* conf, unsigned int* err,
+                                   cudaStream_t stream) {
   const dim3 grid(static_cast<unsigned>(static_cast<long>(rows) * split));
+  const long piece_vecs = ((static_cast<long>(vocab) + 7) / 8 + split - 1) / split;
+  const int log2_split = __builtin_ctz(static_cast<unsigned>(split)), per = static_cast<int>(piece_vecs);
+  if (piece_vecs <= 256 * 4)
+    return launch_kernel_cluster(ensemble_argmax_small_kernel<256, 4>, grid, dim3(256), 0, stream, split, ar, diff,
+                                 vocab, ld, log2_split, per, lambda, ids, conf, err);
+  if (piece_vecs <= 512 * 4)
+    return launch_kernel_cluster(ensemble_argmax_small_kernel<512, 4>, grid, dim3(512), 0, stream, split, ar, diff,
+                                 vocab, ld, log2_split, per, lambda, ids, conf, err);
+  if (piece_vecs <= 512 * 8)
+    return launch_kernel_cluster(ensemble_argmax_small_kernel<512, 8>, grid, dim3(512), 0, stream, split, ar, diff,
+                                 vocab, ld, log2_split, per, lambda, ids, conf, err);
   return launch_kernel_cluster(ensemble_argmax_kernel, grid, dim3(kEnThreads), 0, stream, split, ar, diff, vocab, ld,
                                split, lambda, ids, conf);
 }

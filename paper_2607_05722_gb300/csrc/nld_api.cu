@@ -571,19 +571,14 @@ nld_status_t nld_logits_ensemble_argmax(const void* ar_logits, const void* diff_
   if (!(lambda >= 0.f && lambda <= 1.f)) return NLD_ERR_INVALID_ARG;  // also rejects NaN
   if (!aligned(ar_logits, 16) || !aligned(diff_logits, 16) || !aligned(ids, 4) || !aligned(conf, 4))
     return NLD_ERR_INVALID_ARG;
+  unsigned int* err = nullptr;
   int sms = 0;
-  nld_status_t st = device_state(nullptr, &sms);
+  nld_status_t st = device_state(&err, &sms);
   if (st != NLD_OK) return st;
-  int split = 1;
-  if (rows < sms) {
-    const int by_sms = sms / rows;
-    const int by_len = (vocab / 8) / nld::logits_split_vectors();
-    const int want = by_sms < by_len ? by_sms : by_len;
-    while (split * 2 <= want && split * 2 <= 8) split *= 2;
-  }
+  const int split = logits_split(rows, vocab, sms, 1024);
   return nld::launch_ensemble_argmax(static_cast<const __nv_bfloat16*>(ar_logits),
                                      static_cast<const __nv_bfloat16*>(diff_logits), rows, vocab, ld, split, lambda,
-                                     ids, conf, stream) == cudaSuccess
+                                     ids, conf, err, stream) == cudaSuccess
              ? NLD_OK
              : NLD_ERR_CUDA;
 }

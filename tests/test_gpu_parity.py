@@ -389,6 +389,34 @@ def test_ensemble_matches_oracle(orc, rows, vocab, ld, lam):
     assert np.all(p[np.arange(rows), gi] >= oc - tol), "the GPU's id is a maximiser within the error"
 
 
+@pytest.mark.parametrize("rows,vocab", [(3, 65536), (3, 65537), (2, 131073), (2, 262144), (2, 262145), (200, 8192)])
+def test_ensemble_register_pieces(orc, rows, vocab):
+    """The sizes at which the ensemble kernels' pieces change (1024, 2048 and
+    4096 vectors a CTA, then two reads), with equal logits (every vector can
+    hold the maximum), an empty pair, a one-sided pair and disjoint peaks."""
+    rng = np.random.default_rng(vocab)
+    ld = (vocab + 7) // 8 * 8
+    x = (rng.standard_normal((2, rows, ld)) * 3).astype(np.float32)
+    x[:, :, vocab:] = 1e4
+    x[0, 0, : vocab // 2] = -np.inf                               # the maximum from one side only
+    x[0, 1, vocab // 4] = 14.0                                    # a peak on each side, the lower one wider
+    x[1, 1, vocab // 4 * 3] = 13.0
+    if rows > 2:
+        x[:, 2, :vocab] = 1.5                                     # all equal: id 0
+    if rows > 3:
+        x[:, 3, :vocab] = -np.inf                                 # both empty: id 0, conf 0
+    a, d = W.f32_to_bf16_bits(x[0]), W.f32_to_bf16_bits(x[1])
+    gi, gc = gpu_ensemble(a, d, 0.5, vocab)
+    oi, oc = orc.ensemble_argmax(a, d, 0.5, vocab)
+    assert np.all(np.abs(gc - oc) <= LOGITS_RTOL * oc)
+    p = mixture_f64(a, d, 0.5, vocab)
+    assert np.all(p[np.arange(rows), gi] >= oc - 2 * LOGITS_RTOL * oc)
+    if rows > 2:
+        assert gi[2] == 0
+    if rows > 3:
+        assert gi[3] == 0 and gc[3] == 0.0
+
+
 def test_logits_peaked_rows(orc):
     """Peaked rows (a confident prediction): the confidence near 1 is kept to
     the same relative bound."""
