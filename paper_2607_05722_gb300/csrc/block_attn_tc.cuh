@@ -6,14 +6,12 @@
 // heads times the bl block tokens form R = G*bl <= 256 query rows in one or
 // two 128-row MMA tiles, so each K/V page leaves HBM once per (b, g).
 //
-// Warp roles (5 + 4*MT*CG warps):
-//   warps 0-2 and the last  TMA producers: the boxes of each 64-token K/V tile
-//             (16 tokens x 64 dims each) dealt four ways into a ring of up to
-//             8 stages (produce_kv), warps 0-1 the K boxes, the others the V
-//             boxes (with two softmax groups each kind with its own full/empty
-//             barriers, so that a K slot refills once its score product is
-//             done); TMA issue cost is per warp, so four issuing warps land a
-//             tile sooner.
+// Warp roles (4 + 4*MT*CG warps):
+//   warps 0, 1  TMA producers of K and of V (warp 2 has no role): boxes of 16
+//             to 64 tokens x all head dims into a ring of up to 8 stages
+//             (produce_kv); with two softmax groups K and V each with their
+//             own full/empty barriers, so that a K slot refills once its score
+//             product is done.
 //   warp 3    allocates the TMEM columns; lane 0 loads Q by TMA (one M tile)
 //             and issues every MMA:
 //               S_j = Q K^T     (M=128 rows, N=64*TPS tokens, K=D; double-buffered in TMEM)
@@ -58,7 +56,7 @@
 namespace nld {
 namespace {
 
-constexpr int kProducers = 4;
+constexpr int kProducers = 2;  // warp 0 K, warp 1 V (warp 2 has no role)
 constexpr int kMmaWarp = 3;
 constexpr int kSoftmaxWarp0 = 4;
 
@@ -92,17 +90,12 @@ struct TcCfg {
   static constexpr int kSTok = kTPS * kTileTok;  // tokens (N) of a score product
   static constexpr int kPBufs = 2 * kTPS;        // tiles in flight between the softmax and PV (barrier slots)
   static constexpr int kSmWarps = 4 * MT * CG;   // softmax warps
-  static constexpr int kWarps = 5 + kSmWarps;    // 4 producers, 1 MMA, softmax
+  static constexpr int kWarps = 4 + kSmWarps;    // 2 producers, one without a role, MMA, softmax
   static constexpr int kThreads = 32 * kWarps;
   static constexpr uint32_t kTmemCols = 512;     // MT x (S0 | S1), then MT x CG x O
   static_assert(2 * MT * kSTok + MT * CG * 128 <= 512, "TMEM columns");
 };
 
-// producer index of a warp, or -1: warps 0-2 and the last warp
-template <int MT, int CG>
-__device__ __forceinline__ int producer_index(int warp) {
-  return warp < 3 ? warp : (warp == 4 + 4 * MT * CG ? 3 : -1);
-}
 constexpr float kRescaleLog2 = 8.0f;
 
 // Epilogue staging in the freed K/V ring and Q tiles: 128*MT rows of D fp32
@@ -111,9 +104,9 @@ constexpr float kRescaleLog2 = 8.0f;
 template <int D>
 __host__ __device__ constexpr int merge_pitch() { return D * 4 + 16; }
 
-// K/V ring: the K tiles column-block-major ([column block][stage], so that
-// the K tiles of consecutive stages form one operand of 128 rows), then the
-// V tiles stage-major ([stage][column block]).
+// K/V ring: the K tiles (the tiles of consecutive stages follow one another
+// with the same 8-token group stride, so two form one operand of 128 rows),
+// then the V tiles.
 template <int D, int MT, int TPS>
 struct TcLayout {
   using Geo = TileGeom<D>;
@@ -227,11 +220,11 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kTcStages; ++s) {
-      // one expect_tx arrival per producer warp (of the kind, split scheme)
-      mbar_init(&k_full[s], kSplitKV ? kProducers / 2 : kProducers);
+      // one expect_tx arrival per producer warp
+      mbar_init(&k_full[s], kSplitKV ? 1 : 2);
       mbar_init(&k_empty[s], 1);
       if (kSplitKV) {
-        mbar_init(&v_full[s], kProducers / 2);
+        mbar_init(&v_full[s], 1);
         mbar_init(&v_empty[s], 1);
       }
     }
@@ -283,7 +276,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
   // independent, so they are in flight together.
   PagePrefetch first;
   first.raw = 0;
-  if (producer_index<MT, CG>(warp) >= 0) first.load(a, b, t_begin, 0, lane);
+  if (warp < kProducers) first.load(a, b, t_begin, 0, lane);
   int L = __ldg(a.prefix_lens + b);
   __syncthreads();
   tc_fence_after();
@@ -323,7 +316,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
         a.lse_part[((static_cast<size_t>(split) * a.B + b) * a.Hq + h) * a.bl + i] = -INFINITY;
       }
     }
-  } else if (producer_index<MT, CG>(warp) >= 0) {
+  } else if (warp < kProducers) {
     // ---------------- producers ----------------
     int early_tiles = 0;  // leading tiles made of prefix tokens only
     if (early) {
@@ -332,13 +325,12 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
         ++early_tiles;
       if (early_tiles == 0) grid_dependency_wait();
     }
-    const int pw = producer_index<MT, CG>(warp);
     const int issued = produce_kv<D, kSplitKV>(a, &maps.k, &maps.v, smem, k_full, v_full, k_empty, v_empty, kTcStages,
-                                               g, b, t_begin, t_end, ntiles, lane, pw, kProducers, first, early_tiles);
+                                               g, b, t_begin, t_end, ntiles, lane, warp == 1, first, early_tiles);
     if (lane == 0 && issued < ntiles) {
       // Stopped early on a wait timeout: let the copies already issued land
       // before the CTA exits (bounded).
-      uint64_t* full = kSplitKV && pw >= kProducers / 2 ? v_full : k_full;
+      uint64_t* full = kSplitKV && warp == 1 ? v_full : k_full;
       for (int k = max(0, issued - kTcStages); k < issued; ++k)
         mbar_wait(&full[k % kTcStages], (k / kTcStages) & 1, a.err);
     }
@@ -370,7 +362,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
       // no tile of this CTA still needs; those columns are never used.
       auto issue_s = [&](int j) {
         const int st = (j * kTPS) % kTcStages;
-        const uint32_t k_addr = smem_u32(smem) + static_cast<uint32_t>(st * Geo::kColBlockBytes);
+        const uint32_t k_addr = smem_u32(smem) + static_cast<uint32_t>(st * Geo::kTileBytes);
 #pragma unroll
         for (int mt = 0; mt < MT; ++mt) {
           const uint32_t d = tS(mt, j & 1);
@@ -379,7 +371,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
             const uint32_t koff = (kk & 3) * 32;  // 16 elements along the 128-byte row
             const int cb = kk >> 2;               // 64-dim column block
             const uint64_t ad = sw128_desc(q_addr + mt * Lay::kQBytes + cb * (128 * 128) + koff, 0, 1024);
-            const uint64_t bd = sw128_desc(k_addr + cb * kTcStages * Geo::kColBlockBytes + koff, 0, 1024);
+            const uint64_t bd = sw128_desc(k_addr + cb * 1024 + koff, 0, Geo::kGroup8Bytes);
             umma_bf16(d, ad, bd, idesc_s, kk > 0 ? 1u : 0u);
           }
         }
@@ -406,7 +398,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
           const uint32_t o_acc = tO(mt);
 #pragma unroll
           for (int kt = 0; kt < kTileTok / 16; ++kt) {
-            const uint64_t bd = sw128_desc(v_addr + kt * 16 * 128, Geo::kColBlockBytes, 1024);
+            const uint64_t bd = sw128_desc(v_addr + kt * 2 * Geo::kGroup8Bytes, 1024, Geo::kGroup8Bytes);
             umma_bf16_ts(o_acc, p_tmem + kt * 8, bd, idesc_o, (k > 0 || kt > 0) ? 1u : 0u);
           }
         }
@@ -445,7 +437,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
             const uint32_t p_tmem = tP(j & 1) + static_cast<uint32_t>(h * (kTileTok / 2));
 #pragma unroll
             for (int kt = 0; kt < kTileTok / 16; ++kt) {
-              const uint64_t bd = sw128_desc(v_addr + kt * 16 * 128, Geo::kColBlockBytes, 1024);
+              const uint64_t bd = sw128_desc(v_addr + kt * 2 * Geo::kGroup8Bytes, 1024, Geo::kGroup8Bytes);
               umma_bf16_ts(tO(0), p_tmem + kt * 8, bd, idesc_o, (k > 0 || kt > 0) ? 1u : 0u);
             }
             umma_commit(kSplitKV ? &v_empty[st] : &k_empty[st]);
@@ -523,7 +515,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
       }
     }
     __syncwarp();
-  } else {
+  } else if (warp >= kSoftmaxWarp0) {  // warp 2 has no role
     // ---------------- softmax warps ----------------
     // Warp `quad` reads TMEM lanes 32*quad..+31. With REP > 1 those lanes hold
     // a copy of row block rq = quad % kRowQuads and the warp takes the token
@@ -767,7 +759,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
         }
         if (has) {
           const int valid = t_end - t_own;
-          if (valid < kTileTok && (valid & (kGroupTok - 1))) {
+          if (valid < kTileTok && (valid & (a.box_tok - 1))) {
             // V rows past the sequence end inside its last page: zero them
             // (P is 0 there, but 0 * NaN = NaN).
             const int st = k % kTcStages;
@@ -775,11 +767,11 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
               ok = false;
               break;
             }
-            const int r0 = valid, r1 = (valid + kGroupTok - 1) & ~(kGroupTok - 1);
+            const int r0 = valid, r1 = (valid + a.box_tok - 1) & ~(a.box_tok - 1);
             uint8_t* vt = smem + Lay::kVOff + st * Geo::kTileBytes;
             for (int idx = grp_tid; idx < (r1 - r0) * (D / 8); idx += 128) {
               const int row = r0 + idx / (D / 8), c = idx % (D / 8);
-              *reinterpret_cast<uint4*>(vt + kv_swz(row, c)) = make_uint4(0, 0, 0, 0);
+              *reinterpret_cast<uint4*>(vt + kv_swz<D>(row, c)) = make_uint4(0, 0, 0, 0);
             }
           }
         }
@@ -918,7 +910,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
         const int k = k0 + h;
         if (k >= ntiles) break;
         const int valid = t_end - (t_begin + k * kTileTok);
-        if (valid < kTileTok && (valid & (kGroupTok - 1))) {
+        if (valid < kTileTok && (valid & (a.box_tok - 1))) {
           // Cache slots past the sequence end inside its last page may hold
           // stale or uninitialised data; P is 0 there but 0 * NaN = NaN, so
           // zero those V rows before the PV MMA reads them.
@@ -927,11 +919,11 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
             step_ok = false;
             break;
           }
-          const int r0 = valid, r1 = (valid + kGroupTok - 1) & ~(kGroupTok - 1);
+          const int r0 = valid, r1 = (valid + a.box_tok - 1) & ~(a.box_tok - 1);
           uint8_t* vt = smem + Lay::kVOff + st * Geo::kTileBytes;
           for (int idx = grp_tid; idx < (r1 - r0) * (D / 8); idx += 128 * MT) {
             const int row = r0 + idx / (D / 8), c = idx % (D / 8);
-            *reinterpret_cast<uint4*>(vt + kv_swz(row, c)) = make_uint4(0, 0, 0, 0);
+            *reinterpret_cast<uint4*>(vt + kv_swz<D>(row, c)) = make_uint4(0, 0, 0, 0);
           }
         }
         fence_proxy_async_smem();

@@ -213,19 +213,34 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// 4-D map over a page pool [num_pages, Hkv, P, D] (innermost first: D, P, Hkv,
-// pages); one box is 64 dims x 16 tokens of one (page, KV head), stored with
-// the 128-byte swizzle. Boxes past num_pages read as zeros.
-nld_status_t encode_pool_map(CUtensorMap* map, const void* base, const nld_attn_params_t* p) {
+// Tokens of a K/V box: as many as a page holds, up to a tile, and as the
+// pieces' starts (multiples of `chunk` with more than one split) allow without
+// a box crossing a page: 16, 32 or 64.
+int box_tokens(const nld_attn_params_t* p, const SplitPlan& plan) {
+  int n = p->page_size < nld::kTileTok ? p->page_size : nld::kTileTok;
+  while (plan.splits > 1 && plan.chunk % n != 0) n /= 2;  // chunk is a multiple of 16
+  return n;
+}
+
+// 5-D map over a page pool [num_pages, Hkv, P, D], innermost first: 64 dims,
+// 8 tokens, the 64-dim column blocks, the 8-token groups of a page, (page, KV
+// head). A box is all dims of box_tok tokens of one (page, KV head), in shared
+// memory as [8-token group][column block][8 rows of 128 bytes] with the
+// 128-byte swizzle: 8-token groups a fixed stride apart, as the MMA operands
+// want them, also over the boxes and tiles that follow one another. Boxes past
+// num_pages read as zeros.
+nld_status_t encode_pool_map(CUtensorMap* map, const void* base, const nld_attn_params_t* p, int box_tok) {
   EncodeTiledFn fn = encode_fn();
   if (fn == nullptr) return NLD_ERR_CUDA;
+  const long long planes = static_cast<long long>(p->num_pages) * p->num_kv_heads;
+  if (planes > INT_MAX - p->num_kv_heads) return NLD_ERR_UNSUPPORTED;  // coordinates are int
   const cuuint64_t D = static_cast<cuuint64_t>(p->head_dim);
-  cuuint64_t dims[4] = {D, static_cast<cuuint64_t>(p->page_size), static_cast<cuuint64_t>(p->num_kv_heads),
-                        static_cast<cuuint64_t>(p->num_pages)};
-  cuuint64_t strides[3] = {D * 2, D * 2 * p->page_size, D * 2 * p->page_size * p->num_kv_heads};
-  cuuint32_t box[4] = {64, static_cast<cuuint32_t>(nld::kGroupTok), 1, 1};
-  cuuint32_t estr[4] = {1, 1, 1, 1};
-  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
+  const cuuint64_t P = static_cast<cuuint64_t>(p->page_size);
+  cuuint64_t dims[5] = {64, 8, D / 64, P / 8, static_cast<cuuint64_t>(planes)};
+  cuuint64_t strides[4] = {D * 2, 128, D * 2 * 8, D * 2 * P};
+  cuuint32_t box[5] = {64, 8, static_cast<cuuint32_t>(D / 64), static_cast<cuuint32_t>(box_tok / 8), 1};
+  cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? NLD_OK : NLD_ERR_CUDA;
@@ -384,8 +399,9 @@ nld_status_t block_attn_impl(const nld_attn_params_t* params, const void* q_bloc
   if (st != NLD_OK) return st;
 
   nld::TmaMaps maps;
-  if ((st = encode_pool_map(&maps.k, k_pages, params)) != NLD_OK) return st;
-  if ((st = encode_pool_map(&maps.v, v_pages, params)) != NLD_OK) return st;
+  const int box_tok = box_tokens(params, plan);
+  if ((st = encode_pool_map(&maps.k, k_pages, params, box_tok)) != NLD_OK) return st;
+  if ((st = encode_pool_map(&maps.v, v_pages, params, box_tok)) != NLD_OK) return st;
 
   const int G = params->num_q_heads / params->num_kv_heads;
   const float scale = params->softmax_scale > 0.f ? params->softmax_scale : 1.0f / sqrtf((float)params->head_dim);
@@ -409,6 +425,7 @@ nld_status_t block_attn_impl(const nld_attn_params_t* params, const void* q_bloc
   a.log2_page = __builtin_ctz(static_cast<unsigned>(params->page_size));
   a.num_pages = params->num_pages;
   a.max_pages = params->max_pages_per_seq;
+  a.box_tok = box_tok;
   a.num_splits = plan.splits;
   a.chunk = plan.chunk;
   a.csize = plan.csize;

@@ -20,7 +20,7 @@ constexpr int kModeBlockMask = 2;  // block part of the mask from a per-row tabl
 constexpr int kMaxRows = 256;   // (Hq / Hkv) * block_len handled by one CTA (two 128-row M tiles)
 constexpr int kMaxBlock = 32;   // block_len and the decision width n
 constexpr int kTileTok = 64;    // KV tokens per pipeline stage
-constexpr int kGroupTok = 16;   // KV tokens per TMA box (never crosses a page: P % 16 == 0)
+constexpr int kGroupTok = 16;   // KV tokens per page-table lookup (never cross a page: P % 16 == 0)
 
 // Arguments of the block-attention kernel (one CTA per (split, kv head, sequence)).
 struct AttnArgs {
@@ -36,6 +36,7 @@ struct AttnArgs {
   int B, Hq, Hkv, G, bl, R;    // R = G * bl_c query rows per CTA
   int nh, bl_c;                // block-slot chunks per (split, KV head, sequence) (1 or 2), slots per chunk
   int page_size, log2_page, num_pages, max_pages;
+  int box_tok;                 // KV tokens per TMA box (16, 32 or 64; never crosses a page)
   int num_splits, chunk;       // splits and tokens per split (multiple of 16)
   int mode;                    // NLD_MODE_DIFFUSION, NLD_MODE_VERIFY or kModeBlockMask
   const uint32_t* block_mask;  // [bl] row masks over the block slots (kModeBlockMask only)
@@ -215,17 +216,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, unsign
   return mbar_wait_for(bar, parity, err, kWaitLimitNs);
 }
 
-// 4-D tiled TMA load into shared memory, completing on an mbarrier.
-__device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1,
-                                            int c2, int c3) {
+// 5-D tiled TMA load into shared memory, completing on an mbarrier.
+__device__ __forceinline__ void tma_load_5d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1,
+                                            int c2, int c3, int c4) {
   asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+      "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%3, %4, %5, %6, %7}], [%2];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
       : "memory");
 }
 
-// 3-D tiled TMA load into shared memory, completing on an mbarrier.
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1,
                                             int c2) {
   asm volatile(
@@ -549,20 +549,22 @@ __device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, u
 // K/V tile staging shared by the attention kernels
 // ---------------------------------------------------------------------------
 
-// A stage holds the K tile then the V tile of 64 tokens; each is D/64 column
-// blocks of 64 tokens x 128 bytes, written by TMA with the 128-byte swizzle
-// (chunk c of row r at chunk position c ^ (r % 8) within each 1024-byte atom).
+// A K or V tile of 64 tokens is 8 groups of 8 tokens, each D/64 column blocks
+// of 8 rows of 128 bytes, written by TMA with the 128-byte swizzle (chunk c of
+// row r at chunk position c ^ (r % 8) within each 1024-byte atom).
 template <int D>
 struct TileGeom {
   static constexpr int kColBlocks = D / 64;
-  static constexpr int kColBlockBytes = kTileTok * 128;
-  static constexpr int kTileBytes = kColBlocks * kColBlockBytes;
+  static constexpr int kGroup8Bytes = kColBlocks * 1024;
+  static constexpr int kTileBytes = kTileTok / 8 * kGroup8Bytes;
   static constexpr int kStageBytes = 2 * kTileBytes;
 };
 
 // Byte offset of (token r, 16-byte chunk c) inside a K or V tile.
+template <int D>
 __device__ __forceinline__ uint32_t kv_swz(int r, int c) {
-  return static_cast<uint32_t>((c >> 3) * (kTileTok * 128) + r * 128 + (((c & 7) ^ (r & 7)) << 4));
+  return static_cast<uint32_t>((r >> 3) * TileGeom<D>::kGroup8Bytes + (c >> 3) * 1024 + (r & 7) * 128 +
+                               (((c & 7) ^ (r & 7)) << 4));
 }
 
 // Page id of each 16-token group of a split, loaded ahead: lane j of the
@@ -589,50 +591,51 @@ struct PagePrefetch {
   }
 };
 
-// Producer warp `pw` of `nprod`: streams its share of the TMA boxes of the
-// K/V tiles of tokens [t_begin, t_end) of (sequence b, KV head g) into an
-// nstage ring: K tiles at [column block][stage], so that the K of
-// consecutive stages is contiguous per column block, then V tiles at
-// [stage][column block]. A tile has 4 groups x D/64 column blocks x {K, V} boxes
-// (16 tokens x 64 dims each); they are dealt to the producer warps in equal
-// shares and, within a warp, one box per lane: the first half of the warps
-// load K, the second half V. With kSplit, K and V slots fill and free on
-// their own barriers (k_full/v_full, k_empty/v_empty), so a K slot is
-// refilled as soon as the score product that read it has completed, before
-// the PV product frees the V slot of the same tile; without it a stage's K
-// and V fill on k_full and free on k_empty together. TMA issue cost is per
-// warp, so more producer warps land a tile sooner. A warp's expect_tx covers
-// only its own boxes, so a full barrier expects one arrival per warp (of its
-// kind, with kSplit). `first` holds the page ids of the first 32 groups,
-// already loaded. With kSplit the `early_tiles` leading tiles issued before
-// the dependency wait go out K first: the V warps wait at a named barrier
-// until the K warps have issued the early K boxes, so the first score
-// products' operands are not queued behind V boxes that only the later PV
-// products read. Returns tiles issued.
+// A producer warp: streams the K (or V) boxes of the tiles of tokens
+// [t_begin, t_end) of (sequence b, KV head g) into an nstage ring, K tiles
+// stage-major, then V tiles stage-major; a tile has 64 / box_tok boxes, one
+// per lane. With kSplit, K and V slots fill and free on their own barriers
+// (k_full/v_full, k_empty/v_empty), so a K slot is refilled as soon as the
+// score product that read it has completed, before the PV product frees the V
+// slot of the same tile; without it a stage's K and V fill on k_full and free
+// on k_empty together. A warp's expect_tx covers only its own boxes, so a full
+// barrier expects one arrival per warp (of its kind, with kSplit). `first`
+// holds the page ids of the first 32 groups, already loaded. With kSplit the
+// `early_tiles` leading tiles issued before the dependency wait go out K
+// first: the V warp waits at a named barrier until the K warp has issued the
+// early K boxes, so the first score products' operands are not queued behind
+// V boxes that only the later PV products read. Returns tiles issued.
+//
+// A box holds all head dims of 16 (P = 16), 32 or 64 tokens, so the K and V
+// tiles of 64 tokens take 8 to 2 TMA instructions, one warp each. With boxes
+// of 64 dims x 16 tokens they took 16 (D = 128), dealt over four warps: a 13th
+// warp in the block, which left 128 registers a thread (spills) instead of
+// 168. Verify batches of 8 / 32 / 128 sequences: 50.7 -> 49.4, 105.2 -> 104.4,
+// 359.5 -> 355.0 us; one sequence unchanged.
 template <int D, bool kSplit>
 __device__ __forceinline__ int produce_kv(const AttnArgs& a, const CUtensorMap* tmk, const CUtensorMap* tmv,
                                           uint8_t* stages, uint64_t* k_full, uint64_t* v_full, uint64_t* k_empty,
                                           uint64_t* v_empty, int nstage, int g, int b, int t_begin, int t_end,
-                                          int ntiles, int lane, int pw, int nprod, const PagePrefetch& first,
+                                          int ntiles, int lane, bool warp_v, const PagePrefetch& first,
                                           int early_tiles) {
   using Geo = TileGeom<D>;
-  constexpr int kGroups = kTileTok / kGroupTok;
-  constexpr int kOpsPerTile = kGroups * 2 * Geo::kColBlocks;  // 16 (D=128) or 8 (D=64)
-  const int my_ops = kOpsPerTile / nprod;                     // nprod divides kOpsPerTile (and its halves)
-  const bool warp_v = pw >= nprod / 2;                        // this warp's boxes are all V (else all K)
+  const CUtensorMap* map = warp_v ? tmv : tmk;
   uint64_t* full = kSplit && warp_v ? v_full : k_full;
   uint64_t* empty = kSplit && warp_v ? v_empty : k_empty;
-  const uint32_t bytes = static_cast<uint32_t>(my_ops) * kGroupTok * 128;
+  uint8_t* ring = warp_v ? stages + nstage * Geo::kTileBytes : stages;
+  const int box_tok = a.box_tok;
+  const int boxes = kTileTok / box_tok;
+  const int t_box = lane * box_tok;  // this lane's box within a tile (lanes below `boxes`)
   int page_cur = first.validate(a, t_begin, t_end, 0, lane);
   PagePrefetch nxt;
   nxt.raw = 0;
   if (ntiles > 8) nxt.load(a, b, t_begin, 1, lane);
   int issued = 0;
-  // Named barrier 4: the nprod producer warps, once, before any wait of the
-  // loop (early_tiles <= nstage, so the K warps reach their arrival without
+  // Named barrier 4: the two producer warps, once, before any wait of the
+  // loop (early_tiles <= nstage, so the K warp reaches its arrival without
   // waiting on a slot).
   constexpr int kKFirstBar = 4;
-  if (kSplit && warp_v && early_tiles > 0) named_bar_sync(kKFirstBar, 32 * nprod);
+  if (kSplit && warp_v && early_tiles > 0) named_bar_sync(kKFirstBar, 64);
   for (int k = 0; k < ntiles; ++k) {
     const int st = k % nstage;
     // The first `early_tiles` tiles hold prefix tokens only and may be issued
@@ -648,26 +651,16 @@ __device__ __forceinline__ int produce_kv(const AttnArgs& a, const CUtensorMap* 
       page_cur = nxt.validate(a, t_begin, t_end, batch, lane);
       if ((k + 8) < ntiles) nxt.load(a, b, t_begin, batch + 1, lane);
     }
-    if (lane == 0) mbar_arrive_expect_tx(&full[st], bytes);
+    if (lane == 0) mbar_arrive_expect_tx(&full[st], Geo::kTileBytes);
     __syncwarp();
-    // op -> (group, kind, column block): group fastest, so a warp's boxes
-    // spread over the tile's pages.
-    const int op = pw * my_ops + (lane < my_ops ? lane : 0);
-    const int grp = op % kGroups;
-    const int kind_cb = op / kGroups;  // 0 .. 2*kColBlocks-1
-    const bool is_v = kind_cb >= Geo::kColBlocks;
-    const int cb = kind_cb % Geo::kColBlocks;
-    const int page = __shfl_sync(0xffffffffu, page_cur, ((k & 7) * kGroups + grp) & 31);
-    if (lane < my_ops) {
-      const int t = t_begin + k * kTileTok + grp * kGroupTok;
-      const int slot = page < a.num_pages ? (t & (a.page_size - 1)) : 0;
-      uint8_t* dst = (is_v ? stages + (nstage + st) * Geo::kTileBytes + cb * Geo::kColBlockBytes
-                           : stages + (cb * nstage + st) * Geo::kColBlockBytes) +
-                     grp * kGroupTok * 128;
-      tma_load_4d(dst, is_v ? tmv : tmk, &full[st], cb * 64, slot, g, page);
+    const int page = __shfl_sync(0xffffffffu, page_cur, ((k & 7) * (kTileTok / kGroupTok) + t_box / kGroupTok) & 31);
+    if (lane < boxes) {
+      const int slot = page < a.num_pages ? ((t_begin + k * kTileTok + t_box) & (a.page_size - 1)) : 0;
+      tma_load_5d(ring + st * Geo::kTileBytes + (t_box / 8) * Geo::kGroup8Bytes, map, &full[st], 0, 0, 0, slot >> 3,
+                  page * a.Hkv + g);
     }
     issued = k + 1;
-    if (kSplit && !warp_v && k == early_tiles - 1) named_bar_arrive(kKFirstBar, 32 * nprod);
+    if (kSplit && !warp_v && k == early_tiles - 1) named_bar_arrive(kKFirstBar, 64);
   }
   return issued;
 }

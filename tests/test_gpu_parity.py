@@ -13,7 +13,7 @@ import pytest
 import torch
 
 import oracle_pins
-from gpu_helpers import DeviceCase, compare_attn, oracle_full, rows_per_unit, sample_rows
+from gpu_helpers import DeviceCase, bits_to_bf16, compare_attn, oracle_full, rows_per_unit, sample_rows
 from paper_2607_05722_gb300 import nld
 from paper_2607_05722_gb300 import workloads as W
 
@@ -784,6 +784,31 @@ def test_attention_tail_slots_hold_nan(orc):
             out, lse = dc.run(mode, num_splits=splits)
             ro, rl = oracle_full(orc, case2, mode)
             compare_attn(out, lse, ro, rl, f"nan tail mode={mode} S={splits}")
+
+
+@pytest.mark.parametrize("D,P,splits", [(128, 16, 1), (128, 32, 3), (64, 64, 1), (128, 64, 3), (128, 64, 2),
+                                         (64, 256, 5), (128, 256, 1)])
+def test_attention_kv_boxes(orc, D, P, splits):
+    """K/V boxes of 16, 32 and 64 tokens (the page size, less where the pieces
+    start off that grid), sequence ends inside a box, on its edges and on tile
+    edges, and NaN in every slot past the sequence end of its last page."""
+    lens = [0, 1, P - 9, 64 - 9 + 1, 119, 120, 513, 900]
+    case = W.make_block_attn_case("kv_boxes", len(lens), 12, 3, D, block_len=9, page_size=P, prefix_lens=lens, seed=11)
+    nan = np.uint16(0x7FC0)
+    k_bits, v_bits = case.kv.k_bits.copy(), case.kv.v_bits.copy()
+    for b, L in enumerate(lens):
+        end = L + 9
+        if end % P:
+            page = case.kv.page_table[b, end // P]
+            k_bits[page, :, end % P:, :] = nan
+            v_bits[page, :, end % P:, :] = nan
+    dc = DeviceCase(case)
+    dc.k, dc.v = bits_to_bf16(k_bits), bits_to_bf16(v_bits)
+    for mode in (W.MODE_DIFFUSION, W.MODE_VERIFY):
+        ro, rl = oracle_full(orc, case, mode)
+        for flags in (0, nld.NLD_ATTN_NO_CLUSTER):
+            out, lse = dc.run(mode, num_splits=splits, flags=flags)
+            compare_attn(out, lse, ro, rl, f"kv boxes D={D} P={P} S={splits} mode={mode} flags={flags}")
 
 
 def test_attention_split_sweep(orc):
