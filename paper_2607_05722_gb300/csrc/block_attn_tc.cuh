@@ -29,12 +29,12 @@
 //             in the freed K/V ring in 128-byte-swizzled boxes, which one
 //             thread writes with tiled TMA stores (the bf16 output or bf16
 //             split partials, in packed row order).
-//             With 33..64 packed rows, Q is replicated into the idle lane
-//             quadrants (REP = 2): each copy of a row takes a 32-token slice
+//             With 33..64 packed rows and a split that fits in the ring, Q
+//             is replicated into the idle lane quadrants (REP = 2): each copy of a row takes a 32-token slice
 //             of every tile with its own running max and sum, so every
 //             softmax warp works and each does half of the exponentials; the
 //             copies are merged once, each finalising half of the columns.
-//             With up to 32 or 65..128 rows (CG = 2) two groups of four
+//             Otherwise, with one M tile (CG = 2), two groups of four
 //             softmax warps share the TMEM lanes: group c takes tile 2j + c
 //             of score product j. Both take the row max over both tiles (the
 //             groups' tile maxima exchanged through shared memory), so they
@@ -1342,35 +1342,32 @@ int max_active_clusters_t(int csize) {
   return n;
 }
 
-// Copies of each Q row in the 128 TMEM lanes of one M tile: 4 for up to 32
-// packed rows, 2 for up to 64, else 1 (and 1 with two M tiles).
-// Row copies of the one-group kernel: 33..64 rows take two copies; up to
-// 32 rows and 65..128 rows run on the two-group kernel (1).
+// Copies of each Q row in the 128 TMEM lanes of one M tile: two for 33..64
+// packed rows, else one.
 int tc_replication(int rows) { return rows > 32 && rows <= 64 ? 2 : 1; }
 
 template <int D>
 int max_active_clusters_d(int csize, int rows) {
   if (rows > 128) return max_active_clusters_t<D, 2, 1, 1, 1>(csize);
   switch (tc_replication(rows)) {
-    case 2: return max_active_clusters_t<D, 1, 2, 1, 1>(csize);
+    case 2: return max_active_clusters_t<D, 1, 2, 2, 1>(csize);
     default: return max_active_clusters_t<D, 1, 1, 2, 2>(csize);
   }
 }
 
-// One M tile: 33..64 rows copied twice, with paired score products when a
-// split fits in the ring whole (it is then latency-bound: fewer, wider steps
-// help; the 8B shape's 64 rows measured 7.12 us per launch against 7.32 on
-// the two-group kernel) and single tiles when it streams; up to 32 and
-// 65..128 rows take paired products and two softmax groups, streaming or
-// not (32-row batches measured 50/75/87 -> 55/86/95% of peak at B = 8, 32,
-// 128 against four row copies: the score products run ahead of the PV
-// products there, and each tile takes 8 MMAs instead of 12).
+// One M tile: 33..64 rows are copied twice when a split fits in the ring whole
+// (it is then latency-bound: fewer, wider steps help; the 8B shape's 64 rows
+// measured 7.12 us per launch against 7.32 on the two-group kernel). All others
+// take two softmax groups: the score products run ahead of the PV products
+// there, and each tile takes 8 MMAs instead of 12. 32-row batches measured
+// 50/75/87 -> 55/86/95% of peak at B = 8, 32, 128 against four row copies; 64
+// rows, 24 sequences of 256..4096 tokens 53.7 -> 45.2 us against two copies.
 template <int D, int TPS, bool MASKED>
 cudaError_t launch_tc_rep(const AttnArgs& a, const TmaMaps& maps, cudaStream_t stream) {
-  switch (tc_replication(a.R)) {
-    case 2: return launch_tc_t<D, 1, 2, TPS, MASKED>(a, maps, stream);
-    default: return launch_tc_t<D, 1, 1, 2, MASKED, 2>(a, maps, stream);
+  if constexpr (TPS == 2) {
+    if (tc_replication(a.R) == 2) return launch_tc_t<D, 1, 2, 2, MASKED>(a, maps, stream);
   }
+  return launch_tc_t<D, 1, 1, 2, MASKED, 2>(a, maps, stream);
 }
 
 template <int D, bool MASKED>
