@@ -9,9 +9,9 @@
 // Warp roles (4 + 4*MT*CG warps):
 //   warps 0, 1  TMA producers of K and of V (warp 2 has no role): boxes of 16
 //             to 64 tokens x all head dims into a ring of up to 8 stages
-//             (produce_kv); with two softmax groups K and V each with their
-//             own full/empty barriers, so that a K slot refills once its score
-//             product is done.
+//             (produce_kv); with two softmax groups or two M tiles K and V
+//             each with their own full/empty barriers, so that a K slot
+//             refills once its score product is done.
 //   warp 3    allocates the TMEM columns; lane 0 loads Q by TMA (one M tile)
 //             and issues every MMA:
 //               S_j = Q K^T     (M=128 rows, N=64*TPS tokens, K=D; double-buffered in TMEM)
@@ -30,10 +30,14 @@
 //             thread writes with tiled TMA stores (the bf16 output or bf16
 //             split partials, in packed row order).
 //             With 33..64 packed rows and a split that fits in the ring, Q
-//             is replicated into the idle lane quadrants (REP = 2): each copy of a row takes a 32-token slice
-//             of every tile with its own running max and sum, so every
-//             softmax warp works and each does half of the exponentials; the
-//             copies are merged once, each finalising half of the columns.
+//             is replicated into the idle lane quadrants (REP = 2): each copy
+//             of a row takes a 32-token slice of every tile with its own
+//             running max and sum, so every softmax warp works and each does
+//             half of the exponentials; the copies are merged once, each
+//             finalising half of the columns.
+//             With two M tiles each has a softmax group of its own, and the
+//             tensor core works on one tile while the other's group turns its
+//             scores into P.
 //             Otherwise, with one M tile (CG = 2), two groups of four
 //             softmax warps share the TMEM lanes: group c takes tile 2j + c
 //             of score product j. Both take the row max over both tiles (the
@@ -61,15 +65,20 @@ constexpr int kMmaWarp = 3;
 constexpr int kSoftmaxWarp0 = 4;
 
 // MT 128-row M tiles per CTA (MT = 2 for 129..256 packed rows); 4*MT
-// softmax warps; TPS 64-token K/V tiles per score product. TPS = 2 (one M
-// tile, a split short enough to sit in the ring whole): N = 128 products,
-// which the tensor core runs at full rate (N = 64 at about half), and half
-// as many steps in the chain S -> softmax -> PV. A long split streams with
-// TPS = 1, where a stage frees after each tile and more of the ring stays
-// in flight. P lives in TMEM over its consumed S columns, so the ring takes
-// what shared memory the Q tiles leave (up to 8 stages): a streaming CTA's
-// bandwidth is the bytes it has in flight over the DRAM latency, so every
-// stage counts.
+// softmax warps; TPS = 2 64-token K/V tiles per score product: N = 128
+// products, which the tensor core runs at full rate (N = 64 at about half), and
+// half as many steps in the chain S -> softmax -> PV. The ring takes what
+// shared memory the Q tiles leave (up to 8 stages): a streaming CTA's bandwidth
+// is the bytes it has in flight over the DRAM latency, so every stage counts.
+//
+// Two M tiles: one CTA takes all rows of its (sequence, KV head), so every tile
+// is read once. TMEM: an S buffer a tile (P over its consumed columns) and an O
+// a tile, all 512 columns. A product of 128 tokens takes 32 MMAs; a PV product's
+// cost ~70 cycles each and a score product's ~137 (both operands, 8 KB, from
+// shared memory), which bounds the kernel: 1.80 us per 128 tokens for 160 rows,
+// 1.90 for 256, from L2 or HBM alike, and 1.70 without any softmax arithmetic.
+// Block-slot halves in two CTAs of one M tile each took 1.29 us a CTA, 2.58 for
+// the pair; one CTA with N = 64 products 2.36.
 //
 // CG softmax groups per M tile: with CG = 2 (one M tile of up to 128 rows
 // without row copies, paired products) two groups of four warps share the
@@ -84,7 +93,7 @@ constexpr int kSoftmaxWarp0 = 4;
 // chain S -> softmax -> PV no longer holds the next score products back.
 template <int MT, int TPS, int CG = 1>
 struct TcCfg {
-  static_assert(TPS == 1 || (TPS == 2 && MT == 1), "paired score products with one M tile");
+  static_assert(TPS == 2 || MT == 1, "two M tiles: paired score products");
   static_assert(CG == 1 || (CG == 2 && MT == 1 && TPS == 2), "two softmax groups: one M tile, paired products");
   static constexpr int kTPS = TPS;               // K/V tiles per score product
   static constexpr int kSTok = kTPS * kTileTok;  // tokens (N) of a score product
@@ -92,8 +101,9 @@ struct TcCfg {
   static constexpr int kSmWarps = 4 * MT * CG;   // softmax warps
   static constexpr int kWarps = 4 + kSmWarps;    // 2 producers, one without a role, MMA, softmax
   static constexpr int kThreads = 32 * kWarps;
-  static constexpr uint32_t kTmemCols = 512;     // MT x (S0 | S1), then MT x CG x O
-  static_assert(2 * MT * kSTok + MT * CG * 128 <= 512, "TMEM columns");
+  static constexpr int kSBufs = MT == 2 ? 1 : 2;  // S buffers per M tile
+  static constexpr uint32_t kTmemCols = 512;     // MT x kSBufs x S, then MT x O
+  static_assert(kSBufs * MT * kSTok + MT * 128 <= 512, "TMEM columns");
 };
 
 constexpr float kRescaleLog2 = 8.0f;
@@ -112,25 +122,32 @@ struct TcLayout {
   using Geo = TileGeom<D>;
   static constexpr int kPBufs = TcCfg<MT, TPS>::kPBufs;
   static constexpr int kQBytes = Geo::kColBlocks * 128 * 128;  // one 128-row Q tile, bf16
-  // stages: what is left of 227 KB after Q, 512 bytes of barriers and the
-  // 1024-byte alignment slack, a multiple of TPS, at most 8 (P lives in TMEM)
-  static constexpr int kFitStages = (232448 - 1024 - 512 - 1536 - MT * kQBytes) / Geo::kStageBytes;
-  static constexpr int kStages = (kFitStages < 8 ? kFitStages : 8) / TPS * TPS;
-  static_assert(kStages >= 2 * TPS, "at least two score products in the ring");
-  static constexpr int kVOff = kStages * Geo::kTileBytes;       // V tiles after the K tiles
-  static constexpr int kQOff = kStages * Geo::kStageBytes;
+  // K and V stages: what is left of 227 KB after Q, 512 bytes of barriers, the
+  // 1024-byte alignment slack and the row maxima that two softmax groups
+  // exchange, a multiple of TPS, at most 8 (P lives in TMEM). With two M tiles
+  // and D = 128 the K ring takes the odd product that fits: its slots are free
+  // only when both tiles' score products have completed.
+  static constexpr int kXmBytes = MT == 2 ? 0 : 1536;
+  static constexpr int kFree = 232448 - 1024 - 512 - kXmBytes - MT * kQBytes;
+  static constexpr int kFitStages = kFree / Geo::kStageBytes;
+  static constexpr int kVStages = (kFitStages < 8 ? kFitStages : 8) / TPS * TPS;
+  static constexpr int kKFit = (kFree - kVStages * Geo::kTileBytes) / Geo::kTileBytes;
+  static constexpr int kKStages = MT == 2 ? (kKFit < 8 ? kKFit : 8) / TPS * TPS : kVStages;
+  static_assert(kVStages >= 2 * TPS, "at least two score products in the ring");
+  static constexpr int kVOff = kKStages * Geo::kTileBytes;      // V tiles after the K tiles
+  static constexpr int kQOff = kVOff + kVStages * Geo::kTileBytes;
   static constexpr int kPOff = kQOff + MT * kQBytes;  // end of the ring and Q tiles
   static constexpr int kBarOff = kPOff;
-  // k_full[st], v_full[st], k_empty[st], v_empty[st], s_full[2], s_free[2], p_full[kPBufs], o_done[kPBufs],
+  // [kKStages] k_full, v_full, k_empty, v_empty, s_full[2], s_free[2], p_full[kPBufs], o_done[kPBufs],
   // q_ready, q_full, drain, o_fin, xm_full[2], tmem slot
-  static constexpr int kNumBars = 4 * kStages + 4 + 2 * kPBufs + 4 + 2;
+  static constexpr int kNumBars = 4 * kKStages + 4 + 2 * kPBufs + 4 + 2;
   static_assert(kNumBars * 8 + 16 <= 512, "barrier reserve");
   // two softmax groups: each row's score max per group, truncated to 24 bits
   // (high 16 bits [2][group][TMEM lane], then the next 8 bits, same order),
   // exchanged every step (two buffers by step parity)
   static constexpr int kXmOff = kBarOff + 512;
   static constexpr int kXmLoOff = kXmOff + 2 * 2 * 128 * 2;
-  static constexpr int kBytes = kXmLoOff + 2 * 2 * 128;
+  static constexpr int kBytes = kXmOff + kXmBytes;
   static_assert(kBytes + 1024 <= 232448, "shared memory per CTA");
   static constexpr int kMergeRows = 128 * MT;
   static constexpr int kLseOff = kMergeRows * merge_pitch<D>();
@@ -164,7 +181,15 @@ __device__ __noinline__ int sequence_by_length_rank(const AttnArgs& a, int* scra
   return order[blockIdx.z];
 }
 
-template <int D, int MT, int REP, int TPS, bool MASKED, bool ORDERED, int CG>
+// Which (split, KV head, sequence) a CTA takes: its grid position, with the
+// sequences in grid order or longest first.
+constexpr int kGridOrder = 0, kLongestFirst = 1;
+
+// A CTA's share of the work.
+struct Piece {
+  int b, g, split, chunk;
+};
+template <int D, int MT, int REP, int TPS, bool MASKED, int ORDER, int CG>
 __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
     block_attn_tc_kernel(const __grid_constant__ TmaMaps maps, const AttnArgs a) {
   static_assert(REP == 1 || REP == 2, "replication of 1 or 2 (up to 32 rows run on two softmax groups)");
@@ -173,17 +198,16 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
   using Geo = TileGeom<D>;
   using Cfg = TcCfg<MT, TPS, CG>;
   using Lay = TcLayout<D, MT, TPS>;
-  constexpr int kTcStages = Lay::kStages;
-  // Ring barriers. With two softmax groups (65..128 rows, a split of its own
-  // or a block-slot chunk pair) K and V slots fill and free on their own
+  constexpr int kTcStages = Lay::kKStages;  // K ring; V ring the same but with two M tiles
+  constexpr int kVStages = Lay::kVStages;
+  // Ring barriers. With two softmax groups or two M tiles K and V slots fill
+  // and free on their own
   // barriers, so a K slot is refilled as soon as the score product that read
   // it has completed and the K boxes of the early tiles go out first; the
-  // kernels with one group (row copies, two M tiles) keep one barrier per
-  // stage for K and V together, freed by the PV product. Each scheme
-  // measured faster on its own kernels (the split scheme: long prefix +4%,
-  // 14B chunk pairs +10% once the score products stopped waiting for the PV
-  // products; the joint one: concurrency sweep +6%).
-  constexpr bool kSplitKV = CG == 2;
+  // kernels with row copies keep one barrier per stage for K and V together,
+  // freed by the PV product. Each scheme measured faster on its own kernels
+  // (the split scheme: long prefix +4%; the joint one: short splits).
+  constexpr bool kSplitKV = CG == 2 || MT == 2;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* q_s = smem + Lay::kQOff;
@@ -210,13 +234,13 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  // Block-slot chunks (a.nh = 2 for 129..256 packed rows): the two CTAs of
-  // a (split, KV head, sequence) are adjacent along x and hold block slots
-  // [hc*bl_c, (hc+1)*bl_c) of the G heads each, R = G*bl_c rows. A chunk
-  // holds 65..128 rows, so only the two-group kernels see nh = 2.
-  const int nh = CG == 2 ? a.nh : 1;
-  const int split = static_cast<int>(blockIdx.x) / nh, g = blockIdx.y;
-  const int slot0 = (static_cast<int>(blockIdx.x) - split * nh) * a.bl_c;  // first block slot of this CTA
+  // With NLD_ATTN_PREFIX_READY the prefix lengths, the page table and
+  // prefix-only K/V tiles are read before the dependency wait.
+  const bool early = a.prefix_ready != 0;
+  Piece piece = {static_cast<int>(blockIdx.z), static_cast<int>(blockIdx.y), static_cast<int>(blockIdx.x), a.chunk};
+  const int split = piece.split, g = piece.g;
+  // two M tiles: softmax warps of an M tile that hold real rows
+  auto tile_row_warps = [&](int mt) -> int { return min(4, (a.R - mt * 128 + 31) / 32); };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kTcStages; ++s) {
@@ -229,19 +253,20 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
       }
     }
     for (int j = 0; j < 2; ++j) {
-      mbar_init(&s_full[j], 1);
+      mbar_init(&s_full[j], 1);  // two M tiles: [M tile]
       mbar_init(&s_free[j], Cfg::kSmWarps);
     }
     for (int j = 0; j < Cfg::kPBufs; ++j) {
       // one group: the four warps of an M tile per tile; two groups: all
-      // eight softmax warps per score product (p_full[j % 2])
-      mbar_init(&p_full[j], CG == 2 ? Cfg::kSmWarps : 4 * MT);
+      // eight softmax warps per score product
+      // (p_full[j % 2]); two M tiles: the warps with rows of tile j
+      mbar_init(&p_full[j], CG == 2 ? Cfg::kSmWarps : MT == 2 ? (j < 2 ? tile_row_warps(j) : 1) : 4);
       mbar_init(&o_done[j], 1);
     }
     mbar_init(q_ready, Cfg::kSmWarps);
     mbar_init(q_full, 1);
     mbar_init(drain, 1);
-    if (CG == 2) {
+    if (CG == 2 || MT == 2) {
       mbar_init(o_fin, 1);
       mbar_init(&xm_full[0], Cfg::kSmWarps);
       mbar_init(&xm_full[1], Cfg::kSmWarps);
@@ -262,16 +287,23 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
   // dependency wait. With it, the page table, the prefix lengths and
   // prefix-only K/V tiles are read first, and only the block slots, Q and the
   // outputs wait (producers: in produce_kv; softmax warps: before Q).
-  const bool early = a.prefix_ready != 0;
   grid_launch_dependents();  // dependents launch early; they wait on this grid themselves
   if (!early) grid_dependency_wait();
-  // ORDERED (one split per sequence and more (sequence, KV head) units than
-  // SMs): CTAs start in z order, so CTA z takes the sequence of rank z by
+  // kLongestFirst (one split per sequence and more (sequence, KV head) units
+  // than SMs): CTAs start in z order, so CTA z takes the sequence of rank z by
   // prefix length and the last wave holds the short ones. The ranks are
   // computed in the K/V ring, before any copy into it. A separate
   // instantiation, so the other kernels keep b = blockIdx.z.
-  const int b = ORDERED ? sequence_by_length_rank(a, reinterpret_cast<int*>(smem)) : static_cast<int>(blockIdx.z);
-  const int t_begin = split * a.chunk;
+  // Two CTAs of a cluster take half of their sequence each.
+  if constexpr (ORDER == kLongestFirst) {
+    piece.b = sequence_by_length_rank(a, reinterpret_cast<int*>(smem));
+    if (a.num_splits == 2) {
+      const int tokens = min(max(reinterpret_cast<const int*>(smem)[piece.b], 0), a.max_pages * a.page_size - a.bl) + a.bl;
+      piece.chunk = ((tokens + 1) / 2 + kTileTok - 1) & ~(kTileTok - 1);
+    }
+  }
+  const int b = piece.b;
+  const int t_begin = split * piece.chunk;
   // The producers' first page-id loads and the prefix-length load are
   // independent, so they are in flight together.
   PagePrefetch first;
@@ -288,8 +320,8 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
   constexpr int kTPS = Cfg::kTPS;
   constexpr int kSTok = Cfg::kSTok;
   constexpr int kPBufs = Cfg::kPBufs;
-  auto tS = [&](int mt, int j) -> uint32_t { return tmem + static_cast<uint32_t>((2 * mt + j) * kSTok); };
-  auto tO = [&](int mt) -> uint32_t { return tmem + static_cast<uint32_t>(2 * MT * kSTok + mt * D); };
+  auto tS = [&](int mt, int j) -> uint32_t { return tmem + static_cast<uint32_t>((Cfg::kSBufs * mt + j) * kSTok); };
+  auto tO = [&](int mt) -> uint32_t { return tmem + static_cast<uint32_t>(Cfg::kSBufs * MT * kSTok + mt * D); };
   auto tP = [&](int jb) -> uint32_t { return tmem + static_cast<uint32_t>(2 * kSTok + D + jb * kTileTok); };
   static_assert(CG == 1 || 2 * kSTok + D + 2 * kTileTok <= static_cast<int>(Cfg::kTmemCols), "TMEM columns");
 
@@ -301,7 +333,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
   const int N = L + a.bl;
   const float scl = a.scale_log2;
   const bool diff_mode = a.mode == NLD_MODE_DIFFUSION;
-  const int t_end = min(t_begin + a.chunk, N);
+  const int t_end = min(t_begin + piece.chunk, N);
   const int ntiles = t_begin < t_end ? (t_end - t_begin + kTileTok - 1) / kTileTok : 0;
 
   if (ntiles == 0) {
@@ -312,7 +344,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
       for (int r = threadIdx.x; r < Lay::kMergeRows; r += blockDim.x) lse_stage[r] = -INFINITY;
     } else {
       for (int r = threadIdx.x; r < a.R; r += blockDim.x) {
-        const int i = slot0 + r / a.G, h = g * a.G + (r - (r / a.G) * a.G);
+        const int i = r / a.G, h = g * a.G + (r - (r / a.G) * a.G);
         a.lse_part[((static_cast<size_t>(split) * a.B + b) * a.Hq + h) * a.bl + i] = -INFINITY;
       }
     }
@@ -320,19 +352,20 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
     // ---------------- producers ----------------
     int early_tiles = 0;  // leading tiles made of prefix tokens only
     if (early) {
-      while (early_tiles < kTcStages && early_tiles < ntiles &&
+      while (early_tiles < kVStages && early_tiles < ntiles &&
              min(t_begin + (early_tiles + 1) * kTileTok, t_end) <= L)
         ++early_tiles;
       if (early_tiles == 0) grid_dependency_wait();
     }
-    const int issued = produce_kv<D, kSplitKV>(a, &maps.k, &maps.v, smem, k_full, v_full, k_empty, v_empty, kTcStages,
-                                               g, b, t_begin, t_end, ntiles, lane, warp == 1, first, early_tiles);
+    const int nst = warp == 1 ? kVStages : kTcStages;
+    const int issued =
+        produce_kv<D, kSplitKV>(a, &maps.k, &maps.v, warp == 1 ? smem + Lay::kVOff : smem, k_full, v_full, k_empty,
+                                v_empty, nst, g, b, t_begin, t_end, ntiles, lane, warp == 1, first, early_tiles);
     if (lane == 0 && issued < ntiles) {
       // Stopped early on a wait timeout: let the copies already issued land
       // before the CTA exits (bounded).
       uint64_t* full = kSplitKV && warp == 1 ? v_full : k_full;
-      for (int k = max(0, issued - kTcStages); k < issued; ++k)
-        mbar_wait(&full[k % kTcStages], (k / kTcStages) & 1, a.err);
+      for (int k = max(0, issued - nst); k < issued; ++k) mbar_wait(&full[k % nst], (k / nst) & 1, a.err);
     }
   } else if (warp == kMmaWarp) {
     // ---------------- MMA issuer ----------------
@@ -348,7 +381,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
 #pragma unroll
           for (int cb = 0; cb < D / 64; ++cb)
             tma_load_3d(q_s + cb * (128 * 128) + q * (128 / REP) * 128, &maps.q, q_full, cb * 64, g * a.G,
-                        b * a.bl + slot0);
+                        b * a.bl);
       }
       bool ok = mbar_wait(q_ready, 0, a.err);
       if constexpr (MT == 1) ok = ok && mbar_wait(q_full, 0, a.err);
@@ -356,6 +389,78 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
       const uint32_t q_addr = smem_u32(q_s);
       const uint32_t idesc_s = umma_idesc_bf16(128, kSTok, false);
       const uint32_t idesc_o = umma_idesc_bf16(128, D, true);
+      if constexpr (MT == 2) {
+        // Two M tiles: the score products and PV products of the tiles
+        // alternate, S_{0,j+1} behind PV_{0,j}, S_{1,j+1} behind PV_{1,j}, so
+        // the tensor core works on one tile while the softmax group of the
+        // other turns its S into P. P_{mt,j} lies over S_{mt,j}: the pipe
+        // runs one thread's MMAs in order, so S_{mt,j+1} overwrites it only
+        // after PV_{mt,j}, and s_full of product j + 1 tells the softmax
+        // group that PV_{mt,j} has completed (a commit covers every MMA
+        // before it), which is what a rescale of O needs.
+        const int nprod = (ntiles + 1) / 2;
+        auto wait_tiles = [&](uint64_t* full, int nst, int j) -> bool {
+          const int k = 2 * j;
+          if (!mbar_wait(&full[k % nst], (k / nst) & 1, a.err)) return false;
+          return k + 1 >= ntiles || mbar_wait(&full[(k + 1) % nst], ((k + 1) / nst) & 1, a.err);
+        };
+        auto commit_tiles = [&](uint64_t* empty, int nst, int j) {
+          umma_commit(&empty[(2 * j) % nst]);
+          if (2 * j + 1 < ntiles) umma_commit(&empty[(2 * j + 1) % nst]);
+        };
+        // The second half of a last product with one tile reads a stage no
+        // tile of this CTA still needs; its columns are masked.
+        auto issue_s2 = [&](int mt, int j) {
+          const uint32_t k_addr = smem_u32(smem) + static_cast<uint32_t>(((2 * j) % kTcStages) * Geo::kTileBytes);
+#pragma unroll
+          for (int kk = 0; kk < D / 16; ++kk) {
+            const uint32_t koff = (kk & 3) * 32;
+            const int cb = kk >> 2;
+            umma_bf16(tS(mt, 0), sw128_desc(q_addr + mt * Lay::kQBytes + cb * (128 * 128) + koff, 0, 1024),
+                      sw128_desc(k_addr + cb * 1024 + koff, 0, Geo::kGroup8Bytes), idesc_s,
+                      kk > 0 ? 1u : 0u);
+          }
+          umma_commit(&s_full[mt]);
+        };
+        auto issue_pv2 = [&](int mt, int j) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            if (2 * j + h >= ntiles) break;
+            const uint32_t v_addr = smem_u32(smem + Lay::kVOff + ((2 * j + h) % kVStages) * Geo::kTileBytes);
+#pragma unroll
+            for (int kt = 0; kt < kTileTok / 16; ++kt)
+              umma_bf16_ts(tO(mt), tS(mt, 0) + static_cast<uint32_t>(h * (kTileTok / 2) + kt * 8),
+                           sw128_desc(v_addr + kt * 2 * Geo::kGroup8Bytes, 1024, Geo::kGroup8Bytes), idesc_o,
+                           (j > 0 || h > 0 || kt > 0) ? 1u : 0u);
+          }
+        };
+        ok = ok && wait_tiles(k_full, kTcStages, 0);
+        if (ok) {
+          tc_fence_after();
+          issue_s2(0, 0);
+          issue_s2(1, 0);
+          commit_tiles(k_empty, kTcStages, 0);
+        }
+        for (int j = 0; ok && j < nprod; ++j) {
+          const bool more = j + 1 < nprod;
+          ok = wait_tiles(v_full, kVStages, j);
+#pragma unroll
+          for (int mt = 0; mt < 2; ++mt) {
+            ok = ok && mbar_wait(&p_full[mt], j & 1, a.err);
+            if (!ok) break;
+            tc_fence_after();
+            issue_pv2(mt, j);
+            if (mt == 1) commit_tiles(v_empty, kVStages, j);
+            if (mt == 0 && more) ok = wait_tiles(k_full, kTcStages, j + 1);
+            if (ok && more) issue_s2(mt, j + 1);
+          }
+          if (!ok) break;
+          if (more)
+            commit_tiles(k_empty, kTcStages, j + 1);
+          else
+            umma_commit(o_fin);
+        }
+      }
       // Score product j: tiles kTPS*j .. kTPS*j+kTPS-1, whose K tiles sit in
       // consecutive stages (one operand of kSTok rows per column block). If
       // the last product has a single tile, its second half reads a stage
@@ -478,7 +583,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
           }
         }
       }
-      while (CG == 1 && ok && next_pv < ntiles) {
+      while (CG == 1 && MT == 1 && ok && next_pv < ntiles) {
         bool progressed = false;
         const int t0 = next_s * kTPS;  // first tile of the next score product
         if (next_s < nprod && t0 - kTPS <= next_pv &&
@@ -541,7 +646,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
     const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
     const bool warp_rows = mt * 128 + rq * 32 < a.R;  // warp-uniform: the warp holds a real row
     const bool row_ok = r < a.R;
-    const int row_i = slot0 + r / a.G;                    // block slot of this row
+    const int row_i = r / a.G;                    // block slot of this row
     const int row_h = g * a.G + (r - (r / a.G) * a.G);
     const int sm_tid = threadIdx.x - 32 * kSoftmaxWarp0;  // 0 .. 32*kSmWarps-1 across the softmax warps
     const int grp_tid = sm_tid - cg * 128 * MT;           // 0 .. 128*MT-1 within this softmax group
@@ -613,7 +718,109 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
     };
     float m_run = -INFINITY, l_run = 0.f;
     bool ok = true;
-    if constexpr (CG == 2) {
+    if constexpr (MT == 2) {
+      // Two M tiles, a softmax group each: its step is a whole product, 128
+      // columns a thread. P goes over the S columns it has read.
+      const int nprod = (ntiles + 1) / 2;
+      const int row_warps = tile_row_warps(mt);
+      for (int j = 0; warp_rows && j < nprod; ++j) {
+        const int t_own = t_begin + 2 * j * kTileTok;
+        if (!warp_wait(&s_full[mt], j & 1)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        float s[2 * kTileTok];
+        tmem_ld128(tS(mt, 0) + lane_off, s);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          uint64_t vis;
+          if constexpr (MASKED) {
+            vis = column_mask(t_own + h * kTileTok);
+          } else {
+            const int nv = lim - (t_own + h * kTileTok);
+            vis = nv >= 64 ? ~0ull : nv <= 0 ? 0ull : (1ull << nv) - 1ull;
+          }
+          if (!__all_sync(0xffffffffu, vis == ~0ull)) {
+#pragma unroll
+            for (int e = 0; e < kTileTok; ++e)
+              s[h * kTileTok + e] = ((vis >> e) & 1ull) ? s[h * kTileTok + e] : -INFINITY;
+          }
+        }
+        float pm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+        for (int e = 0; e < 2 * kTileTok; e += 8) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) pm[q] = fmax3(pm[q], s[e + 2 * q], s[e + 2 * q + 1]);
+        }
+        const float mx = fmax3(pm[0], pm[1], fmaxf(pm[2], pm[3])) * scl;  // base-2 units
+        float alpha = 1.f;
+        bool rescale = false;
+        if (m_run == -INFINITY) {
+          m_run = mx;  // nothing accumulated for this row yet
+        } else if (mx > m_run + kRescaleLog2) {
+          alpha = ex2(m_run - mx);
+          m_run = mx;
+          l_run *= alpha;
+          rescale = true;
+        }
+        if (__any_sync(0xffffffffu, rescale)) {
+          // O holds the PV products before j, all completed (s_full)
+          if (lane == 0) atomicAdd(a.rescales, 1ull);
+#pragma unroll 1
+          for (int c = 0; c < D / 16; ++c) {
+            float o[16];
+            const uint32_t ta = tO(mt) + lane_off + static_cast<uint32_t>(c * 16);
+            tmem_ld16(ta, o);
+            uint32_t w[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) w[e] = __float_as_uint(o[e] * alpha);
+            tmem_st_u32<16>(ta, w);
+          }
+        }
+        {
+          const float nmu = m_run == -INFINITY ? 0.f : -m_run;
+          const float2 sc2 = make_float2(scl, scl), nm2 = make_float2(nmu, nmu);
+          float2 ls[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+          const uint32_t tp = tS(mt, 0) + lane_off;
+#pragma unroll
+          for (int c = 0; c < 2 * kTileTok / 16; ++c) {
+            uint32_t w[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              const float2 x = fma2(make_float2(s[c * 16 + 2 * e], s[c * 16 + 2 * e + 1]), sc2, nm2);
+              const float2 pp = make_float2(ex2(x.x), ex2(x.y));
+              ls[e & 1] = add2(ls[e & 1], pp);
+              w[e] = pack_bf16(pp.x, pp.y);
+            }
+            tmem_st_u32<8>(tp + static_cast<uint32_t>(c * 8), w);
+          }
+          l_run += (ls[0].x + ls[0].y) + (ls[1].x + ls[1].y);
+          tmem_wait_st();
+        }
+        const int valid = t_end - t_own;  // tokens of this product
+        if (valid < 2 * kTileTok && (valid & (a.box_tok - 1))) {
+          // V rows past the sequence end inside its last page: each group
+          // zeroes them before its PV product (P is 0 there, but 0 * NaN =
+          // NaN; the other group's PV reads the same zeros).
+          const int kz = 2 * j + valid / kTileTok, st = kz % kVStages;
+          if (!warp_wait(&v_full[st], (kz / kVStages) & 1)) {
+            ok = false;
+            break;
+          }
+          const int r0 = valid % kTileTok, r1 = (r0 + a.box_tok - 1) & ~(a.box_tok - 1);
+          uint8_t* vt = smem + Lay::kVOff + st * Geo::kTileBytes;
+          for (int idx = sm_tid - mt * 128; idx < (r1 - r0) * (D / 8); idx += 32 * row_warps) {
+            const int row = r0 + idx / (D / 8), c = idx % (D / 8);
+            *reinterpret_cast<uint4*>(vt + kv_swz<D>(row, c)) = make_uint4(0, 0, 0, 0);
+          }
+        }
+        fence_proxy_async_smem();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&p_full[mt]);
+      }
+    } else if constexpr (CG == 2) {
       // Two softmax groups over every score product j: group c takes tile
       // 2j + c. The row max of a step is taken over both tiles of the product
       // (each group's tile max, exchanged through shared memory), so the two
@@ -783,7 +990,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
     }
     // One softmax group: a step is one tile, or the whole product with row
     // copies and paired products.
-    for (int k0 = 0; CG == 1 && k0 < ntiles; k0 += kU) {  // k0: first tile of the step
+    for (int k0 = 0; CG == 1 && MT == 1 && k0 < ntiles; k0 += kU) {  // k0: first tile of the step
       const int j = k0 / kTPS, half = k0 % kTPS;  // score product and the step's first 64-token half
       const int step_t0 = t_begin + k0 * kTileTok;
       const int k_own = k0 + h_own;               // the tile holding this thread's columns
@@ -942,7 +1149,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
     // fires, so the K/V ring is free for staging. Warp-uniform, like every condition around the warp-collective
     // TMEM loads and stores below.
     const bool o_ready = __all_sync(
-        0xffffffffu, ok && (CG == 2 ? mbar_wait(o_fin, 0, a.err)
+        0xffffffffu, ok && (CG == 2 || MT == 2 ? mbar_wait(o_fin, 0, a.err)
                                     : mbar_wait(&o_done[(ntiles - 1) % kPBufs], ((ntiles - 1) / kPBufs) & 1, a.err)));
     // Copies of a row (REP > 1) hold its O over disjoint token slices, merged
     // by the split-combine rule (Sec. 3 Mode 2, here on one SM). The work is
@@ -1150,9 +1357,9 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
 #pragma unroll
           for (int x = sr * (D / 64 / kStoreRounds); x < (sr + 1) * (D / 64 / kStoreRounds); ++x) {
             if (split_out)
-              tma_store_4d(&maps.o, smem + x * box_stride, x * 64, g * a.G, slot0, split * a.B + b);
+              tma_store_4d(&maps.o, smem + x * box_stride, x * 64, g * a.G, 0, split * a.B + b);
             else
-              tma_store_3d(&maps.o, smem + x * box_stride, x * 64, g * a.G, b * a.bl + slot0);
+              tma_store_3d(&maps.o, smem + x * box_stride, x * 64, g * a.G, b * a.bl);
           }
           bulk_commit();
         }
@@ -1272,12 +1479,12 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
   }
 }
 
-template <int D, int MT, int REP, int TPS, bool MASKED, bool ORDERED, int CG>
+template <int D, int MT, int REP, int TPS, bool MASKED, int ORDER, int CG>
 cudaError_t configure_tc(int dev) {
   static int configured[64] = {0};
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!__atomic_load_n(&configured[dev], __ATOMIC_ACQUIRE)) {
-    cudaError_t e = cudaFuncSetAttribute(block_attn_tc_kernel<D, MT, REP, TPS, MASKED, ORDERED, CG>,
+    cudaError_t e = cudaFuncSetAttribute(block_attn_tc_kernel<D, MT, REP, TPS, MASKED, ORDER, CG>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(TcLayout<D, MT, TPS>::kBytes + 1024));
     if (e != cudaSuccess) return e;
@@ -1286,26 +1493,22 @@ cudaError_t configure_tc(int dev) {
   return cudaSuccess;
 }
 
-template <int D, int MT, int REP, int TPS, bool MASKED, bool ORDERED, int CG>
+template <int D, int MT, int REP, int TPS, bool MASKED, int ORDER, int CG>
 cudaError_t launch_tc_o(const AttnArgs& a, const TmaMaps& maps, cudaStream_t stream) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  if ((e = configure_tc<D, MT, REP, TPS, MASKED, ORDERED, CG>(dev)) != cudaSuccess) return e;
-  dim3 grid(a.num_splits * a.nh, a.Hkv, a.B);
-  return launch_kernel_cluster(block_attn_tc_kernel<D, MT, REP, TPS, MASKED, ORDERED, CG>, grid,
+  if ((e = configure_tc<D, MT, REP, TPS, MASKED, ORDER, CG>(dev)) != cudaSuccess) return e;
+  const dim3 grid(a.num_splits, a.Hkv, a.B);
+  return launch_kernel_cluster(block_attn_tc_kernel<D, MT, REP, TPS, MASKED, ORDER, CG>, grid,
                                dim3(TcCfg<MT, TPS, CG>::kThreads), TcLayout<D, MT, TPS>::kBytes + 1024, stream,
                                a.csize, maps, a);
 }
 
-// The longest-first order only for the unmasked passes (the table-mask
-// passes run at the block shapes of one sequence).
 template <int D, int MT, int REP, int TPS, bool MASKED, int CG = 1>
 cudaError_t launch_tc_t(const AttnArgs& a, const TmaMaps& maps, cudaStream_t stream) {
-  if constexpr (!MASKED) {
-    if (a.order_by_length) return launch_tc_o<D, MT, REP, TPS, false, true, CG>(a, maps, stream);
-  }
-  return launch_tc_o<D, MT, REP, TPS, MASKED, false, CG>(a, maps, stream);
+  if (a.order_by_length) return launch_tc_o<D, MT, REP, TPS, MASKED, kLongestFirst, CG>(a, maps, stream);
+  return launch_tc_o<D, MT, REP, TPS, MASKED, kGridOrder, CG>(a, maps, stream);
 }
 
 // Resident clusters of the kernel a plan would launch (one CTA per SM
@@ -1320,7 +1523,7 @@ int max_active_clusters_t(int csize) {
   const int slot = csize == 2 ? 0 : csize == 4 ? 1 : csize == 8 ? 2 : 3;
   int v = __atomic_load_n(&cache[dev][slot], __ATOMIC_ACQUIRE);
   if (v) return v - 1;
-  if (configure_tc<D, MT, REP, TPS, false, false, CG>(dev) != cudaSuccess) return 0;
+  if (configure_tc<D, MT, REP, TPS, false, kGridOrder, CG>(dev) != cudaSuccess) return 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(csize, 1, 1);
   cfg.blockDim = dim3(TcCfg<MT, TPS, CG>::kThreads);
@@ -1333,7 +1536,7 @@ int max_active_clusters_t(int csize) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, block_attn_tc_kernel<D, MT, REP, TPS, false, false, CG>, &cfg) !=
+  if (cudaOccupancyMaxActiveClusters(&n, block_attn_tc_kernel<D, MT, REP, TPS, false, kGridOrder, CG>, &cfg) !=
       cudaSuccess) {
     cudaGetLastError();
     n = 0;
@@ -1348,7 +1551,7 @@ int tc_replication(int rows) { return rows > 32 && rows <= 64 ? 2 : 1; }
 
 template <int D>
 int max_active_clusters_d(int csize, int rows) {
-  if (rows > 128) return max_active_clusters_t<D, 2, 1, 1, 1>(csize);
+  if (rows > 128) return max_active_clusters_t<D, 2, 1, 2, 1>(csize);
   switch (tc_replication(rows)) {
     case 2: return max_active_clusters_t<D, 1, 2, 2, 1>(csize);
     default: return max_active_clusters_t<D, 1, 1, 2, 2>(csize);
@@ -1372,11 +1575,8 @@ cudaError_t launch_tc_rep(const AttnArgs& a, const TmaMaps& maps, cudaStream_t s
 
 template <int D, bool MASKED>
 cudaError_t launch_tc_d(const AttnArgs& a, const TmaMaps& maps, cudaStream_t stream) {
-  // Block-slot chunks hold 65..128 rows, which only the two-group kernels
-  // take (they read a.nh; the others assume one chunk).
-  if (a.nh != 1 && (a.R <= 64 || a.R > 128)) return cudaErrorInvalidValue;
-  if (a.R > 128) return launch_tc_t<D, 2, 1, 1, MASKED>(a, maps, stream);
-  if (a.chunk <= TcLayout<D, 1, 2>::kStages * kTileTok) return launch_tc_rep<D, 2, MASKED>(a, maps, stream);
+  if (a.R > 128) return launch_tc_t<D, 2, 1, 2, MASKED>(a, maps, stream);
+  if (a.chunk <= TcLayout<D, 1, 2>::kKStages * kTileTok) return launch_tc_rep<D, 2, MASKED>(a, maps, stream);
   return launch_tc_rep<D, 1, MASKED>(a, maps, stream);
 }
 

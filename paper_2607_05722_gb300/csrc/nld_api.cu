@@ -91,15 +91,7 @@ struct SplitPlan {
   int chunk;     // tokens per split
   int csize;     // cluster size (1 = none)
   int partials;  // splits / csize
-  int nh;        // block-slot chunks: CTAs per (split, sequence, KV head) (1 or 2)
 };
-
-// 129..256 packed rows with an even block length run as two CTAs per
-// (split, sequence, KV head), each with half of the block slots (at most 128
-// rows: one M tile); the pair streams the same K/V tiles at the same time,
-// so the second read is served by L2. An odd block length keeps one CTA with
-// two M tiles.
-int slot_chunks(int rows, int block_len) { return rows > 128 && block_len % 2 == 0 ? 2 : 1; }
 
 // Longest split that still runs paired score products at both head sizes
 // (the ring holds at least 6 tiles at head_dim 128).
@@ -112,10 +104,14 @@ void plan_splits_for(const nld_attn_params_t* p, int block_len, int sms, Cluster
                      SplitPlan* out) {
   const long long max_tokens = static_cast<long long>(p->max_pages_per_seq) * p->page_size;
   const int rows = (p->num_q_heads / p->num_kv_heads) * block_len;
-  const int nh = slot_chunks(rows, block_len);
-  const long long units = static_cast<long long>(p->batch) * p->num_kv_heads * nh;  // CTAs per split
+  const long long units = static_cast<long long>(p->batch) * p->num_kv_heads;  // CTAs per split
   const bool tc = nld::tc_supports(rows, p->head_dim);
-  const bool clusters = tc && nh == 1 && !(p->flags & NLD_ATTN_NO_CLUSTER);
+  // 129..256 rows of an even block length stay unsplit (and never take the
+  // cluster plans below) from half as many units on: their split partials are
+  // bf16, and plans of that many units have always merged in fp32.
+  const bool wide_even = rows > 128 && block_len % 2 == 0;
+  const long long unsplit_units = wide_even ? 2 * units : units;
+  const bool clusters = tc && !wide_even && !(p->flags & NLD_ATTN_NO_CLUSTER);
   const bool automatic = p->num_splits == 0;
   int want = p->num_splits;
   int csize = 1;
@@ -125,10 +121,11 @@ void plan_splits_for(const nld_attn_params_t* p, int block_len, int sms, Cluster
     // ragged lengths (not known on the host) the longest sequence would
     // otherwise set the time; pieces past a shorter sequence's end exit at
     // once. With more units than SMs the hardware scheduler balances them.
-    long long s = sms / units;
-    if (units < sms) {  // a single wave: the longest range would set the time
-      const long long by_chunk = (max_tokens + kMaxAutoChunk - 1) / kMaxAutoChunk;
+    const long long by_chunk = (max_tokens + kMaxAutoChunk - 1) / kMaxAutoChunk;
+    long long s = sms / unsplit_units;
+    if (unsplit_units < sms) {  // a single wave: the longest range would set the time
       if (s < by_chunk) s = by_chunk;
+      if (s > 1 && s < sms / units) s = sms / units;
     }
     const long long by_tiles = (max_tokens + nld::kTileTok - 1) / nld::kTileTok;  // >= one tile per split
     if (s > by_tiles) s = by_tiles;
@@ -141,6 +138,17 @@ void plan_splits_for(const nld_attn_params_t* p, int block_len, int sms, Cluster
         want = cs;
         csize = cs;
       }
+    }
+    // Unsplit units of 129..256 rows that fit in one wave: each runs as a
+    // cluster of two CTAs that take half of its sequence, longest first, and
+    // merge on chip in fp32, so that ragged lengths fill the SMs (14B heads, 16
+    // sequences of 8192..16384 tokens: one CTA each 230 us, pairs 197). With
+    // up to 128 rows, whole sequences measured faster (24 sequences of 64 rows,
+    // 192 units: 60 us against 64; 32 of 32 rows, 256 units: 96 against 111).
+    if (want == 1 && rows > 128 && units < sms && unsplit_units >= sms && p->batch > 1 && p->batch <= 1024 &&
+        max_tokens > kMaxAutoChunk && !(p->flags & NLD_ATTN_NO_CLUSTER) && 2 * clusters_resident(2) >= sms - 1) {
+      want = 2;
+      csize = 2;
     }
   } else if (clusters && want >= 2) {
     for (int cs = 8; cs >= 2; cs >>= 1)
@@ -170,7 +178,6 @@ void plan_splits_for(const nld_attn_params_t* p, int block_len, int sms, Cluster
   out->splits = static_cast<int>(splits);
   out->csize = csize;
   out->partials = static_cast<int>(splits / csize);
-  out->nh = nh;
 }
 
 nld_status_t plan_splits(const nld_attn_params_t* p, int block_len, SplitPlan* out) {
@@ -254,7 +261,7 @@ nld_status_t encode_block_map(CUtensorMap* map, const void* base, const nld::Att
   cuuint32_t estr[3] = {1, 1, 1};
   cuuint64_t dims[3] = {static_cast<cuuint64_t>(D), static_cast<cuuint64_t>(a.Hq), static_cast<cuuint64_t>(a.B) * a.bl};
   cuuint64_t strides[2] = {static_cast<cuuint64_t>(D) * 2, static_cast<cuuint64_t>(D) * 2 * a.Hq};
-  cuuint32_t box[3] = {64, static_cast<cuuint32_t>(a.G), static_cast<cuuint32_t>(a.bl_c)};
+  cuuint32_t box[3] = {64, static_cast<cuuint32_t>(a.G), static_cast<cuuint32_t>(a.bl)};
   CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -277,7 +284,7 @@ nld_status_t encode_out_map(CUtensorMap* map, const nld::AttnArgs& a, int D) {
   cuuint64_t dims[4] = {static_cast<cuuint64_t>(D), static_cast<cuuint64_t>(a.Hq), static_cast<cuuint64_t>(a.bl),
                         static_cast<cuuint64_t>(units)};
   cuuint64_t strides[3] = {row * a.bl, row, row * a.bl * a.Hq};
-  cuuint32_t box[4] = {64, static_cast<cuuint32_t>(a.G), static_cast<cuuint32_t>(a.bl_c), 1};
+  cuuint32_t box[4] = {64, static_cast<cuuint32_t>(a.G), static_cast<cuuint32_t>(a.bl), 1};
   CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, a.o_part, dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -418,9 +425,7 @@ nld_status_t block_attn_impl(const nld_attn_params_t* params, const void* q_bloc
   a.Hkv = params->num_kv_heads;
   a.G = G;
   a.bl = block_len;
-  a.nh = plan.nh;
-  a.bl_c = block_len / plan.nh;
-  a.R = G * a.bl_c;
+  a.R = G * block_len;
   a.page_size = params->page_size;
   a.log2_page = __builtin_ctz(static_cast<unsigned>(params->page_size));
   a.num_pages = params->num_pages;
@@ -435,12 +440,15 @@ nld_status_t block_attn_impl(const nld_attn_params_t* params, const void* q_bloc
   a.scale_log2 = scale * nld::kLog2e;
   a.prefix_ready = (params->flags & NLD_ATTN_PREFIX_READY) ? 1 : 0;
   {
-    // Longest sequences first when one split each leaves more units than SMs
-    // (several waves): the last wave then holds the short sequences.
+    // Longest sequences first when one split (or one cluster pair, whose CTAs
+    // take half of their own sequence) each leaves several waves: the last
+    // wave then holds the short sequences.
     int sms = 0;
     if ((st = device_state(nullptr, &sms)) != NLD_OK) return st;
-    a.order_by_length = (plan.splits == 1 && plan.csize == 1 && a.B > 1 && a.B <= 1024 &&
-                         static_cast<long long>(a.B) * a.Hkv * a.nh > sms)
+    const bool halves = params->num_splits == 0 && plan.csize == 2 && plan.splits == 2 &&
+                        static_cast<long long>(a.B) * a.Hkv * 2 >= sms;
+    a.order_by_length = (((plan.splits == 1 && static_cast<long long>(a.B) * a.Hkv > sms) || halves) && a.B > 1 &&
+                         a.B <= 1024)
                             ? 1
                             : 0;
   }

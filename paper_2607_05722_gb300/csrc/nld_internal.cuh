@@ -33,8 +33,7 @@ struct AttnArgs {
   float* lse_part;             // [S, B, Hq, bl]
   unsigned int* err;           // device error word
   unsigned long long* rescales;  // running-max rescale events (diagnostic counter)
-  int B, Hq, Hkv, G, bl, R;    // R = G * bl_c query rows per CTA
-  int nh, bl_c;                // block-slot chunks per (split, KV head, sequence) (1 or 2), slots per chunk
+  int B, Hq, Hkv, G, bl, R;    // R = G * bl query rows per CTA
   int page_size, log2_page, num_pages, max_pages;
   int box_tok;                 // KV tokens per TMA box (16, 32 or 64; never crosses a page)
   int num_splits, chunk;       // splits and tokens per split (multiple of 16)
@@ -491,6 +490,20 @@ __device__ __forceinline__ void tmem_ld64(uint32_t taddr, float* out) {
   for (int j = 0; j < 64; ++j) out[j] = __uint_as_float(r[j]);
 }
 
+// 128 columns in two loads (early-clobber outputs: the second load still reads
+// its address after the first has written registers).
+__device__ __forceinline__ void tmem_ld128(uint32_t taddr, float* out) {
+  uint32_t r[128];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x64.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, %48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63}, [%128];\n\t"
+               "tcgen05.ld.sync.aligned.32x32b.x64.b32 {%64, %65, %66, %67, %68, %69, %70, %71, %72, %73, %74, %75, %76, %77, %78, %79, %80, %81, %82, %83, %84, %85, %86, %87, %88, %89, %90, %91, %92, %93, %94, %95, %96, %97, %98, %99, %100, %101, %102, %103, %104, %105, %106, %107, %108, %109, %110, %111, %112, %113, %114, %115, %116, %117, %118, %119, %120, %121, %122, %123, %124, %125, %126, %127}, [%129];\n\t"
+               "tcgen05.wait::ld.sync.aligned;"
+               : "=&r"(r[0]), "=&r"(r[1]), "=&r"(r[2]), "=&r"(r[3]), "=&r"(r[4]), "=&r"(r[5]), "=&r"(r[6]), "=&r"(r[7]), "=&r"(r[8]), "=&r"(r[9]), "=&r"(r[10]), "=&r"(r[11]), "=&r"(r[12]), "=&r"(r[13]), "=&r"(r[14]), "=&r"(r[15]), "=&r"(r[16]), "=&r"(r[17]), "=&r"(r[18]), "=&r"(r[19]), "=&r"(r[20]), "=&r"(r[21]), "=&r"(r[22]), "=&r"(r[23]), "=&r"(r[24]), "=&r"(r[25]), "=&r"(r[26]), "=&r"(r[27]), "=&r"(r[28]), "=&r"(r[29]), "=&r"(r[30]), "=&r"(r[31]), "=&r"(r[32]), "=&r"(r[33]), "=&r"(r[34]), "=&r"(r[35]), "=&r"(r[36]), "=&r"(r[37]), "=&r"(r[38]), "=&r"(r[39]), "=&r"(r[40]), "=&r"(r[41]), "=&r"(r[42]), "=&r"(r[43]), "=&r"(r[44]), "=&r"(r[45]), "=&r"(r[46]), "=&r"(r[47]), "=&r"(r[48]), "=&r"(r[49]), "=&r"(r[50]), "=&r"(r[51]), "=&r"(r[52]), "=&r"(r[53]), "=&r"(r[54]), "=&r"(r[55]), "=&r"(r[56]), "=&r"(r[57]), "=&r"(r[58]), "=&r"(r[59]), "=&r"(r[60]), "=&r"(r[61]), "=&r"(r[62]), "=&r"(r[63]), "=&r"(r[64]), "=&r"(r[65]), "=&r"(r[66]), "=&r"(r[67]), "=&r"(r[68]), "=&r"(r[69]), "=&r"(r[70]), "=&r"(r[71]), "=&r"(r[72]), "=&r"(r[73]), "=&r"(r[74]), "=&r"(r[75]), "=&r"(r[76]), "=&r"(r[77]), "=&r"(r[78]), "=&r"(r[79]), "=&r"(r[80]), "=&r"(r[81]), "=&r"(r[82]), "=&r"(r[83]), "=&r"(r[84]), "=&r"(r[85]), "=&r"(r[86]), "=&r"(r[87]), "=&r"(r[88]), "=&r"(r[89]), "=&r"(r[90]), "=&r"(r[91]), "=&r"(r[92]), "=&r"(r[93]), "=&r"(r[94]), "=&r"(r[95]), "=&r"(r[96]), "=&r"(r[97]), "=&r"(r[98]), "=&r"(r[99]), "=&r"(r[100]), "=&r"(r[101]), "=&r"(r[102]), "=&r"(r[103]), "=&r"(r[104]), "=&r"(r[105]), "=&r"(r[106]), "=&r"(r[107]), "=&r"(r[108]), "=&r"(r[109]), "=&r"(r[110]), "=&r"(r[111]), "=&r"(r[112]), "=&r"(r[113]), "=&r"(r[114]), "=&r"(r[115]), "=&r"(r[116]), "=&r"(r[117]), "=&r"(r[118]), "=&r"(r[119]), "=&r"(r[120]), "=&r"(r[121]), "=&r"(r[122]), "=&r"(r[123]), "=&r"(r[124]), "=&r"(r[125]), "=&r"(r[126]), "=&r"(r[127])
+               : "r"(taddr), "r"(taddr + 64)
+               : "memory");
+#pragma unroll
+  for (int j = 0; j < 128; ++j) out[j] = __uint_as_float(r[j]);
+}
+
 // Warp-collective: each lane writes 32 consecutive fp32 columns of its TMEM lane and waits.
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const float* in) {
   uint32_t r[32];
@@ -592,9 +605,8 @@ struct PagePrefetch {
 };
 
 // A producer warp: streams the K (or V) boxes of the tiles of tokens
-// [t_begin, t_end) of (sequence b, KV head g) into an nstage ring, K tiles
-// stage-major, then V tiles stage-major; a tile has 64 / box_tok boxes, one
-// per lane. With kSplit, K and V slots fill and free on their own barriers
+// [t_begin, t_end) of (sequence b, KV head g) into its ring of nstage tiles; a
+// tile has 64 / box_tok boxes, one per lane. With kSplit, K and V slots fill and free on their own barriers
 // (k_full/v_full, k_empty/v_empty), so a K slot is refilled as soon as the
 // score product that read it has completed, before the PV product frees the V
 // slot of the same tile; without it a stage's K and V fill on k_full and free
@@ -614,7 +626,7 @@ struct PagePrefetch {
 // 359.5 -> 355.0 us; one sequence unchanged.
 template <int D, bool kSplit>
 __device__ __forceinline__ int produce_kv(const AttnArgs& a, const CUtensorMap* tmk, const CUtensorMap* tmv,
-                                          uint8_t* stages, uint64_t* k_full, uint64_t* v_full, uint64_t* k_empty,
+                                          uint8_t* ring, uint64_t* k_full, uint64_t* v_full, uint64_t* k_empty,
                                           uint64_t* v_empty, int nstage, int g, int b, int t_begin, int t_end,
                                           int ntiles, int lane, bool warp_v, const PagePrefetch& first,
                                           int early_tiles) {
@@ -622,7 +634,6 @@ __device__ __forceinline__ int produce_kv(const AttnArgs& a, const CUtensorMap* 
   const CUtensorMap* map = warp_v ? tmv : tmk;
   uint64_t* full = kSplit && warp_v ? v_full : k_full;
   uint64_t* empty = kSplit && warp_v ? v_empty : k_empty;
-  uint8_t* ring = warp_v ? stages + nstage * Geo::kTileBytes : stages;
   const int box_tok = a.box_tok;
   const int boxes = kTileTok / box_tok;
   const int t_box = lane * box_tok;  // this lane's box within a tile (lanes below `boxes`)

@@ -811,6 +811,43 @@ def test_attention_kv_boxes(orc, D, P, splits):
             compare_attn(out, lse, ro, rl, f"kv boxes D={D} P={P} S={splits} mode={mode} flags={flags}")
 
 
+@pytest.mark.parametrize("G,bl,D", [(43, 3, 128), (5, 32, 128), (8, 31, 64), (8, 32, 128), (129, 1, 64)])
+def test_attention_two_row_tiles(orc, G, bl, D):
+    """129..256 packed rows (two M tiles of one CTA): one and more score
+    products of one and two K/V tiles, sequence ends inside a tile, one split,
+    streaming splits and a table mask."""
+    lens = [0, 40, 130, 700]
+    case = W.make_block_attn_case("two_tiles", len(lens), G * 2, 2, D, block_len=bl, page_size=16, prefix_lens=lens,
+                                  seed=5)
+    dc = DeviceCase(case)
+    for mode in (W.MODE_DIFFUSION, W.MODE_VERIFY):
+        ro, rl = oracle_full(orc, case, mode)
+        for splits in (1, 3):
+            out, lse = dc.run(mode, num_splits=splits, flags=nld.NLD_ATTN_NO_CLUSTER)
+            compare_attn(out, lse, ro, rl, f"two tiles G={G} bl={bl} S={splits} mode={mode}")
+    table = torch.tensor([(1 << (i + 1)) - 1 if i < 31 else -1 for i in range(bl)], dtype=torch.int64)
+    table = table.to(torch.int32).cuda()  # the causal mask as a table: the verify pass
+    p = dc.params(num_splits=1)
+    out2, lse2 = torch.empty_like(out), torch.empty_like(lse)
+    nld.nld_block_attn_masked(p, dc.q[W.MODE_VERIFY], dc.k, dc.v, dc.table, dc.prefix, bl, table, out2, lse2, None)
+    compare_attn(out2, lse2, ro, rl, f"two tiles G={G} bl={bl} table")
+
+
+def test_attention_halves_of_ragged_sequences(orc):
+    """Unsplit sequences of 129..256 rows as cluster pairs, each CTA half of its
+    own sequence, longest first: lengths from empty to the longest, with a half
+    of no key for the shortest."""
+    lens = [0, 1, 47, 48, 50, 64, 111, 112, 113, 200, 500, 2047, 2080] + [90 + 53 * i for i in range(26)]
+    case = W.make_block_attn_case("halves", len(lens), 20, 2, 64, block_len=16, page_size=16, prefix_lens=lens, seed=6)
+    dc = DeviceCase(case)
+    assert nld.nld_block_attn_num_splits(dc.params(), 16) == 1  # merged on chip or never split
+    for mode in (W.MODE_DIFFUSION, W.MODE_VERIFY):
+        ro, rl = oracle_full(orc, case, mode)
+        for flags in (0, nld.NLD_ATTN_PREFIX_READY, nld.NLD_ATTN_NO_CLUSTER):
+            out, lse = dc.run(mode, flags=flags)
+            compare_attn(out, lse, ro, rl, f"halves mode={mode} flags={flags}")
+
+
 def test_attention_split_sweep(orc):
     case = W.make_block_attn_case("sweep", 1, 8, 2, 128, 16, 16, [1000], seed=9)
     dc = DeviceCase(case)
