@@ -141,7 +141,8 @@ struct TcLayout {
   // [kKStages] k_full, v_full, k_empty, v_empty, s_full[2], s_free[2], p_full[kPBufs], o_done[kPBufs],
   // q_ready, q_full, drain, o_fin, xm_full[2], tmem slot
   static constexpr int kNumBars = 4 * kKStages + 4 + 2 * kPBufs + 4 + 2;
-  static_assert(kNumBars * 8 + 16 <= 512, "barrier reserve");
+  static constexpr int kPieceOff = 512 - 32;  // the CTA's piece (balanced pieces)
+  static_assert(kNumBars * 8 + 16 <= kPieceOff, "barrier reserve");
   // two softmax groups: each row's score max per group, truncated to 24 bits
   // (high 16 bits [2][group][TMEM lane], then the next 8 bits, same order),
   // exchanged every step (two buffers by step parity)
@@ -182,13 +183,80 @@ __device__ __noinline__ int sequence_by_length_rank(const AttnArgs& a, int* scra
 }
 
 // Which (split, KV head, sequence) a CTA takes: its grid position, with the
-// sequences in grid order or longest first.
-constexpr int kGridOrder = 0, kLongestFirst = 1;
+// sequences in grid order or longest first, or a piece of balanced_piece().
+constexpr int kGridOrder = 0, kLongestFirst = 1, kBalanced = 2;
 
-// A CTA's share of the work.
+// Pieces of one launch over sequences of different lengths, chosen on the
+// device, where the lengths are. Sequence b is cut into n_b equal pieces of at
+// most T tokens (whole tiles; n_b <= a.num_splits), with T taken from 32
+// candidates by the estimated time in tokens: the largest piece if all pieces
+// run in one wave, else the mean load of an SM plus half a piece (the pieces
+// start largest first). kPieceTokens is what a piece costs beside its tokens
+// (first tiles, epilogue: about 4 us). All CTAs compute the same plan, and CTA
+// i takes the i-th piece, none (b = -1) past the last. One warp does it, lane
+// b holding sequence b, while the others set the CTA up: the chain of length
+// load, search and page-id load is what it costs, about 2 us a CTA (3 us with
+// the whole block searching through shared memory).
 struct Piece {
-  int b, g, split, chunk;
+  int b, g, split, chunk, pieces;
 };
+constexpr int kPieceTokens = 300;
+
+__device__ __forceinline__ int pieces_of(int tokens, float inv_t, int max_pieces) {
+  return min(max(__float2int_ru(__fmul_rd(__int2float_rd(tokens), inv_t)), 1), max_pieces);
+}
+
+__device__ __noinline__ void balanced_piece(const AttnArgs& a, Piece* out) {
+  constexpr unsigned kFull = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const bool mine = lane < a.B;
+  const int lmax = a.max_pages * a.page_size - a.bl;
+  const int len = mine ? min(max(__ldg(a.prefix_lens + lane), 0), lmax) + a.bl : 0;
+  const int nmax = __reduce_max_sync(kFull, len);
+  const int t0 = ((nmax + a.num_splits - 1) / a.num_splits + 63) & ~63;
+  const int step = max(64, ((max(nmax - t0, 0) + 30) / 31 + 63) & ~63);  // the last candidate reaches nmax
+  float inv_t = __frcp_rd(__int2float_ru(t0 + lane * step));             // rounded down: one piece at T >= nmax
+  int total = 0, cmax = 0;
+  float load = 0.f;
+  for (int b0 = 0; b0 < a.B; b0 += 8) {  // eight sequences' chains in flight; lanes past the batch hold none
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int tokens = __shfl_sync(kFull, len, b0 + u);
+      const int n = tokens > 0 ? pieces_of(tokens, inv_t, a.num_splits) : 0;
+      const int c = (__float2int_ru(__fdividef(static_cast<float>(tokens), static_cast<float>(max(n, 1)))) + 63) & ~63;
+      total += n;
+      cmax = max(cmax, c);
+      load += static_cast<float>(n * (c + kPieceTokens));
+    }
+  }
+  total *= a.Hkv;
+  load *= static_cast<float>(a.Hkv);
+  float est = static_cast<float>(cmax + kPieceTokens);
+  if (total > a.sms)
+    est = fmaxf(est, __fdividef(load, static_cast<float>(a.sms)) + 0.5f * __fdividef(load, static_cast<float>(total)));
+  unsigned key = ~0u;
+  if (total <= static_cast<int>(gridDim.x))
+    key = (min(static_cast<unsigned>(est * 0.0625f), 0x7fffffeu) << 5) | static_cast<unsigned>(lane);
+  const unsigned best = __reduce_min_sync(kFull, key);
+  // the exact pieces of the chosen T: never more than the candidate counted
+  inv_t = __shfl_sync(kFull, inv_t, static_cast<int>(best & 31u));
+  const int n = pieces_of(len, inv_t, a.num_splits);
+  const int chunk = mine ? ((len + n - 1) / n + 63) & ~63 : 64;
+  const int count = (len + chunk - 1) / chunk;  // 0 past the batch
+  int first = 0;  // pieces of the sequences before this one, largest pieces first
+  for (int b0 = 0; b0 < a.B; b0 += 8) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int cu = __shfl_sync(kFull, chunk, b0 + u), nu = __shfl_sync(kFull, count, b0 + u);
+      first += (cu > chunk || (cu == chunk && b0 + u < lane)) ? nu : 0;
+    }
+  }
+  const int i = static_cast<int>(blockIdx.x) - first * a.Hkv;
+  const bool hit = mine && i >= 0 && i < count * a.Hkv;
+  if (hit) *out = {lane, i % a.Hkv, i / a.Hkv, chunk, count};
+  if (__ballot_sync(kFull, hit) == 0u && lane == 0) out->b = -1;
+}
+
 template <int D, int MT, int REP, int TPS, bool MASKED, int ORDER, int CG>
 __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
     block_attn_tc_kernel(const __grid_constant__ TmaMaps maps, const AttnArgs a) {
@@ -237,8 +305,13 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
   // With NLD_ATTN_PREFIX_READY the prefix lengths, the page table and
   // prefix-only K/V tiles are read before the dependency wait.
   const bool early = a.prefix_ready != 0;
-  Piece piece = {static_cast<int>(blockIdx.z), static_cast<int>(blockIdx.y), static_cast<int>(blockIdx.x), a.chunk};
-  const int split = piece.split, g = piece.g;
+  Piece piece = {static_cast<int>(blockIdx.z), static_cast<int>(blockIdx.y), static_cast<int>(blockIdx.x), a.chunk, 0};
+  Piece* picked = reinterpret_cast<Piece*>(reinterpret_cast<uint8_t*>(bars) + Lay::kPieceOff);
+  if constexpr (ORDER == kBalanced) {
+    grid_launch_dependents();
+    if (!early) grid_dependency_wait();
+    if (warp == 2) balanced_piece(a, picked);
+  }
   // two M tiles: softmax warps of an M tile that hold real rows
   auto tile_row_warps = [&](int mt) -> int { return min(4, (a.R - mt * 128 + 31) / 32); };
 
@@ -283,12 +356,26 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
     tmem_alloc(tmem_slot, Cfg::kTmemCols);
     tc_fence_before();
   }
+  if constexpr (ORDER == kBalanced) {
+    __syncthreads();
+    piece = *picked;
+    if (piece.b < 0) {  // more CTAs than pieces
+      if (warp == kMmaWarp) {
+        tc_fence_after();
+        tmem_dealloc(*tmem_slot, Cfg::kTmemCols);
+      }
+      return;
+    }
+  }
+  const int split = piece.split, g = piece.g;
   // Without NLD_ATTN_PREFIX_READY nothing global is read before the
   // dependency wait. With it, the page table, the prefix lengths and
   // prefix-only K/V tiles are read first, and only the block slots, Q and the
   // outputs wait (producers: in produce_kv; softmax warps: before Q).
-  grid_launch_dependents();  // dependents launch early; they wait on this grid themselves
-  if (!early) grid_dependency_wait();
+  if constexpr (ORDER != kBalanced) {
+    grid_launch_dependents();  // dependents launch early; they wait on this grid themselves
+    if (!early) grid_dependency_wait();
+  }
   // kLongestFirst (one split per sequence and more (sequence, KV head) units
   // than SMs): CTAs start in z order, so CTA z takes the sequence of rank z by
   // prefix length and the last wave holds the short ones. The ranks are
@@ -685,6 +772,16 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
     }
 
     if (MT == 1 && early) grid_dependency_wait();  // before the mask table and the outputs
+    if constexpr (ORDER == kBalanced) {
+      // The sequence's unused split slots carry no keys.
+      if (split == 0) {
+        for (int idx = sm_tid; idx < (a.num_splits - piece.pieces) * a.R; idx += 32 * Cfg::kSmWarps) {
+          const int s = piece.pieces + idx / a.R, ri = idx % a.R;
+          const int i = ri / a.G, h = g * a.G + (ri - i * a.G);
+          a.lse_part[((static_cast<size_t>(s) * a.B + b) * a.Hq + h) * a.bl + i] = -INFINITY;
+        }
+      }
+    }
 
     // The keys this row may see inside [t_begin, t_end) are exactly t < lim
     // (Sec. 2.2: the whole prefix; in the draft pass every block slot, in the
@@ -1499,7 +1596,7 @@ cudaError_t launch_tc_o(const AttnArgs& a, const TmaMaps& maps, cudaStream_t str
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if ((e = configure_tc<D, MT, REP, TPS, MASKED, ORDER, CG>(dev)) != cudaSuccess) return e;
-  const dim3 grid(a.num_splits, a.Hkv, a.B);
+  const dim3 grid = ORDER == kBalanced ? dim3(a.balanced_ctas) : dim3(a.num_splits, a.Hkv, a.B);
   return launch_kernel_cluster(block_attn_tc_kernel<D, MT, REP, TPS, MASKED, ORDER, CG>, grid,
                                dim3(TcCfg<MT, TPS, CG>::kThreads), TcLayout<D, MT, TPS>::kBytes + 1024, stream,
                                a.csize, maps, a);
@@ -1508,6 +1605,9 @@ cudaError_t launch_tc_o(const AttnArgs& a, const TmaMaps& maps, cudaStream_t str
 template <int D, int MT, int REP, int TPS, bool MASKED, int CG = 1>
 cudaError_t launch_tc_t(const AttnArgs& a, const TmaMaps& maps, cudaStream_t stream) {
   if (a.order_by_length) return launch_tc_o<D, MT, REP, TPS, MASKED, kLongestFirst, CG>(a, maps, stream);
+  if constexpr (REP == 1) {  // balanced pieces stream; row copies take short splits
+    if (a.balanced_ctas > 0) return launch_tc_o<D, MT, REP, TPS, MASKED, kBalanced, CG>(a, maps, stream);
+  }
   return launch_tc_o<D, MT, REP, TPS, MASKED, kGridOrder, CG>(a, maps, stream);
 }
 

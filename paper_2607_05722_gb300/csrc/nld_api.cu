@@ -97,6 +97,12 @@ struct SplitPlan {
 // (the ring holds at least 6 tiles at head_dim 128).
 constexpr long long kPairedChunk = 384;
 
+// Several sequences share a launch whose pieces the kernel may balance over
+// the SMs, knowing their lengths.
+bool can_balance(const nld_attn_params_t* p) {
+  return p->num_splits == 0 && p->batch > 1 && p->batch <= nld::kMaxBalanced;
+}
+
 // The plan for `sms` SMs; `clusters_resident(cs)` says how many clusters of
 // cs CTAs can be resident at once (0: none considered).
 template <typename ClustersResident>
@@ -124,7 +130,10 @@ void plan_splits_for(const nld_attn_params_t* p, int block_len, int sms, Cluster
     const long long by_chunk = (max_tokens + kMaxAutoChunk - 1) / kMaxAutoChunk;
     long long s = sms / unsplit_units;
     if (unsplit_units < sms) {  // a single wave: the longest range would set the time
-      if (s < by_chunk) s = by_chunk;
+      // at most one slot more than two waves of CTAs have (balanced pieces use
+      // no more, and the combine reads every slot)
+      const long long by_waves = (2 * sms + units - 1) / units + 1;
+      if (s < by_chunk) s = by_chunk < by_waves ? by_chunk : by_waves;
       if (s > 1 && s < sms / units) s = sms / units;
     }
     const long long by_tiles = (max_tokens + nld::kTileTok - 1) / nld::kTileTok;  // >= one tile per split
@@ -451,6 +460,25 @@ nld_status_t block_attn_impl(const nld_attn_params_t* params, const void* q_bloc
                          a.B <= 1024)
                             ? 1
                             : 0;
+  }
+  // Balanced pieces: a plan of several streaming pieces a sequence, none of
+  // them in clusters, more slots than SMs. The launch has CTAs for two waves,
+  // or one per slot. Measured against the plan's own pieces (8B heads, 32 rows):
+  // 8 sequences of 512..8192 tokens 43.4 -> 38.6 us, 8 of 4096 39.8 -> 32.4, 18
+  // of 8192 115 -> 103; 14B heads, 4 of 4096..16384 77 -> 59. A CTA learns its
+  // piece about 2 us later, so a single wave keeps the plan's pieces, and so
+  // does a plan of at most three that fill their last wave to 90% (12 of 4096:
+  // 46.5 us against 50.5).
+  if (can_balance(params) && plan.csize == 1 && plan.splits > 1 && plan.chunk > kPairedChunk) {
+    int sms = 0;
+    if ((st = device_state(nullptr, &sms)) != NLD_OK) return st;
+    const long long units = static_cast<long long>(a.B) * a.Hkv;
+    const long long ctas = units * plan.splits;
+    const long long waves = (ctas + sms - 1) / sms;
+    if (ctas > sms && units <= 2 * sms && !(plan.splits <= 3 && 10 * ctas >= 9 * waves * sms)) {
+      a.sms = sms;
+      a.balanced_ctas = static_cast<int>(ctas < 2 * sms ? ctas : 2 * sms);
+    }
   }
   if (plan.partials > 1) {
     a.o_part = static_cast<__nv_bfloat16*>(workspace);

@@ -17,6 +17,7 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr int kMaxSplits = 128;
 constexpr int kModeBlockMask = 2;  // block part of the mask from a per-row table
+constexpr int kMaxBalanced = 32;  // sequences of a launch with balanced pieces
 constexpr int kMaxRows = 256;   // (Hq / Hkv) * block_len handled by one CTA (two 128-row M tiles)
 constexpr int kMaxBlock = 32;   // block_len and the decision width n
 constexpr int kTileTok = 64;    // KV tokens per pipeline stage
@@ -42,6 +43,8 @@ struct AttnArgs {
   float scale_log2;            // softmax scale * log2(e)
   int prefix_ready;            // NLD_ATTN_PREFIX_READY: prefix K/V may be read before the dependency wait
   int order_by_length;         // CTA z takes the sequence of rank z by prefix length (longest first)
+  int balanced_ctas;           // > 0: CTAs of a launch whose pieces are balanced on the device (else 0)
+  int sms;                     // SMs, for that
   int csize;                   // thread-block cluster size along the splits (1 = no cluster)
   int num_partials;            // partials written per (b, h, i): num_splits / csize (1 = final output)
 };

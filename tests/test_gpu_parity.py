@@ -848,6 +848,40 @@ def test_attention_halves_of_ragged_sequences(orc):
             compare_attn(out, lse, ro, rl, f"halves mode={mode} flags={flags}")
 
 
+BALANCED_LENS = {
+    "equal": [5000] * 7,
+    "one long": [9000, 0, 1, 2, 40],
+    "spread": [0, 10, 500, 900, 1500, 2300, 3100, 5000, 8000],
+    "many": [13 * i * i % 4999 for i in range(32)],
+}
+
+
+@pytest.mark.parametrize("name", sorted(BALANCED_LENS))
+@pytest.mark.parametrize("G,bl,P", [(4, 8, 16), (5, 32, 64)])
+def test_attention_balanced_pieces(orc, name, G, bl, P):
+    """Several sequences whose pieces are balanced on the device: equal lengths,
+    one that dwarfs the others, a spread and the most sequences it takes;
+    unused split slots hold no keys, also after a call that used them."""
+    lens = BALANCED_LENS[name]
+    Hkv = 8 if len(lens) <= 9 else 2
+    case = W.make_block_attn_case("balanced", len(lens), G * Hkv, Hkv, 64, block_len=bl, page_size=P, prefix_lens=lens,
+                                  seed=8)
+    dc = DeviceCase(case)
+    slots = nld.nld_block_attn_num_splits(dc.params(flags=nld.NLD_ATTN_NO_CLUSTER), bl)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert slots > 1 and slots * len(lens) * Hkv > sms  # the plans whose pieces are balanced
+    rows = sample_rows(case, 400, 3)
+    kv = case.kv
+    for mode in (W.MODE_DIFFUSION, W.MODE_VERIFY):
+        for flags in (nld.NLD_ATTN_NO_CLUSTER, nld.NLD_ATTN_NO_CLUSTER | nld.NLD_ATTN_PREFIX_READY):
+            out, lse = dc.run(mode, flags=flags)
+            ro, rl = orc.block_attn_rows(dc.q_bits(mode), kv.k_bits, kv.v_bits, kv.page_table, kv.prefix_lens,
+                                         case.num_q_heads, case.num_kv_heads, bl, mode, case.scale, rows)
+            o = out[rows[:, 0], rows[:, 1], rows[:, 2]]
+            l = lse[rows[:, 0], rows[:, 2], rows[:, 1]]
+            compare_attn(o, l, ro, rl, f"balanced {name} G={G} mode={mode} flags={flags}")
+
+
 def test_attention_split_sweep(orc):
     case = W.make_block_attn_case("sweep", 1, 8, 2, 128, 16, 16, [1000], seed=9)
     dc = DeviceCase(case)
