@@ -122,17 +122,27 @@ def _check(status: int, what: str):
         raise NldError(status, what)
 
 
-def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+# A call's own work on the host is about 3 us; the checks and marshalling below
+# are kept to about as much (a decision call took 8.6 us, an attention call
+# 14.1, with a Stream object and c_void_p objects made for each argument).
+def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
+    return None if t is None else t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)  # absent in CPU builds
+
+
+def _stream(stream) -> int:
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _expect(t: torch.Tensor, dtype, shape, name):
+    if t.dtype is dtype and t.shape == shape and t.is_cuda and t.is_contiguous():
+        return
     if t.dtype != dtype:
         raise TypeError(f"{name}: dtype {t.dtype}, expected {dtype}")
     if tuple(t.shape) != tuple(shape):
