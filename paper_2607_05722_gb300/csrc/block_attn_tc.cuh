@@ -1617,11 +1617,11 @@ cudaError_t launch_tc_t(const AttnArgs& a, const TmaMaps& maps, cudaStream_t str
 // uses the instantiation that runs).
 template <int D, int MT, int REP, int TPS, int CG>
 int max_active_clusters_t(int csize) {
-  static int cache[64][4];  // [device][cluster size 2/4/8] + 1 (0 = not queried)
+  static int cache[64][9];  // [device][cluster size] + 1 (0 = not queried)
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  const int slot = csize == 2 ? 0 : csize == 4 ? 1 : csize == 8 ? 2 : 3;
-  int v = __atomic_load_n(&cache[dev][slot], __ATOMIC_ACQUIRE);
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || csize < 2 || csize > 8)
+    return 0;
+  int v = __atomic_load_n(&cache[dev][csize], __ATOMIC_ACQUIRE);
   if (v) return v - 1;
   if (configure_tc<D, MT, REP, TPS, false, kGridOrder, CG>(dev) != cudaSuccess) return 0;
   cudaLaunchConfig_t cfg = {};
@@ -1641,7 +1641,7 @@ int max_active_clusters_t(int csize) {
     cudaGetLastError();
     n = 0;
   }
-  __atomic_store_n(&cache[dev][slot], n + 1, __ATOMIC_RELEASE);
+  __atomic_store_n(&cache[dev][csize], n + 1, __ATOMIC_RELEASE);
   return n;
 }
 

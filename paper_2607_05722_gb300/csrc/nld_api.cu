@@ -79,9 +79,8 @@ nld_status_t check_params(const nld_attn_params_t* p, int block_len) {
 // On the tcgen05 kernel the splits of a (sequence, KV head) can run as one
 // thread-block cluster that merges its results on chip and writes the final
 // output, so no workspace and no combine launch are needed. An automatic plan
-// takes floor(SMs / units) splits (one wave) and, when that is 2..8, rounds
-// it down to 2, 4 or 8 and uses one cluster per unit if those clusters are
-// resident at once. An explicit split count of 2, 4 or 8 uses one cluster; a
+// takes floor(SMs / units) splits (one wave) and, when that is 2..8, uses one
+// cluster of as many CTAs per unit as are resident for all units at once. An explicit split count of 2, 4 or 8 uses one cluster; a
 // larger count divisible by 8, 4 or 2 uses clusters of that size, leaving
 // one partial per cluster for the combine.
 constexpr long long kMaxAutoChunk = 2048;  // tokens per piece in an automatic plan (1 MiB of K+V at D=128)
@@ -142,8 +141,14 @@ void plan_splits_for(const nld_attn_params_t* p, int block_len, int sms, Cluster
     if (s < 1) s = 1;
     want = static_cast<int>(s);
     if (clusters && want >= 2 && want <= 8) {
-      const int cs = want >= 8 ? 8 : want >= 4 ? 4 : 2;
-      if (units <= clusters_resident(cs)) {
+      // The largest cluster resident for every unit at once: 8B heads, 3
+      // sequences of 4000 tokens as clusters of 6 15.6 us, of 4 16.4; 5 of 3000
+      // of 3 17.1, of 2 20.4. Sizes between the powers of two only for pieces
+      // of two score products or more (28 units of 912 tokens: 5 pieces 10.5
+      // us, 4 pieces 10.1).
+      int cs = want;
+      while (cs >= 2 && (units > clusters_resident(cs) || (!is_pow2(cs) && max_tokens < 256 * cs))) --cs;
+      if (cs >= 2) {
         want = cs;
         csize = cs;
       }
@@ -176,7 +181,7 @@ void plan_splits_for(const nld_attn_params_t* p, int block_len, int sms, Cluster
     const long long c2 = (chunk + 2 * nld::kTileTok - 1) / (2 * nld::kTileTok) * (2 * nld::kTileTok);
     const long long s2 = (max_tokens + c2 - 1) / c2;
     if (s2 * 100 >= static_cast<long long>(want) * 85) chunk = c2;
-  } else if (automatic && csize == 1 && tc) {
+  } else if (automatic && tc) {
     // Streaming splits end on a whole tile when that keeps their number.
     const long long c1 = (chunk + nld::kTileTok - 1) / nld::kTileTok * nld::kTileTok;
     if ((max_tokens + c1 - 1) / c1 == (max_tokens + chunk - 1) / chunk) chunk = c1;

@@ -882,6 +882,24 @@ def test_attention_balanced_pieces(orc, name, G, bl, P):
             compare_attn(o, l, ro, rl, f"balanced {name} G={G} mode={mode} flags={flags}")
 
 
+@pytest.mark.parametrize("B,Hkv,G,bl", [(3, 8, 4, 16), (5, 8, 4, 8), (7, 4, 5, 7), (5, 4, 7, 19)])
+def test_attention_automatic_clusters(orc, B, Hkv, G, bl):
+    """Automatic plans that merge on chip in clusters of any size from 2 to 8:
+    6, 3, 5 and 7 resident CTAs a unit, where the device has them."""
+    lens = [2600 - 517 * b for b in range(B)] if B < 6 else [2600 - 371 * b for b in range(B)]
+    case = W.make_block_attn_case("auto_clusters", B, Hkv * G, Hkv, 64, block_len=bl, page_size=32, prefix_lens=lens,
+                                  seed=9)
+    dc = DeviceCase(case)
+    rows = sample_rows(case, 300, 4)
+    kv = case.kv
+    for mode in (W.MODE_DIFFUSION, W.MODE_VERIFY):
+        out, lse = dc.run(mode)
+        ro, rl = orc.block_attn_rows(dc.q_bits(mode), kv.k_bits, kv.v_bits, kv.page_table, kv.prefix_lens,
+                                     case.num_q_heads, case.num_kv_heads, bl, mode, case.scale, rows)
+        compare_attn(out[rows[:, 0], rows[:, 1], rows[:, 2]], lse[rows[:, 0], rows[:, 2], rows[:, 1]], ro, rl,
+                     f"auto clusters B={B} mode={mode}")
+
+
 def test_attention_split_sweep(orc):
     case = W.make_block_attn_case("sweep", 1, 8, 2, 128, 16, 16, [1000], seed=9)
     dc = DeviceCase(case)
