@@ -77,8 +77,8 @@ constexpr int kSoftmaxWarp0 = 4;
 // cost ~70 cycles each and a score product's ~137 (both operands, 8 KB, from
 // shared memory), which bounds the kernel: 1.80 us per 128 tokens for 160 rows,
 // 1.90 for 256, from L2 or HBM alike, and 1.70 without any softmax arithmetic.
-// Block-slot halves in two CTAs of one M tile each took 1.29 us a CTA, 2.58 for
-// the pair; one CTA with N = 64 products 2.36.
+// Block-slot halves in two CTAs of one M tile each take 1.29 us a CTA, 2.58 for
+// the pair (they stay for short pieces); one CTA with N = 64 products took 2.36.
 //
 // CG softmax groups per M tile: with CG = 2 (one M tile of up to 128 rows
 // without row copies, paired products) two groups of four warps share the
@@ -367,7 +367,12 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
       return;
     }
   }
-  const int split = piece.split, g = piece.g;
+  // Block-slot halves (a.nh = 2: short pieces of 129..256 packed rows): the two
+  // CTAs of a (split, KV head, sequence) are adjacent along x and hold block
+  // slots [hc*bl_c, (hc+1)*bl_c) of the G heads each, R = G*bl_c rows.
+  constexpr bool kHalves = CG == 2 && ORDER == kGridOrder;
+  const int split = kHalves ? piece.split / a.nh : piece.split, g = piece.g;
+  const int slot0 = kHalves ? (piece.split - split * a.nh) * a.bl_c : 0;  // first block slot of this CTA
   // Without NLD_ATTN_PREFIX_READY nothing global is read before the
   // dependency wait. With it, the page table, the prefix lengths and
   // prefix-only K/V tiles are read first, and only the block slots, Q and the
@@ -431,7 +436,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
       for (int r = threadIdx.x; r < Lay::kMergeRows; r += blockDim.x) lse_stage[r] = -INFINITY;
     } else {
       for (int r = threadIdx.x; r < a.R; r += blockDim.x) {
-        const int i = r / a.G, h = g * a.G + (r - (r / a.G) * a.G);
+        const int i = slot0 + r / a.G, h = g * a.G + (r - (r / a.G) * a.G);
         a.lse_part[((static_cast<size_t>(split) * a.B + b) * a.Hq + h) * a.bl + i] = -INFINITY;
       }
     }
@@ -468,7 +473,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
 #pragma unroll
           for (int cb = 0; cb < D / 64; ++cb)
             tma_load_3d(q_s + cb * (128 * 128) + q * (128 / REP) * 128, &maps.q, q_full, cb * 64, g * a.G,
-                        b * a.bl);
+                        b * a.bl + slot0);
       }
       bool ok = mbar_wait(q_ready, 0, a.err);
       if constexpr (MT == 1) ok = ok && mbar_wait(q_full, 0, a.err);
@@ -733,7 +738,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
     const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
     const bool warp_rows = mt * 128 + rq * 32 < a.R;  // warp-uniform: the warp holds a real row
     const bool row_ok = r < a.R;
-    const int row_i = r / a.G;                    // block slot of this row
+    const int row_i = slot0 + r / a.G;            // block slot of this row
     const int row_h = g * a.G + (r - (r / a.G) * a.G);
     const int sm_tid = threadIdx.x - 32 * kSoftmaxWarp0;  // 0 .. 32*kSmWarps-1 across the softmax warps
     const int grp_tid = sm_tid - cg * 128 * MT;           // 0 .. 128*MT-1 within this softmax group
@@ -1454,9 +1459,9 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
 #pragma unroll
           for (int x = sr * (D / 64 / kStoreRounds); x < (sr + 1) * (D / 64 / kStoreRounds); ++x) {
             if (split_out)
-              tma_store_4d(&maps.o, smem + x * box_stride, x * 64, g * a.G, 0, split * a.B + b);
+              tma_store_4d(&maps.o, smem + x * box_stride, x * 64, g * a.G, slot0, split * a.B + b);
             else
-              tma_store_3d(&maps.o, smem + x * box_stride, x * 64, g * a.G, b * a.bl);
+              tma_store_3d(&maps.o, smem + x * box_stride, x * 64, g * a.G, b * a.bl + slot0);
           }
           bulk_commit();
         }
@@ -1596,7 +1601,7 @@ cudaError_t launch_tc_o(const AttnArgs& a, const TmaMaps& maps, cudaStream_t str
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if ((e = configure_tc<D, MT, REP, TPS, MASKED, ORDER, CG>(dev)) != cudaSuccess) return e;
-  const dim3 grid = ORDER == kBalanced ? dim3(a.balanced_ctas) : dim3(a.num_splits, a.Hkv, a.B);
+  const dim3 grid = ORDER == kBalanced ? dim3(a.balanced_ctas) : dim3(a.num_splits * a.nh, a.Hkv, a.B);
   return launch_kernel_cluster(block_attn_tc_kernel<D, MT, REP, TPS, MASKED, ORDER, CG>, grid,
                                dim3(TcCfg<MT, TPS, CG>::kThreads), TcLayout<D, MT, TPS>::kBytes + 1024, stream,
                                a.csize, maps, a);
@@ -1675,6 +1680,12 @@ cudaError_t launch_tc_rep(const AttnArgs& a, const TmaMaps& maps, cudaStream_t s
 
 template <int D, bool MASKED>
 cudaError_t launch_tc_d(const AttnArgs& a, const TmaMaps& maps, cudaStream_t stream) {
+  // Block-slot halves hold 65..128 rows, which only the two-group kernels in
+  // grid order take (they read a.nh; the others assume one CTA).
+  if (a.nh != 1) {
+    if (a.R <= 64 || a.R > 128 || a.order_by_length || a.balanced_ctas > 0) return cudaErrorInvalidValue;
+    return launch_tc_o<D, 1, 1, 2, MASKED, kGridOrder, 2>(a, maps, stream);
+  }
   if (a.R > 128) return launch_tc_t<D, 2, 1, 2, MASKED>(a, maps, stream);
   if (a.chunk <= TcLayout<D, 1, 2>::kKStages * kTileTok) return launch_tc_rep<D, 2, MASKED>(a, maps, stream);
   return launch_tc_rep<D, 1, MASKED>(a, maps, stream);

@@ -80,9 +80,10 @@ nld_status_t check_params(const nld_attn_params_t* p, int block_len) {
 // thread-block cluster that merges its results on chip and writes the final
 // output, so no workspace and no combine launch are needed. An automatic plan
 // takes floor(SMs / units) splits (one wave) and, when that is 2..8, uses one
-// cluster of as many CTAs per unit as are resident for all units at once. An explicit split count of 2, 4 or 8 uses one cluster; a
-// larger count divisible by 8, 4 or 2 uses clusters of that size, leaving
-// one partial per cluster for the combine.
+// cluster of as many CTAs per unit as are resident for all units at once. An
+// explicit split count of 2, 4 or 8 uses one cluster; a larger count divisible
+// by 8, 4 or 2 uses clusters of that size, leaving one partial per cluster for
+// the combine.
 constexpr long long kMaxAutoChunk = 2048;  // tokens per piece in an automatic plan (1 MiB of K+V at D=128)
 
 struct SplitPlan {
@@ -95,6 +96,15 @@ struct SplitPlan {
 // Longest split that still runs paired score products at both head sizes
 // (the ring holds at least 6 tiles at head_dim 128).
 constexpr long long kPairedChunk = 384;
+
+// A piece of 129..256 rows runs as two CTAs of half the block slots each where
+// all of those fit in one wave: the pair reads every tile twice, but a half's
+// chain is shorter (1.29 us per 128 tokens against 1.80 with two M tiles, Q by
+// TMA, half the rows to store). Automatic plans cut pieces for that up to this
+// length, and else twice as many for one CTA each: one sequence, 14B heads, 1000
+// / 4096 / 16384 tokens take 9.7 / 13.1 / 26.7 us as halves, 12.0 / 13.9 / 24.3
+// with two M tiles.
+constexpr long long kHalvesChunk = 512;
 
 // Several sequences share a launch whose pieces the kernel may balance over
 // the SMs, knowing their lengths.
@@ -133,7 +143,8 @@ void plan_splits_for(const nld_attn_params_t* p, int block_len, int sms, Cluster
       // no more, and the combine reads every slot)
       const long long by_waves = (2 * sms + units - 1) / units + 1;
       if (s < by_chunk) s = by_chunk < by_waves ? by_chunk : by_waves;
-      if (s > 1 && s < sms / units) s = sms / units;
+      // More pieces where they run as one CTA each, not as block-slot halves.
+      if (s > 1 && s < sms / units && max_tokens > s * kHalvesChunk) s = sms / units;
     }
     const long long by_tiles = (max_tokens + nld::kTileTok - 1) / nld::kTileTok;  // >= one tile per split
     if (s > by_tiles) s = by_tiles;
@@ -141,14 +152,17 @@ void plan_splits_for(const nld_attn_params_t* p, int block_len, int sms, Cluster
     if (s < 1) s = 1;
     want = static_cast<int>(s);
     if (clusters && want >= 2 && want <= 8) {
-      // The largest cluster resident for every unit at once: 8B heads, 3
+      // The largest cluster resident for every unit at once, not below the
+      // power of two under `want` (a third of the SMs idle costs more than the
+      // combine): 8B heads, 3
       // sequences of 4000 tokens as clusters of 6 15.6 us, of 4 16.4; 5 of 3000
       // of 3 17.1, of 2 20.4. Sizes between the powers of two only for pieces
       // of two score products or more (28 units of 912 tokens: 5 pieces 10.5
       // us, 4 pieces 10.1).
+      const int floor2 = want >= 8 ? 8 : want >= 4 ? 4 : 2;
       int cs = want;
-      while (cs >= 2 && (units > clusters_resident(cs) || (!is_pow2(cs) && max_tokens < 256 * cs))) --cs;
-      if (cs >= 2) {
+      while (cs >= floor2 && (units > clusters_resident(cs) || (!is_pow2(cs) && max_tokens < 256 * cs))) --cs;
+      if (cs >= floor2) {
         want = cs;
         csize = cs;
       }
@@ -181,7 +195,7 @@ void plan_splits_for(const nld_attn_params_t* p, int block_len, int sms, Cluster
     const long long c2 = (chunk + 2 * nld::kTileTok - 1) / (2 * nld::kTileTok) * (2 * nld::kTileTok);
     const long long s2 = (max_tokens + c2 - 1) / c2;
     if (s2 * 100 >= static_cast<long long>(want) * 85) chunk = c2;
-  } else if (automatic && tc) {
+  } else if (automatic && tc && (csize == 1 || chunk > kPairedChunk)) {
     // Streaming splits end on a whole tile when that keeps their number.
     const long long c1 = (chunk + nld::kTileTok - 1) / nld::kTileTok * nld::kTileTok;
     if ((max_tokens + c1 - 1) / c1 == (max_tokens + chunk - 1) / chunk) chunk = c1;
@@ -236,8 +250,11 @@ EncodeTiledFn encode_fn() {
 
 // Tokens of a K/V box: as many as a page holds, up to a tile, and as the
 // pieces' starts (multiples of `chunk` with more than one split) allow without
-// a box crossing a page: 16, 32 or 64.
+// a box crossing a page: 16, 32 or 64. Short pieces are bound by latency, not
+// by TMA issue, and the zeroing of V rows past a sequence's end, up to a box
+// less one row, is part of it: 16.
 int box_tokens(const nld_attn_params_t* p, const SplitPlan& plan) {
+  if (plan.chunk <= kPairedChunk) return 16;
   int n = p->page_size < nld::kTileTok ? p->page_size : nld::kTileTok;
   while (plan.splits > 1 && plan.chunk % n != 0) n /= 2;  // chunk is a multiple of 16
   return n;
@@ -275,7 +292,7 @@ nld_status_t encode_block_map(CUtensorMap* map, const void* base, const nld::Att
   cuuint32_t estr[3] = {1, 1, 1};
   cuuint64_t dims[3] = {static_cast<cuuint64_t>(D), static_cast<cuuint64_t>(a.Hq), static_cast<cuuint64_t>(a.B) * a.bl};
   cuuint64_t strides[2] = {static_cast<cuuint64_t>(D) * 2, static_cast<cuuint64_t>(D) * 2 * a.Hq};
-  cuuint32_t box[3] = {64, static_cast<cuuint32_t>(a.G), static_cast<cuuint32_t>(a.bl)};
+  cuuint32_t box[3] = {64, static_cast<cuuint32_t>(a.G), static_cast<cuuint32_t>(a.bl_c)};
   CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -298,7 +315,7 @@ nld_status_t encode_out_map(CUtensorMap* map, const nld::AttnArgs& a, int D) {
   cuuint64_t dims[4] = {static_cast<cuuint64_t>(D), static_cast<cuuint64_t>(a.Hq), static_cast<cuuint64_t>(a.bl),
                         static_cast<cuuint64_t>(units)};
   cuuint64_t strides[3] = {row * a.bl, row, row * a.bl * a.Hq};
-  cuuint32_t box[4] = {64, static_cast<cuuint32_t>(a.G), static_cast<cuuint32_t>(a.bl), 1};
+  cuuint32_t box[4] = {64, static_cast<cuuint32_t>(a.G), static_cast<cuuint32_t>(a.bl_c), 1};
   CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, a.o_part, dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -439,7 +456,15 @@ nld_status_t block_attn_impl(const nld_attn_params_t* params, const void* q_bloc
   a.Hkv = params->num_kv_heads;
   a.G = G;
   a.bl = block_len;
-  a.R = G * block_len;
+  {
+    int sms = 0;
+    if ((st = device_state(nullptr, &sms)) != NLD_OK) return st;
+    const bool halves = G * block_len > 128 && block_len % 2 == 0 && plan.csize == 1 &&
+                        2ll * a.B * a.Hkv * plan.splits <= sms;
+    a.nh = halves ? 2 : 1;
+  }
+  a.bl_c = block_len / a.nh;
+  a.R = G * a.bl_c;
   a.page_size = params->page_size;
   a.log2_page = __builtin_ctz(static_cast<unsigned>(params->page_size));
   a.num_pages = params->num_pages;

@@ -34,7 +34,8 @@ struct AttnArgs {
   float* lse_part;             // [S, B, Hq, bl]
   unsigned int* err;           // device error word
   unsigned long long* rescales;  // running-max rescale events (diagnostic counter)
-  int B, Hq, Hkv, G, bl, R;    // R = G * bl query rows per CTA
+  int B, Hq, Hkv, G, bl, R;    // R = G * bl_c query rows per CTA
+  int nh, bl_c;                // CTAs per (split, KV head, sequence) (1 or 2), block slots of each
   int page_size, log2_page, num_pages, max_pages;
   int box_tok;                 // KV tokens per TMA box (16, 32 or 64; never crosses a page)
   int num_splits, chunk;       // splits and tokens per split (multiple of 16)
