@@ -371,8 +371,8 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
   // CTAs of a (split, KV head, sequence) are adjacent along x and hold block
   // slots [hc*bl_c, (hc+1)*bl_c) of the G heads each, R = G*bl_c rows.
   constexpr bool kHalves = CG == 2 && ORDER == kGridOrder;
-  const int split = kHalves ? piece.split / a.nh : piece.split, g = piece.g;
-  const int slot0 = kHalves ? (piece.split - split * a.nh) * a.bl_c : 0;  // first block slot of this CTA
+  const int split = kHalves ? piece.split >> (a.nh - 1) : piece.split, g = piece.g;
+  const int slot0 = kHalves ? (piece.split & (a.nh - 1)) * a.bl_c : 0;  // first block slot of this CTA
   // Without NLD_ATTN_PREFIX_READY nothing global is read before the
   // dependency wait. With it, the page table, the prefix lengths and
   // prefix-only K/V tiles are read first, and only the block slots, Q and the

@@ -13,6 +13,8 @@
 // 9.7 us, 16 / 4 heads, 1000 tokens (16 splits) 7.5 -> 6.6, against ten
 // dependent shuffles for max and sum, all 32 shuffles at any split count and
 // 64-bit row divisions after the wait.
+#include <type_traits>
+
 #include "nld_internal.cuh"
 
 namespace nld {
@@ -28,7 +30,7 @@ __device__ __forceinline__ float warp_max(float x) {
 // Row `row` of R = B*Hq*bl rows (partial row order [B, Hq, bl]), row orow of the
 // output [B, bl, Hq]; o_part [S, R, D] bf16, lse_part [S, R] (natural log).
 // Warp-collective.
-template <int D>
+template <int D, int kRound>
 __device__ __forceinline__ void merge_split_row(const __nv_bfloat16* __restrict__ o_part,
                                                 const float* __restrict__ lse_part,
                                                 int S, long R, long row, long orow,
@@ -36,10 +38,9 @@ __device__ __forceinline__ void merge_split_row(const __nv_bfloat16* __restrict_
   constexpr int V = D / 32;  // dims per lane (2 or 4)
   const int lane = threadIdx.x & 31;
 
-  // One memory round trip per 32 splits: each lane loads its share of the
+  // One memory round trip per kRound splits: each lane loads its share of the
   // partial rows at the same time as the lse values.
   constexpr int kMaxPerLane = kMaxSplits / 32;
-  constexpr int kRound = 32;
   const long split_stride = R * static_cast<long>(D);
   const __nv_bfloat16* base = o_part + row * D + lane * V;
   float ls[kMaxPerLane];
@@ -91,7 +92,7 @@ __device__ __forceinline__ void merge_split_row(const __nv_bfloat16* __restrict_
         if (s0 + u8 >= S) break;  // warp-uniform
 #pragma unroll
         for (int u = u8; u < u8 + 8; ++u) {
-          const float wu = __shfl_sync(0xffffffffu, wsrc, u);  // 0 past S
+          const float wu = __shfl_sync(0xffffffffu, wsrc, (s0 & 31) + u);  // 0 past S
           csum += wu;                                         // every lane takes the whole sum
           if (wu > 0.f) {
 #pragma unroll
@@ -118,7 +119,7 @@ __device__ __forceinline__ void merge_split_row(const __nv_bfloat16* __restrict_
 
 constexpr int kCombineWarps = 8;
 
-template <int D>
+template <int D, int kRound>
 __global__ void __launch_bounds__(kCombineWarps * 32)
     combine_kernel(const __nv_bfloat16* __restrict__ o_part, const float* __restrict__ lse_part, int S, int B, int Hq,
                    int bl, __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
@@ -133,44 +134,49 @@ __global__ void __launch_bounds__(kCombineWarps * 32)
   const long orow = (static_cast<long>(b) * bl + i) * Hq + h;
   grid_dependency_wait();
   if (row >= R) return;
-  merge_split_row<D>(o_part, lse_part, S, R, row, orow, out, lse);
+  merge_split_row<D, kRound>(o_part, lse_part, S, R, row, orow, out, lse);
 }
 
-// The combine is bound by the rate at which an SM pulls partial rows from
-// L2, so its CTAs should sit on as many SMs as possible. At 96 registers a
-// thread two CTAs fit on one SM and the scheduler packs them; when the grid
-// fits in one wave, a dynamic shared-memory request of more than half an SM
-// (used for nothing) keeps it to one CTA per SM (measured at 17 partials x
-// 512 rows: 3.0 -> 2.8 us). Larger grids launch without it.
-constexpr int kSpreadSmemBytes = 120 * 1024;
+// The combine is bound by the rate at which an SM pulls partial rows from L2,
+// so its CTAs should sit on as many SMs as possible, but the scheduler packs
+// them. A dynamic shared-memory request (used for nothing) allows each SM no
+// more CTAs than an even spread puts there, up to four, 1/(n+1) of an SM and a
+// little each (measured at 17 partials x 512 rows, one CTA a SM: 3.0 -> 2.8 us;
+// two to four a SM with rounds of 8 or 16 splits, whose registers leave room for
+// them: 5 slots x 6144 rows, pass with its combine 47.6 -> 45.8 us, 9 x 2560
+// 17.8 -> 17.4; without the spread the smaller kernels pack, 9 x 1280 12.1 ->
+// 12.8). Larger grids launch without it.
+constexpr int kMaxSpread = 4;
+constexpr int spread_bytes(int per_sm) { return 227 * 1024 / (per_sm + 1) + 1024; }
 
-template <int D>
+template <int D, int kRound>
 cudaError_t configure_combine(int dev) {
   static int configured[64] = {0};
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!__atomic_load_n(&configured[dev], __ATOMIC_ACQUIRE)) {
     cudaError_t e =
-        cudaFuncSetAttribute(combine_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpreadSmemBytes);
+        cudaFuncSetAttribute(combine_kernel<D, kRound>, cudaFuncAttributeMaxDynamicSharedMemorySize, spread_bytes(1));
     if (e != cudaSuccess) return e;
     __atomic_store_n(&configured[dev], 1, __ATOMIC_RELEASE);
   }
   return cudaSuccess;
 }
 
-template <int D>
+template <int D, int kRound>
 cudaError_t launch_combine_d(const __nv_bfloat16* o_part, const float* lse_part, int S, int B, int Hq, int bl,
                              __nv_bfloat16* out, float* lse, int sm_count, cudaStream_t stream) {
   const long R = static_cast<long>(B) * Hq * bl;
   const unsigned blocks = static_cast<unsigned>((R + kCombineWarps - 1) / kCombineWarps);
   size_t smem = 0;
-  if (static_cast<long>(blocks) <= sm_count) {
+  const int per_sm = static_cast<int>((blocks + sm_count - 1) / sm_count);
+  if (per_sm <= kMaxSpread) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if ((e = configure_combine<D>(dev)) != cudaSuccess) return e;
-    smem = kSpreadSmemBytes;
+    if ((e = configure_combine<D, kRound>(dev)) != cudaSuccess) return e;
+    smem = spread_bytes(per_sm);
   }
-  return launch_kernel(combine_kernel<D>, dim3(blocks), dim3(kCombineWarps * 32), smem, stream, o_part, lse_part, S,
+  return launch_kernel(combine_kernel<D, kRound>, dim3(blocks), dim3(kCombineWarps * 32), smem, stream, o_part, lse_part, S,
                        B, Hq, bl, out, lse);
 }
 
@@ -178,8 +184,16 @@ cudaError_t launch_combine_d(const __nv_bfloat16* o_part, const float* lse_part,
 
 cudaError_t launch_combine(const __nv_bfloat16* o_part, const float* lse_part, int S, int B, int Hq, int bl, int D,
                            __nv_bfloat16* out, float* lse, int sm_count, cudaStream_t stream) {
-  if (D == 128) return launch_combine_d<128>(o_part, lse_part, S, B, Hq, bl, out, lse, sm_count, stream);
-  return launch_combine_d<64>(o_part, lse_part, S, B, Hq, bl, out, lse, sm_count, stream);
+  auto go = [&](auto d) {
+    constexpr int kD = decltype(d)::value;
+    const long rows = static_cast<long>(B) * Hq * bl;
+    const long blocks = (rows + kCombineWarps - 1) / kCombineWarps;
+    if (S <= 8) return launch_combine_d<kD, 8>(o_part, lse_part, S, B, Hq, bl, out, lse, sm_count, stream);
+    if (S <= 16 || blocks > 2l * sm_count)
+      return launch_combine_d<kD, 16>(o_part, lse_part, S, B, Hq, bl, out, lse, sm_count, stream);
+    return launch_combine_d<kD, 32>(o_part, lse_part, S, B, Hq, bl, out, lse, sm_count, stream);
+  };
+  return D == 128 ? go(std::integral_constant<int, 128>{}) : go(std::integral_constant<int, 64>{});
 }
 
 }  // namespace nld

@@ -539,6 +539,31 @@ def test_combine_matches_oracle(orc, S, D):
     assert np.max(np.abs(gl[fin] - rl[fin])) <= 1e-4
 
 
+@pytest.mark.parametrize("S", [8, 9, 16, 17, 32, 33])
+@pytest.mark.parametrize("B,Hq,bl,D", [(1, 8, 3, 128), (2, 40, 32, 128), (9, 20, 31, 64), (2, 7, 13, 64)])
+def test_combine_split_and_grid_edges(orc, S, B, Hq, bl, D):
+    """Split counts around the rounds of 8, 16 and 32, rows from one CTA to more
+    than four a SM; same bounds as above."""
+    rng = np.random.default_rng(S * 100 + B)
+    o_bits = W.f32_to_bf16_bits(rng.standard_normal((S, B, Hq, bl, D)).astype(np.float32))
+    l = (rng.standard_normal((S, B, Hq, bl)) * 3).astype(np.float32)
+    l[rng.random(l.shape) < 0.3] = -np.inf
+    o_bits[np.broadcast_to((l == -np.inf)[..., None], o_bits.shape)] = 0x7FC0
+    out = torch.empty((B, bl, Hq, D), dtype=torch.bfloat16, device="cuda")
+    lse = torch.empty((B, Hq, bl), dtype=torch.float32, device="cuda")
+    o_dev = torch.from_numpy(np.ascontiguousarray(o_bits).view(np.int16)).view(torch.bfloat16).cuda()
+    nld.nld_split_kv_combine(o_dev, torch.from_numpy(l).cuda(), out, lse)
+    o = np.nan_to_num(W.bf16_bits_to_f32(o_bits), nan=0.0).reshape(S, -1, D)
+    ro, rl = orc.combine(o, l.reshape(S, -1))
+    ro = ro.reshape(B, Hq, bl, D).transpose(0, 2, 1, 3)
+    rl = rl.reshape(B, Hq, bl)
+    assert np.all(np.abs(out.float().cpu().numpy() - ro) <= 2.0 ** -8 * np.abs(ro) + 1e-5)
+    gl = lse.cpu().numpy()
+    fin = np.isfinite(rl)
+    assert np.array_equal(np.isfinite(gl), fin)
+    assert np.max(np.abs(gl[fin] - rl[fin])) <= 1e-4
+
+
 # ---------------------------------------------------------------------------
 # attention: small cases, every row
 # ---------------------------------------------------------------------------
