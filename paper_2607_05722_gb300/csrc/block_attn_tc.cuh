@@ -73,11 +73,13 @@ constexpr int kSoftmaxWarp0 = 4;
 //
 // Two M tiles: one CTA takes all rows of its (sequence, KV head), so every tile
 // is read once. TMEM: an S buffer a tile (P over its consumed columns) and an O
-// a tile, all 512 columns. A product of 128 tokens takes 32 MMAs; a PV product's
-// cost ~70 cycles each and a score product's ~137 (both operands, 8 KB, from
-// shared memory), which bounds the kernel: 1.80 us per 128 tokens for 160 rows,
-// 1.90 for 256, from L2 or HBM alike, and 1.70 without any softmax arithmetic.
-// Block-slot halves in two CTAs of one M tile each take 1.29 us a CTA, 2.58 for
+// a tile, all 512 columns. A product of 128 tokens takes 32 MMAs, and the one
+// thread that issues them bounds the kernel: eight PV MMAs hold it ~70 cycles
+// each, eight score MMAs ~98 (both operands from shared memory), a wait on a
+// barrier that is ready ~110 and a commit ~50. 1.67 us per 128 tokens for 160
+// rows, 1.78 for 248, from L2 or HBM alike (1.80 and 1.90 with K/V barriers for
+// each tile instead of each product; without any softmax arithmetic 0.1 less).
+// Block-slot halves in two CTAs of one M tile each take 1.15 us a CTA, 2.3 for
 // the pair (they stay for short pieces); one CTA with N = 64 products took 2.36.
 //
 // CG softmax groups per M tile: with CG = 2 (one M tile of up to 128 rows
@@ -280,10 +282,14 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* q_s = smem + Lay::kQOff;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Lay::kBarOff);
-  uint64_t* k_full = bars;                   // K (one-group kernels: K and V) slot of stage st landed
-  uint64_t* v_full = bars + kTcStages;       // V slot of stage st landed (split scheme)
-  uint64_t* k_empty = bars + 2 * kTcStages;  // the product that read K (one group: the PV product) of stage st completed
-  uint64_t* v_empty = bars + 3 * kTcStages;  // the PV product that read V of stage st completed (split scheme)
+  // Split scheme: a barrier per slot of two tiles, those of a product (each
+  // wait and commit holds the MMA thread 50 to 100 cycles). Row copies: a
+  // barrier per tile.
+  constexpr int kKSlots = kTcStages / 2, kVSlots = kVStages / 2;
+  uint64_t* k_full = bars;                   // K of the slot landed (row copies: K and V of the stage)
+  uint64_t* v_full = bars + kTcStages;       // V of the slot landed (split scheme)
+  uint64_t* k_empty = bars + 2 * kTcStages;  // the score product that read it (row copies: the PV product) completed
+  uint64_t* v_empty = bars + 3 * kTcStages;  // the PV products that read it completed (split scheme)
   uint64_t* s_full = bars + 4 * kTcStages;
   uint64_t* s_free = s_full + 2;
   uint64_t* p_full = s_free + 2;
@@ -457,7 +463,8 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
       // Stopped early on a wait timeout: let the copies already issued land
       // before the CTA exits (bounded).
       uint64_t* full = kSplitKV && warp == 1 ? v_full : k_full;
-      for (int k = max(0, issued - nst); k < issued; ++k) mbar_wait(&full[k % nst], (k / nst) & 1, a.err);
+      const int done = kSplitKV ? issued / 2 : issued, ring = kSplitKV ? nst / 2 : nst;  // it stops between products
+      for (int k = max(0, done - ring); k < done; ++k) mbar_wait(&full[k % ring], (k / ring) & 1, a.err);
     }
   } else if (warp == kMmaWarp) {
     // ---------------- MMA issuer ----------------
@@ -491,14 +498,8 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
         // group that PV_{mt,j} has completed (a commit covers every MMA
         // before it), which is what a rescale of O needs.
         const int nprod = (ntiles + 1) / 2;
-        auto wait_tiles = [&](uint64_t* full, int nst, int j) -> bool {
-          const int k = 2 * j;
-          if (!mbar_wait(&full[k % nst], (k / nst) & 1, a.err)) return false;
-          return k + 1 >= ntiles || mbar_wait(&full[(k + 1) % nst], ((k + 1) / nst) & 1, a.err);
-        };
-        auto commit_tiles = [&](uint64_t* empty, int nst, int j) {
-          umma_commit(&empty[(2 * j) % nst]);
-          if (2 * j + 1 < ntiles) umma_commit(&empty[(2 * j + 1) % nst]);
+        auto wait_slot = [&](uint64_t* full, int slots, int j) -> bool {
+          return mbar_wait(&full[j % slots], (j / slots) & 1, a.err);
         };
         // The second half of a last product with one tile reads a stage no
         // tile of this CTA still needs; its columns are masked.
@@ -526,29 +527,29 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
                            (j > 0 || h > 0 || kt > 0) ? 1u : 0u);
           }
         };
-        ok = ok && wait_tiles(k_full, kTcStages, 0);
+        ok = ok && wait_slot(k_full, kKSlots, 0);
         if (ok) {
           tc_fence_after();
           issue_s2(0, 0);
           issue_s2(1, 0);
-          commit_tiles(k_empty, kTcStages, 0);
+          umma_commit(&k_empty[0]);
         }
         for (int j = 0; ok && j < nprod; ++j) {
           const bool more = j + 1 < nprod;
-          ok = wait_tiles(v_full, kVStages, j);
+          ok = wait_slot(v_full, kVSlots, j);
 #pragma unroll
           for (int mt = 0; mt < 2; ++mt) {
             ok = ok && mbar_wait(&p_full[mt], j & 1, a.err);
             if (!ok) break;
             tc_fence_after();
             issue_pv2(mt, j);
-            if (mt == 1) commit_tiles(v_empty, kVStages, j);
-            if (mt == 0 && more) ok = wait_tiles(k_full, kTcStages, j + 1);
+            if (mt == 1) umma_commit(&v_empty[j % kVSlots]);
+            if (mt == 0 && more) ok = wait_slot(k_full, kKSlots, j + 1);
             if (ok && more) issue_s2(mt, j + 1);
           }
           if (!ok) break;
           if (more)
-            commit_tiles(k_empty, kTcStages, j + 1);
+            umma_commit(&k_empty[(j + 1) % kKSlots]);
           else
             umma_commit(o_fin);
         }
@@ -573,12 +574,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
           }
         }
         umma_commit(&s_full[j & 1]);
-        // Split scheme: the K slots of this product are free once it
-        // completes (a last product with one tile frees only that tile's slot).
-        if (kSplitKV) {
-          umma_commit(&k_empty[st]);
-          if (kTPS == 2 && j * kTPS + 1 < ntiles) umma_commit(&k_empty[(st + 1) % kTcStages]);
-        }
+        if (kSplitKV) umma_commit(&k_empty[j % kKSlots]);  // the K slot is free once the product completes
       };
       // One softmax group: P of tile h of a product starts at S column h*32
       // (one warp reads the whole product's columns before writing).
@@ -600,7 +596,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
           }
         }
         umma_commit(&o_done[k % kPBufs]);
-        umma_commit(kSplitKV ? &v_empty[st] : &k_empty[st]);
+        umma_commit(&k_empty[st]);
       };
       // Event-driven issue: score product j needs its K tiles and a free S
       // buffer (the softmax warps have read product j-2), and waits until
@@ -620,10 +616,9 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
         // j waits only for its K tiles and for the softmax warps to have read
         // product j - 2 from the S buffer it overwrites, and runs up to two
         // products ahead of the softmax. The PV products of product j (both
-        // tiles into the one O) wait for P_j from all eight softmax warps and,
-        // split scheme, for the V tiles. Each tile's PV commits its stage's
-        // empty barrier, which the softmax warps also read as "PV of this
-        // tile completed".
+        // tiles into the one O) wait for P_j from all eight softmax warps and
+        // for the V tiles, and commit the slot's empty barrier, which the
+        // softmax warps also read as "the PV products of j completed".
         auto issue_pv2 = [&](int j) {
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
@@ -637,26 +632,21 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
               const uint64_t bd = sw128_desc(v_addr + kt * 2 * Geo::kGroup8Bytes, 1024, Geo::kGroup8Bytes);
               umma_bf16_ts(tO(0), p_tmem + kt * 8, bd, idesc_o, (k > 0 || kt > 0) ? 1u : 0u);
             }
-            umma_commit(kSplitKV ? &v_empty[st] : &k_empty[st]);
           }
+          umma_commit(&v_empty[j % kVSlots]);
           if (j == nprod - 1) umma_commit(o_fin);
         };
         int next_p = 0;
         while (ok && next_p < nprod) {
           bool progressed = false;
-          const int t0 = 2 * next_s;
-          if (next_s < nprod && mbar_test(&k_full[t0 % kTcStages], (t0 / kTcStages) & 1) &&
-              (t0 + 1 >= ntiles || mbar_test(&k_full[(t0 + 1) % kTcStages], ((t0 + 1) / kTcStages) & 1)) &&
+          if (next_s < nprod && mbar_test(&k_full[next_s % kKSlots], (next_s / kKSlots) & 1) &&
               (next_s < 2 || mbar_test(&s_free[next_s & 1], ((next_s - 2) >> 1) & 1))) {
             tc_fence_after();
             issue_s(next_s++);
             progressed = true;
           }
-          const int p0 = 2 * next_p;
           if (next_p < next_s && mbar_test(&p_full[next_p & 1], (next_p >> 1) & 1) &&
-              (!kSplitKV || (mbar_test(&v_full[p0 % kTcStages], (p0 / kTcStages) & 1) &&
-                             (p0 + 1 >= ntiles ||
-                              mbar_test(&v_full[(p0 + 1) % kTcStages], ((p0 + 1) / kTcStages) & 1))))) {
+              mbar_test(&v_full[next_p % kVSlots], (next_p / kVSlots) & 1)) {
             tc_fence_after();
             issue_pv2(next_p++);
             progressed = true;
@@ -686,8 +676,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
           issue_s(next_s++);
           progressed = true;
         }
-        if (next_pv < next_s * kTPS && mbar_test(&p_full[next_pv % kPBufs], (next_pv / kPBufs) & 1) &&
-            (!kSplitKV || mbar_test(&v_full[next_pv % kTcStages], (next_pv / kTcStages) & 1))) {
+        if (next_pv < next_s * kTPS && mbar_test(&p_full[next_pv % kPBufs], (next_pv / kPBufs) & 1)) {
           tc_fence_after();
           issue_pv(next_pv++);
           progressed = true;
@@ -906,7 +895,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
           // zeroes them before its PV product (P is 0 there, but 0 * NaN =
           // NaN; the other group's PV reads the same zeros).
           const int kz = 2 * j + valid / kTileTok, st = kz % kVStages;
-          if (!warp_wait(&v_full[st], (kz / kVStages) & 1)) {
+          if (!warp_wait(&v_full[j % kVSlots], (j / kVSlots) & 1)) {
             ok = false;
             break;
           }
@@ -931,12 +920,12 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
       // j % 2 once the PV products of product j - 2 (which read that buffer)
       // have completed; every warp waits for that before it hands product j
       // over, so no warp is ever two products ahead on p_full. The empty
-      // barrier of a tile's stage (committed after its PV product) tells the
-      // softmax warps that PV has completed; a parity wait on it is exact
-      // because every earlier phase of that barrier was waited for two steps
-      // before.
+      // barrier of the slot (committed after its PV products) tells the
+      // softmax warps that they have completed; a parity wait on it is exact
+      // because the slot's previous phase, three products or more before, was
+      // waited for at an earlier step.
       const int nprod = (ntiles + 1) / 2;
-      uint64_t* pv_done = kSplitKV ? v_empty : k_empty;
+      static_assert(CG == 1 || kVSlots >= 3, "three products in the ring");
       for (int j = 0; j < nprod; ++j) {
         const int k = 2 * j + cg;        // this group's tile
         const bool has = k < ntiles;     // warp-uniform (the last product may hold one tile)
@@ -1014,10 +1003,9 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
         }
         if (__any_sync(0xffffffffu, rescale)) {
           // The shared O holds the PV products of products < j: wait for the
-          // last of them (tile 2j - 1; j >= 1 here), then this group scales
-          // its half of O's columns for this warp's rows.
-          const int kl = 2 * j - 1;
-          if (!warp_wait(&pv_done[kl % kTcStages], (kl / kTcStages) & 1)) {
+          // last of them (j >= 1 here), then this group scales its half of
+          // O's columns for this warp's rows.
+          if (!warp_wait(&v_empty[(j - 1) % kVSlots], ((j - 1) / kVSlots) & 1)) {
             ok = false;
             break;
           }
@@ -1035,12 +1023,11 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
         }
         if (j >= 2) {
           // P buffer j % 2 is free once the PV products of product j - 2
-          // (last tile 2j - 3) have completed. Every warp waits, with rows
+          // have completed. Every warp waits, with rows
           // or not: a warp that skipped it could run ahead and arrive on
           // p_full[j % 2] for product j + 2 before the others had arrived
           // for product j, releasing PV_j early.
-          const int kp = 2 * j - 3;
-          if (!warp_wait(&pv_done[kp % kTcStages], (kp / kTcStages) & 1)) {
+          if (!warp_wait(&v_empty[(j - 2) % kVSlots], ((j - 2) / kVSlots) & 1)) {
             ok = false;
             break;
           }
@@ -1072,7 +1059,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
             // V rows past the sequence end inside its last page: zero them
             // (P is 0 there, but 0 * NaN = NaN).
             const int st = k % kTcStages;
-            if (!warp_wait(kSplitKV ? &v_full[st] : &k_full[st], (k / kTcStages) & 1)) {
+            if (!warp_wait(&v_full[j % kVSlots], (j / kVSlots) & 1)) {
               ok = false;
               break;
             }
@@ -1224,7 +1211,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
           // stale or uninitialised data; P is 0 there but 0 * NaN = NaN, so
           // zero those V rows before the PV MMA reads them.
           const int st = k % kTcStages;
-          if (!warp_wait(kSplitKV ? &v_full[st] : &k_full[st], (k / kTcStages) & 1)) {
+          if (!warp_wait(&k_full[st], (k / kTcStages) & 1)) {
             step_ok = false;
             break;
           }

@@ -99,7 +99,7 @@ constexpr long long kPairedChunk = 384;
 
 // A piece of 129..256 rows runs as two CTAs of half the block slots each where
 // all of those fit in one wave: the pair reads every tile twice, but a half's
-// chain is shorter (1.29 us per 128 tokens against 1.80 with two M tiles, Q by
+// chain is shorter (1.15 us per 128 tokens against 1.67 with two M tiles, Q by
 // TMA, half the rows to store). Automatic plans cut pieces for that up to this
 // length, and else twice as many for one CTA each: one sequence, 14B heads, 1000
 // / 4096 / 16384 tokens take 9.7 / 13.1 / 26.7 us as halves, 12.0 / 13.9 / 24.3

@@ -611,10 +611,10 @@ struct PagePrefetch {
 // A producer warp: streams the K (or V) boxes of the tiles of tokens
 // [t_begin, t_end) of (sequence b, KV head g) into its ring of nstage tiles; a
 // tile has 64 / box_tok boxes, one per lane. With kSplit, K and V slots fill and free on their own barriers
-// (k_full/v_full, k_empty/v_empty), so a K slot is refilled as soon as the
-// score product that read it has completed, before the PV product frees the V
-// slot of the same tile; without it a stage's K and V fill on k_full and free
-// on k_empty together. A warp's expect_tx covers only its own boxes, so a full
+// (k_full/v_full, k_empty/v_empty), one per slot of two tiles (nstage is even),
+// so a K slot is refilled as soon as the score product that read it has
+// completed, before the PV products free the V slot of the same tiles; without
+// it a stage's K and V fill on k_full and free on k_empty together. A warp's expect_tx covers only its own boxes, so a full
 // barrier expects one arrival per warp (of its kind, with kSplit). `first`
 // holds the page ids of the first 32 groups, already loaded. With kSplit the
 // `early_tiles` leading tiles issued before the dependency wait go out K
@@ -651,14 +651,17 @@ __device__ __forceinline__ int produce_kv(const AttnArgs& a, const CUtensorMap* 
   // waiting on a slot).
   constexpr int kKFirstBar = 4;
   if (kSplit && warp_v && early_tiles > 0) named_bar_sync(kKFirstBar, 64);
+  const int per_slot = kSplit ? 2 : 1, nslot = nstage / per_slot;
   for (int k = 0; k < ntiles; ++k) {
     const int st = k % nstage;
+    const int use = k / per_slot, slot_bar = use % nslot;  // the barrier's use and slot
+    const bool first_of_slot = !kSplit || (k & 1) == 0;
     // The first `early_tiles` tiles hold prefix tokens only and may be issued
     // before the dependency wait (NLD_ATTN_PREFIX_READY); the rest wait.
     if (k == early_tiles && early_tiles > 0) grid_dependency_wait();
-    if (k >= nstage) {
+    if (k >= nstage && first_of_slot) {
       int ok = 1;
-      if (lane == 0) ok = mbar_wait(&empty[st], ((k / nstage) - 1) & 1, a.err) ? 1 : 0;
+      if (lane == 0) ok = mbar_wait(&empty[slot_bar], ((use / nslot) - 1) & 1, a.err) ? 1 : 0;
       if (!__shfl_sync(0xffffffffu, ok, 0)) break;
     }
     if (k > 0 && (k & 7) == 0) {
@@ -666,12 +669,13 @@ __device__ __forceinline__ int produce_kv(const AttnArgs& a, const CUtensorMap* 
       page_cur = nxt.validate(a, t_begin, t_end, batch, lane);
       if ((k + 8) < ntiles) nxt.load(a, b, t_begin, batch + 1, lane);
     }
-    if (lane == 0) mbar_arrive_expect_tx(&full[st], Geo::kTileBytes);
+    if (lane == 0 && first_of_slot)
+      mbar_arrive_expect_tx(&full[slot_bar], kSplit && k + 1 < ntiles ? 2 * Geo::kTileBytes : Geo::kTileBytes);
     __syncwarp();
     const int page = __shfl_sync(0xffffffffu, page_cur, ((k & 7) * (kTileTok / kGroupTok) + t_box / kGroupTok) & 31);
     if (lane < boxes) {
       const int slot = page < a.num_pages ? ((t_begin + k * kTileTok + t_box) & (a.page_size - 1)) : 0;
-      tma_load_5d(ring + st * Geo::kTileBytes + (t_box / 8) * Geo::kGroup8Bytes, map, &full[st], 0, 0, 0, slot >> 3,
+      tma_load_5d(ring + st * Geo::kTileBytes + (t_box / 8) * Geo::kGroup8Bytes, map, &full[slot_bar], 0, 0, 0, slot >> 3,
                   page * a.Hkv + g);
     }
     issued = k + 1;
