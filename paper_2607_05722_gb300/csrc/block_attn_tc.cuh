@@ -95,8 +95,8 @@ constexpr int kSoftmaxWarp0 = 4;
 // chain S -> softmax -> PV no longer holds the next score products back.
 template <int MT, int TPS, int CG = 1>
 struct TcCfg {
-  static_assert(TPS == 2 || MT == 1, "two M tiles: paired score products");
-  static_assert(CG == 1 || (CG == 2 && MT == 1 && TPS == 2), "two softmax groups: one M tile, paired products");
+  static_assert(TPS == 2, "paired score products");
+  static_assert(CG == 1 || (CG == 2 && MT == 1), "two softmax groups: one M tile");
   static constexpr int kTPS = TPS;               // K/V tiles per score product
   static constexpr int kSTok = kTPS * kTileTok;  // tokens (N) of a score product
   static constexpr int kPBufs = 2 * kTPS;        // tiles in flight between the softmax and PV (barrier slots)
@@ -670,7 +670,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
         const int t0 = next_s * kTPS;  // first tile of the next score product
         if (next_s < nprod && t0 - kTPS <= next_pv &&
             mbar_test(&k_full[t0 % kTcStages], (t0 / kTcStages) & 1) &&
-            (kTPS == 1 || t0 + 1 >= ntiles || mbar_test(&k_full[(t0 + 1) % kTcStages], ((t0 + 1) / kTcStages) & 1)) &&
+            (t0 + 1 >= ntiles || mbar_test(&k_full[(t0 + 1) % kTcStages], ((t0 + 1) / kTcStages) & 1)) &&
             (next_s < 2 || mbar_test(&s_free[next_s & 1], ((next_s - 2) >> 1) & 1))) {
           tc_fence_after();
           issue_s(next_s++);
@@ -1657,9 +1657,9 @@ int max_active_clusters_d(int csize, int rows) {
 // there, and each tile takes 8 MMAs instead of 12. 32-row batches measured
 // 50/75/87 -> 55/86/95% of peak at B = 8, 32, 128 against four row copies; 64
 // rows, 24 sequences of 256..4096 tokens 53.7 -> 45.2 us against two copies.
-template <int D, int TPS, bool MASKED>
+template <int D, bool FITS, bool MASKED>  // FITS: a split sits in the ring whole
 cudaError_t launch_tc_rep(const AttnArgs& a, const TmaMaps& maps, cudaStream_t stream) {
-  if constexpr (TPS == 2) {
+  if constexpr (FITS) {
     if (tc_replication(a.R) == 2) return launch_tc_t<D, 1, 2, 2, MASKED>(a, maps, stream);
   }
   return launch_tc_t<D, 1, 1, 2, MASKED, 2>(a, maps, stream);
@@ -1674,8 +1674,8 @@ cudaError_t launch_tc_d(const AttnArgs& a, const TmaMaps& maps, cudaStream_t str
     return launch_tc_o<D, 1, 1, 2, MASKED, kGridOrder, 2>(a, maps, stream);
   }
   if (a.R > 128) return launch_tc_t<D, 2, 1, 2, MASKED>(a, maps, stream);
-  if (a.chunk <= TcLayout<D, 1, 2>::kKStages * kTileTok) return launch_tc_rep<D, 2, MASKED>(a, maps, stream);
-  return launch_tc_rep<D, 1, MASKED>(a, maps, stream);
+  if (a.chunk <= TcLayout<D, 1, 2>::kKStages * kTileTok) return launch_tc_rep<D, true, MASKED>(a, maps, stream);
+  return launch_tc_rep<D, false, MASKED>(a, maps, stream);
 }
 
 }  // namespace

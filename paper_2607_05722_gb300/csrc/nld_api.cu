@@ -267,14 +267,14 @@ int box_tokens(const nld_attn_params_t* p, const SplitPlan& plan) {
 // 128-byte swizzle: 8-token groups a fixed stride apart, as the MMA operands
 // want them, also over the boxes and tiles that follow one another. Boxes past
 // num_pages read as zeros.
-nld_status_t encode_pool_map(CUtensorMap* map, const void* base, const nld_attn_params_t* p, int box_tok) {
+nld_status_t encode_pool_map(CUtensorMap* map, const void* base, const nld_attn_params_t* p, int num_pages,
+                             int box_tok) {
   EncodeTiledFn fn = encode_fn();
   if (fn == nullptr) return NLD_ERR_CUDA;
-  const long long planes = static_cast<long long>(p->num_pages) * p->num_kv_heads;
-  if (planes > INT_MAX - p->num_kv_heads) return NLD_ERR_UNSUPPORTED;  // coordinates are int
+  const cuuint64_t planes = static_cast<cuuint64_t>(num_pages) * p->num_kv_heads;
   const cuuint64_t D = static_cast<cuuint64_t>(p->head_dim);
   const cuuint64_t P = static_cast<cuuint64_t>(p->page_size);
-  cuuint64_t dims[5] = {64, 8, D / 64, P / 8, static_cast<cuuint64_t>(planes)};
+  cuuint64_t dims[5] = {64, 8, D / 64, P / 8, planes};
   cuuint64_t strides[4] = {D * 2, 128, D * 2 * 8, D * 2 * P};
   cuuint32_t box[5] = {64, 8, static_cast<cuuint32_t>(D / 64), static_cast<cuuint32_t>(box_tok / 8), 1};
   cuuint32_t estr[5] = {1, 1, 1, 1, 1};
@@ -438,8 +438,12 @@ nld_status_t block_attn_impl(const nld_attn_params_t* params, const void* q_bloc
 
   nld::TmaMaps maps;
   const int box_tok = box_tokens(params, plan);
-  if ((st = encode_pool_map(&maps.k, k_pages, params, box_tok)) != NLD_OK) return st;
-  if ((st = encode_pool_map(&maps.v, v_pages, params, box_tok)) != NLD_OK) return st;
+  // (page, KV head) coordinates are int, the page past the pool among them; a
+  // pool of more planes than that would take over 4 TB.
+  const int max_pool = INT_MAX / params->num_kv_heads - 1;
+  const int num_pages = params->num_pages < max_pool ? params->num_pages : max_pool;
+  if ((st = encode_pool_map(&maps.k, k_pages, params, num_pages, box_tok)) != NLD_OK) return st;
+  if ((st = encode_pool_map(&maps.v, v_pages, params, num_pages, box_tok)) != NLD_OK) return st;
 
   const int G = params->num_q_heads / params->num_kv_heads;
   const float scale = params->softmax_scale > 0.f ? params->softmax_scale : 1.0f / sqrtf((float)params->head_dim);
@@ -467,7 +471,7 @@ nld_status_t block_attn_impl(const nld_attn_params_t* params, const void* q_bloc
   a.R = G * a.bl_c;
   a.page_size = params->page_size;
   a.log2_page = __builtin_ctz(static_cast<unsigned>(params->page_size));
-  a.num_pages = params->num_pages;
+  a.num_pages = num_pages;
   a.max_pages = params->max_pages_per_seq;
   a.box_tok = box_tok;
   a.num_splits = plan.splits;
@@ -481,13 +485,17 @@ nld_status_t block_attn_impl(const nld_attn_params_t* params, const void* q_bloc
   {
     // Longest sequences first when one split (or one cluster pair, whose CTAs
     // take half of their own sequence) each leaves several waves: the last
-    // wave then holds the short sequences.
+    // wave then holds the short sequences. With a table mask only ranges above
+    // 2048 tokens, since the ranking takes about 1 us of a CTA's start (31
+    // sequences of 277..555 tokens: 31.4 us ordered, 30.8 in grid order).
+    const bool long_enough = mode != nld::kModeBlockMask ||
+                             static_cast<long long>(params->max_pages_per_seq) * params->page_size > kMaxAutoChunk;
     int sms = 0;
     if ((st = device_state(nullptr, &sms)) != NLD_OK) return st;
     const bool halves = params->num_splits == 0 && plan.csize == 2 && plan.splits == 2 &&
                         static_cast<long long>(a.B) * a.Hkv * 2 >= sms;
     a.order_by_length = (((plan.splits == 1 && static_cast<long long>(a.B) * a.Hkv > sms) || halves) && a.B > 1 &&
-                         a.B <= 1024)
+                         a.B <= 1024 && long_enough)
                             ? 1
                             : 0;
   }
