@@ -134,7 +134,7 @@ int nld_block_attn_kernels(const nld_attn_params_t *params, int block_len);
  * 2), exactly as nld_block_attn launches it. An automatic plan
  * (num_splits = 0) is given as if no cluster were resident: on a device
  * where the plan's 2..8 pieces per (sequence, KV head) fit as resident
- * clusters, the launched plan instead uses one cluster of 2, 4 or 8 per
+ * clusters, the launched plan instead uses one cluster of 2 to 8 per
  * (sequence, KV head) and one partial, and nld_block_attn_num_splits
  * reports that. Returns 0, or -1 for invalid parameters. Touches no device;
  * for tests and capacity planning.
