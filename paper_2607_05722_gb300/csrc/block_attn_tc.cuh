@@ -74,11 +74,12 @@ constexpr int kSoftmaxWarp0 = 4;
 // Two M tiles: one CTA takes all rows of its (sequence, KV head), so every tile
 // is read once. TMEM: an S buffer a tile (P over its consumed columns) and an O
 // a tile, all 512 columns. A product of 128 tokens takes 32 MMAs, and the one
-// thread that issues them bounds the kernel: eight PV MMAs hold it ~70 cycles
-// each, eight score MMAs ~98 (both operands from shared memory), a wait on a
-// barrier that is ready ~110 and a commit ~50. 1.67 us per 128 tokens for 160
-// rows, 1.78 for 248, from L2 or HBM alike (1.80 and 1.90 with K/V barriers for
-// each tile instead of each product; without any softmax arithmetic 0.1 less).
+// thread that issues them bounds the kernel, held by the tensor pipe: 16 PV MMAs
+// ~70 cycles each, 16 score MMAs ~98 (both operands from shared memory), a
+// commit ~50. 1.67 us per 128 tokens for 160 rows, 1.78 for 248, from L2 or HBM
+// alike (1.80 and 1.90 with K/V barriers for each tile instead of each product;
+// without any softmax arithmetic 0.1 less; the same with the thread's waits for
+// K and V done by a softmax warp).
 // Block-slot halves in two CTAs of one M tile each take 1.15 us a CTA, 2.3 for
 // the pair (they stay for short pieces); one CTA with N = 64 products took 2.36.
 //
