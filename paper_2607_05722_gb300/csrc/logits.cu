@@ -17,6 +17,7 @@
 // and confidence 0.
 #include <limits.h>
 
+#include "logits_rows.cuh"
 #include "nld_internal.cuh"
 
 namespace nld {
@@ -293,39 +294,6 @@ __device__ __forceinline__ uint32_t bf16x2_max(uint32_t a, uint32_t b) {
 }
 __device__ __forceinline__ uint32_t vec_max(uint4 w) { return bf16x2_max(bf16x2_max(w.x, w.y), bf16x2_max(w.z, w.w)); }
 
-constexpr uint32_t kNegInf2 = 0xFF80FF80u;  // two bf16 -inf
-
-// Row vectors v0 + t + j*THREADS < v1 into w, all loads in flight (-inf past
-// v1; rows are readable to a multiple of 8).
-template <int THREADS, int VECS>
-__device__ __forceinline__ void load_logit_vecs(const uint4* row, int v0, int v1, int t, uint4 (&w)[VECS]) {
-#pragma unroll
-  for (int j = 0; j < VECS; ++j) {
-    const int v = v0 + t + j * THREADS;
-    w[j] = v < v1 ? __ldg(row + v) : make_uint4(kNegInf2, kNegInf2, kNegInf2, kNegInf2);
-  }
-}
-
-// -inf past the vocabulary in a last vector that it does not fill. Apart from
-// the loads: a branch on the loaded values would wait for them.
-template <int THREADS, int VECS>
-__device__ __forceinline__ void mask_last_vec(int v0, int v1, int t, int vocab, uint4 (&w)[VECS]) {
-  if (v1 * 8 > vocab && (v1 - 1 - v0 - t) % THREADS == 0) {  // this thread holds the partial last vector
-#pragma unroll
-    for (int j = 0; j < VECS; ++j)
-      if (v0 + t + j * THREADS == v1 - 1) {
-        uint32_t q[4] = {w[j].x, w[j].y, w[j].z, w[j].w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int first = (v1 - 1) * 8 + 2 * e;  // the pair's first logit
-          if (first >= vocab) q[e] = kNegInf2;
-          else if (first + 1 == vocab) q[e] = (q[e] & 0xFFFFu) | (kNegInf2 & 0xFFFF0000u);
-        }
-        w[j] = make_uint4(q[0], q[1], q[2], q[3]);
-      }
-  }
-}
-
 // acc += exp(x - m) over the 8 logits of w, m finite: a pair of logits takes
 // two widenings, a paired subtract, multiply and add and two exponentials (4
 // cycles of the MUFU pipe per warp instruction here).
@@ -395,8 +363,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
   grid_dependency_wait();                   // the logits come from the previous kernel
   const uint4* grow = reinterpret_cast<const uint4*>(logits + row * ld);
   uint4 w[kLsMaxVecs];
-  load_logit_vecs<THREADS>(grow, v0, v1, t, w);
-  mask_last_vec<THREADS>(v0, v1, t, vocab, w);
+  load_logit_vecs<THREADS>(grow, v0, v1, t, vocab, w);
   // the max of this thread's logits (NaN is passed over), then of the warp's
   uint32_t vm[kLsMaxVecs];
   uint32_t pm = kNegInf2;
@@ -705,12 +672,11 @@ __global__ void __launch_bounds__(THREADS, VECS == 4 ? 1024 / THREADS : 1)
   grid_launch_dependents();
   grid_dependency_wait();  // the logits come from earlier kernels
   uint4 wa[VECS], wb[VECS];
-  load_logit_vecs<THREADS>(reinterpret_cast<const uint4*>(ar + row * ld), v0, v1, t, wa);
-  load_logit_vecs<THREADS>(reinterpret_cast<const uint4*>(diff + row * ld), v0, v1, t, wb);
+  load_logit_vecs<THREADS>(reinterpret_cast<const uint4*>(ar + row * ld), v0, v1, t, vocab, wa);
+  load_logit_vecs<THREADS>(reinterpret_cast<const uint4*>(diff + row * ld), v0, v1, t, vocab, wb);
 
   // ---- pass 1: (max, sum) of each row over this piece ----
   auto fold = [&](uint4(&w)[VECS], float& m, float& s) {
-    mask_last_vec<THREADS>(v0, v1, t, vocab, w);
     uint32_t pm = kNegInf2;
 #pragma unroll
     for (int j = 0; j < VECS; ++j) pm = bf16x2_max(pm, vec_max(w[j]));
