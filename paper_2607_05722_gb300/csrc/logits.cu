@@ -17,6 +17,8 @@
 // and confidence 0.
 #include <limits.h>
 
+#include <type_traits>
+
 #include "logits_rows.cuh"
 #include "nld_internal.cuh"
 
@@ -336,7 +338,7 @@ __device__ __forceinline__ int first_of_max(const uint4 (&w)[VECS], const uint32
   return jb * STRIDE + e;
 }
 
-template <int THREADS>
+template <int THREADS, int VECS, bool TAIL>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
     logits_argmax_small_kernel(const __nv_bfloat16* __restrict__ logits, int vocab, long ld, int log2_split, int per,
                                int32_t* __restrict__ ids, float* __restrict__ conf, unsigned int* err) {
@@ -362,13 +364,14 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
   grid_launch_dependents();                 // dependents launch early; they wait on this grid themselves
   grid_dependency_wait();                   // the logits come from the previous kernel
   const uint4* grow = reinterpret_cast<const uint4*>(logits + row * ld);
-  uint4 w[kLsMaxVecs];
+  uint4 w[VECS];
   load_logit_vecs<THREADS>(grow, v0, v1, t, vocab, w);
+  if constexpr (TAIL) load_logit_tail<THREADS>(grow, v0, v1, t, vocab, w);
   // the max of this thread's logits (NaN is passed over), then of the warp's
-  uint32_t vm[kLsMaxVecs];
+  uint32_t vm[VECS];
   uint32_t pm = kNegInf2;
 #pragma unroll
-  for (int j = 0; j < kLsMaxVecs; ++j) {
+  for (int j = 0; j < VECS; ++j) {
     vm[j] = vec_max(w[j]);
     pm = bf16x2_max(pm, vm[j]);
   }
@@ -380,7 +383,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
   float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
   const float mref = mw == -INFINITY ? 0.f : mw;
 #pragma unroll
-  for (int j = 0; j < kLsMaxVecs; ++j) add_exps(w[j], mref, acc[j & 1]);
+  for (int j = 0; j < VECS; ++j) add_exps(w[j], mref, acc[j & 1]);
   float s = (acc[0].x + acc[0].y) + (acc[1].x + acc[1].y);
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
@@ -644,8 +647,8 @@ __global__ void __launch_bounds__(kEnThreads)
 // barriers first): 160 x 100003 25.1 us (reading both rows twice, with two
 // exponentials a logit each time: 54.6), 16 x 131072 5.5 us (12.7), 512 x
 // 131072 74 us (132).
-template <int THREADS, int VECS>
-__global__ void __launch_bounds__(THREADS, VECS == 4 ? 1024 / THREADS : 1)
+template <int THREADS, int VECS, bool TAIL>
+__global__ void __launch_bounds__(THREADS, VECS <= 4 ? 1024 / THREADS : 1)
     ensemble_argmax_small_kernel(const __nv_bfloat16* __restrict__ ar, const __nv_bfloat16* __restrict__ diff,
                                  int vocab, long ld, int log2_split, int per, float lambda, int32_t* __restrict__ ids,
                                  float* __restrict__ conf, unsigned int* err) {
@@ -672,17 +675,25 @@ __global__ void __launch_bounds__(THREADS, VECS == 4 ? 1024 / THREADS : 1)
   grid_launch_dependents();
   grid_dependency_wait();  // the logits come from earlier kernels
   uint4 wa[VECS], wb[VECS];
-  load_logit_vecs<THREADS>(reinterpret_cast<const uint4*>(ar + row * ld), v0, v1, t, vocab, wa);
-  load_logit_vecs<THREADS>(reinterpret_cast<const uint4*>(diff + row * ld), v0, v1, t, vocab, wb);
+  const uint4* ga = reinterpret_cast<const uint4*>(ar + row * ld);
+  const uint4* gb = reinterpret_cast<const uint4*>(diff + row * ld);
+  load_logit_vecs<THREADS>(ga, v0, v1, t, vocab, wa);
+  load_logit_vecs<THREADS>(gb, v0, v1, t, vocab, wb);
 
   // ---- pass 1: (max, sum) of each row over this piece ----
-  auto fold = [&](uint4(&w)[VECS], float& m, float& s) {
+  auto fold = [&](const uint4* row_vecs, uint4(&w)[VECS], float& m, float& s) {
+    if constexpr (TAIL) load_logit_tail<THREADS>(row_vecs, v0, v1, t, vocab, w);
     uint32_t pm = kNegInf2;
 #pragma unroll
     for (int j = 0; j < VECS; ++j) pm = bf16x2_max(pm, vec_max(w[j]));
     float lo, hi;
     unpack_bf16(pm, lo, hi);
     m = warp_max(fmaxf(lo, hi));
+    s = 0.f;
+    // A warp past the piece has no sum to take. The branch also keeps the second
+    // row's maxima behind the first row's exponentials (512 x 262144: 180 us
+    // without it, 172 with).
+    if (m == -INFINITY && v0 + warp * 32 >= v1) return;
     float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
     const float mref = m == -INFINITY ? 0.f : m;
 #pragma unroll
@@ -700,8 +711,8 @@ __global__ void __launch_bounds__(THREADS, VECS == 4 ? 1024 / THREADS : 1)
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
   };
   float ma, sa, mb, sb;
-  fold(wa, ma, sa);
-  fold(wb, mb, sb);
+  fold(ga, wa, ma, sa);
+  fold(gb, wb, mb, sb);
   if (lane == 0) {
     red[warp][0] = ma; red[warp][1] = sa; red[warp][2] = mb; red[warp][3] = sb;
   }
@@ -829,24 +840,43 @@ __global__ void __launch_bounds__(THREADS, VECS == 4 ? 1024 / THREADS : 1)
 
 }  // namespace
 
+namespace {
+// launch(THREADS, VECS) with the fewest vectors a thread that hold a piece:
+// slots past the piece are filler whose exponentials cost as much as a logit's
+// (1000 rows x 1000: 125 vectors in 2048 slots 12.4 us, in 256 slots 7.8; 1000
+// x 40000: 1250 in 2048 48.0 us, in 1280 43.8). A test of each slot instead
+// costs full pieces 3 to 6%.
+template <int THREADS, int VECS, int MAX, typename Launch>
+cudaError_t with_vecs(long piece_vecs, Launch launch) {
+  if constexpr (VECS < MAX) {
+    if (piece_vecs > THREADS * VECS) return with_vecs<THREADS, VECS + 1, MAX>(piece_vecs, launch);
+  }
+  return launch(std::integral_constant<int, THREADS>{}, std::integral_constant<int, VECS>{});
+}
+}  // namespace
+
 int logits_split_vectors() { return kLgStageVecs; }
 int logits_piece_limit() { return 512 * kLsMaxVecs; }
 
 cudaError_t launch_ensemble_argmax(const __nv_bfloat16* ar, const __nv_bfloat16* diff, int rows, int vocab, long ld,
                                    int split, float lambda, int32_t* ids, float* conf, unsigned int* err,
                                    cudaStream_t stream) {
+  const bool stream_rows = split == 0;  // whole rows, read twice, whatever their length
+  if (stream_rows) split = 1;
   const dim3 grid(static_cast<unsigned>(static_cast<long>(rows) * split));
   const long piece_vecs = ((static_cast<long>(vocab) + 7) / 8 + split - 1) / split;
   const int log2_split = __builtin_ctz(static_cast<unsigned>(split)), per = static_cast<int>(piece_vecs);
-  if (piece_vecs <= 256 * 4)
-    return launch_kernel_cluster(ensemble_argmax_small_kernel<256, 4>, grid, dim3(256), 0, stream, split, ar, diff,
+  auto in_registers = [&](auto threads, auto vecs) {
+    constexpr int kT = decltype(threads)::value, kV = decltype(vecs)::value;
+    auto* kernel = vocab % 8 ? ensemble_argmax_small_kernel<kT, kV, true> : ensemble_argmax_small_kernel<kT, kV, false>;
+    return launch_kernel_cluster(kernel, grid, dim3(kT), 0, stream, split, ar, diff,
                                  vocab, ld, log2_split, per, lambda, ids, conf, err);
-  if (piece_vecs <= 512 * 4)
-    return launch_kernel_cluster(ensemble_argmax_small_kernel<512, 4>, grid, dim3(512), 0, stream, split, ar, diff,
-                                 vocab, ld, log2_split, per, lambda, ids, conf, err);
-  if (piece_vecs <= 512 * 8)
-    return launch_kernel_cluster(ensemble_argmax_small_kernel<512, 8>, grid, dim3(512), 0, stream, split, ar, diff,
-                                 vocab, ld, log2_split, per, lambda, ids, conf, err);
+  };
+  if (stream_rows)
+    return launch_kernel_cluster(ensemble_argmax_kernel, grid, dim3(kEnThreads), 0, stream, split, ar, diff, vocab, ld,
+                                 split, lambda, ids, conf);
+  if (piece_vecs <= 256 * 4) return with_vecs<256, 1, 4>(piece_vecs, in_registers);
+  if (piece_vecs <= 512 * kLsMaxVecs) return with_vecs<512, 3, kLsMaxVecs>(piece_vecs, in_registers);
   return launch_kernel_cluster(ensemble_argmax_kernel, grid, dim3(kEnThreads), 0, stream, split, ar, diff, vocab, ld,
                                split, lambda, ids, conf);
 }
@@ -866,12 +896,14 @@ cudaError_t launch_logits_argmax(const __nv_bfloat16* logits, int rows, int voca
   const dim3 grid(static_cast<unsigned>(static_cast<long>(rows) * split));
   const long piece_vecs = ((static_cast<long>(vocab) + 7) / 8 + split - 1) / split;
   const int log2_split = __builtin_ctz(static_cast<unsigned>(split));
-  if (piece_vecs <= 256L * kLsMaxVecs)
-    return launch_kernel_cluster(logits_argmax_small_kernel<256>, grid, dim3(256), 0, stream, split, logits, vocab, ld,
+  auto in_registers = [&](auto threads, auto vecs) {
+    constexpr int kT = decltype(threads)::value, kV = decltype(vecs)::value;
+    auto* kernel = vocab % 8 ? logits_argmax_small_kernel<kT, kV, true> : logits_argmax_small_kernel<kT, kV, false>;
+    return launch_kernel_cluster(kernel, grid, dim3(kT), 0, stream, split, logits, vocab, ld,
                                  log2_split, static_cast<int>(piece_vecs), ids, conf, err);
-  if (piece_vecs <= 512L * kLsMaxVecs)
-    return launch_kernel_cluster(logits_argmax_small_kernel<512>, grid, dim3(512), 0, stream, split, logits, vocab, ld,
-                                 log2_split, static_cast<int>(piece_vecs), ids, conf, err);
+  };
+  if (piece_vecs <= 256L * kLsMaxVecs) return with_vecs<256, 1, kLsMaxVecs>(piece_vecs, in_registers);
+  if (piece_vecs <= 512L * kLsMaxVecs) return with_vecs<512, 5, kLsMaxVecs>(piece_vecs, in_registers);
   return launch_kernel_cluster(logits_argmax_kernel, grid, dim3(kLgThreads), kLgSmemBytes, stream, split, logits,
                                vocab, ld, split, ids, conf, err);
 }

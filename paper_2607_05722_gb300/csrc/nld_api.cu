@@ -324,24 +324,62 @@ nld_status_t encode_out_map(CUtensorMap* map, const nld::AttnArgs& a, int D) {
 
 // Pieces (CTAs of one cluster, 1..8) per row of the logits kernels. With fewer
 // rows than SMs: enough to fill the SMs once, of at least 1024 vectors of 8
-// logits each. Then, with any number of rows, as many as bring a piece down to
-// `fit` vectors, what the kernels that keep a piece in registers take with
-// their smallest CTAs, where 8 pieces can be kept in registers at all: at 128
-// rows x 131072 pieces of 2048 vectors take 9.3 us, whole rows streamed 21.9;
-// more pieces than that only add merges (512 rows x 32000: 2 pieces 8.9 us, 4
-// pieces 12.2).
-int logits_split(int rows, int vocab, int sms, int fit) {
+// logits each. Then as many as bring a piece down to `fit` vectors, where 8
+// pieces can be kept in registers at all; a row that one CTA can keep (4096
+// vectors) is cut no further once its pieces fill the SMs (1000 rows x 20000: 4
+// pieces 24.6 us, whole 19.1; as ensemble 31.4 and 21.4). Times here and below:
+// a pass of two reductions with their decisions, or of one ensemble.
+int logits_pieces(int rows, long nvec, int sms, int fit) {
   int split = 1;
   if (rows < sms) {
     const int by_sms = sms / rows;
-    const int by_len = (vocab / 8) / nld::logits_split_vectors();
-    const int want = by_sms < by_len ? by_sms : by_len;
+    const long by_len = nvec / nld::logits_split_vectors();
+    const long want = by_sms < by_len ? by_sms : by_len;
     while (split * 2 <= want && split * 2 <= 8) split *= 2;
   }
-  const long nvec = (static_cast<long>(vocab) + 7) / 8;
-  if (nvec <= 8L * nld::logits_piece_limit())
-    while (split < 8 && nvec > static_cast<long>(split) * fit) split *= 2;
+  const long whole = nld::logits_piece_limit();
+  if (nvec <= 8 * whole)
+    while (split < 8 && nvec > static_cast<long>(split) * fit && (nvec > whole || 2L * split * rows <= sms)) split *= 2;
   return split;
+}
+
+// The pieces' CTAs each pay a chain of merges, so with many rows the streaming
+// kernel, one CTA a row, is ahead where pieces are short for their CTA: at 1000
+// rows x 150000 (8 pieces of 2344 vectors) 128 us against 168, at 3000 x 80000
+// (1250) 200 against 215, at 1000 x 72001 (1126) 75 against 78; at 512 x 200001
+// (3126) both 102, and 200 x 150000 is 45 us in pieces, 51 streamed.
+int logits_split(int rows, int vocab, int sms) {
+  const long nvec = (static_cast<long>(vocab) + 7) / 8;
+  const int split = logits_pieces(rows, nvec, sms, 2048);
+  const long per = (nvec + split - 1) / split;
+  if (split == 8 && rows >= 2 * sms && per > 2048 && per < 3200) return 1;
+  if (split == 8 && ((rows >= 12 * sms && per < 1408) || (rows >= 6 * sms && per < 1200))) return 1;
+  return split;
+}
+
+// 0: the streaming kernel. It reads a row pair twice, and is still ahead of
+// pieces at many rows: with pieces over 2048 vectors, one CTA an SM, at 400 rows
+// x 150000 (2344 vectors) 109 us against 118, 512 x 200001 (3126) 155 against
+// 169, 1000 x 262144 (4096) 305 against 332, and behind at 304 x 170000 (111
+// against 103), 512 x 262144 (195 against 172); below that where a CTA's slots
+// are not nearly full: 1000 rows x 40000 (625 of 768) 54 us against 60, 1000 x
+// 100003 (1563 of 2048) 125 against 142, 700 x 100003 106 against 99, and 512 x
+// 72001 (1126 of 1536) 61 against 68, 512 x 80000 (1250) 66 each; whole rows
+// in one CTA at 3000 x 16392 (2049 of 2560) 58 against 66, 1000 x 16392 23
+// against 21.
+int ensemble_split(int rows, int vocab, int sms) {
+  const long nvec = (static_cast<long>(vocab) + 7) / 8;
+  const int split = logits_pieces(rows, nvec, sms, 1024);
+  const long per = (nvec + split - 1) / split;
+  if (rows < 2 * sms) return split;
+  if (per > 2048) {
+    if (split == 1) return rows >= 12 * sms && per < 2400 ? 0 : 1;
+    return rows >= 6 * sms || per < (rows >= 3 * sms ? 3584 : 2600) ? 0 : split;
+  }
+  if (split > 1 && rows >= 3 * sms && per > 1024 && per < 1200) return 0;
+  const int threads = per <= 1024 ? 256 : 512;
+  const long slots = (per + threads - 1) / threads * threads;
+  return split > 1 && rows >= 6 * sms && 16 * per < 15 * slots ? 0 : split;
 }
 
 }  // namespace
@@ -649,7 +687,7 @@ nld_status_t nld_logits_argmax(const void* logits, int rows, int vocab, int ld, 
   int sms = 0;
   nld_status_t st = device_state(&err, &sms);
   if (st != NLD_OK) return st;
-  const int split = logits_split(rows, vocab, sms, 2048);
+  const int split = logits_split(rows, vocab, sms);
   return nld::launch_logits_argmax(static_cast<const __nv_bfloat16*>(logits), rows, vocab, ld, split, ids, conf, err,
                                    stream) == cudaSuccess
              ? NLD_OK
@@ -666,7 +704,7 @@ nld_status_t nld_logits_ensemble_argmax(const void* ar_logits, const void* diff_
   int sms = 0;
   nld_status_t st = device_state(&err, &sms);
   if (st != NLD_OK) return st;
-  const int split = logits_split(rows, vocab, sms, 1024);
+  const int split = ensemble_split(rows, vocab, sms);
   return nld::launch_ensemble_argmax(static_cast<const __nv_bfloat16*>(ar_logits),
                                      static_cast<const __nv_bfloat16*>(diff_logits), rows, vocab, ld, split, lambda,
                                      ids, conf, err, stream) == cudaSuccess

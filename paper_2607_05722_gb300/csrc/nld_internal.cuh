@@ -79,7 +79,8 @@ cudaError_t launch_logits_argmax(const __nv_bfloat16* logits, int rows, int voca
                                  float* conf, unsigned int* err, cudaStream_t stream);
 int logits_split_vectors();  // 16-byte vectors a CTA streams per ring stage
 int logits_piece_limit();    // 16-byte vectors of a piece that the register kernels take at most
-// AR-diffusion ensemble verifier: `split` CTAs per row pair (a cluster when > 1).
+// AR-diffusion ensemble verifier: `split` CTAs per row pair (a cluster when > 1;
+// 0: one CTA that reads the row pair twice).
 cudaError_t launch_ensemble_argmax(const __nv_bfloat16* ar, const __nv_bfloat16* diff, int rows, int vocab, long ld,
                                    int split, float lambda, int32_t* ids, float* conf, unsigned int* err,
                                    cudaStream_t stream);

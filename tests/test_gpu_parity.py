@@ -417,6 +417,45 @@ def test_ensemble_register_pieces(orc, rows, vocab):
         assert gi[3] == 0 and gc[3] == 0.0
 
 
+def _check_logit_rows(orc, bits_a, bits_d, vocab, copies=1):
+    """Both reductions on `copies` copies of the rows against the oracle's on one."""
+    check = [np.tile(v, copies) for v in orc.logits_argmax(bits_a, vocab)]
+    a, d = np.tile(bits_a, (copies, 1)), np.tile(bits_d, (copies, 1))
+    check_logits(gpu_logits(a, vocab), check, f"rows={a.shape[0]} V={vocab}")
+    gi, gc = gpu_ensemble(a, d, 0.5, vocab)
+    oc = np.tile(orc.ensemble_argmax(bits_a, bits_d, 0.5, vocab)[1], copies)
+    assert np.all(np.abs(gc - oc) <= LOGITS_RTOL * oc)
+    p = mixture_f64(bits_a, bits_d, 0.5, vocab)
+    at = p[np.arange(a.shape[0]) % bits_a.shape[0], gi]
+    assert np.all(at >= oc - 2 * LOGITS_RTOL * oc)
+
+
+# one vector more than 0..7 times 256 and 4..7 times 512: each number of
+# vectors a thread holds, with a partial last vector; 32768: all slots full
+@pytest.mark.parametrize("vocab", [5, 2053, 4101, 6149, 8197, 10245, 12293, 14341, 16389, 20485, 24581, 28677, 32768])
+def test_logits_vectors_per_thread(orc, vocab):
+    rng = np.random.default_rng(vocab)
+    ld = (vocab + 7) // 8 * 8
+    x = (rng.standard_normal((2, 16, ld)) * 3).astype(np.float32)
+    x[:, :, vocab:] = 1e4
+    for r, at in enumerate((0, vocab // 2, vocab - 1)):
+        x[:, r, at] = 20.0                                        # the maximum in the first and the last vector
+    x[:, 3, vocab - 1] = x[:, 3, 0] = 25.0                        # a tie: the lower index
+    x[0, 4, : vocab - 1] = -np.inf                                # only the last logit
+    a, d = W.f32_to_bf16_bits(x[0]), W.f32_to_bf16_bits(x[1])
+    _check_logit_rows(orc, a, d, vocab, copies=10)                # 160 rows: a row to a CTA
+
+
+@pytest.mark.parametrize("vocab,copies", [(140001, 39), (40001, 115), (16392, 229), (72001, 229)])
+def test_logits_many_rows(orc, vocab, copies):
+    """Numbers of rows (312, 920, 1832) from which a streaming kernel takes over."""
+    rng = np.random.default_rng(vocab)
+    x = (rng.standard_normal((2, 8, (vocab + 7) // 8 * 8)) * 3).astype(np.float32)
+    x[:, :, vocab:] = 1e4
+    x[:, 0, vocab - 1] = 25.0
+    _check_logit_rows(orc, W.f32_to_bf16_bits(x[0]), W.f32_to_bf16_bits(x[1]), vocab, copies)
+
+
 def test_logits_peaked_rows(orc):
     """Peaked rows (a confident prediction): the confidence near 1 is kept to
     the same relative bound."""

@@ -15,6 +15,7 @@ HARNESS = r"""
 #include <vector>
 #define __device__
 #define __forceinline__ inline
+struct alignas(8) uint2 { uint32_t x, y; };
 struct alignas(16) uint4 { uint32_t x, y, z, w; };
 static uint4 make_uint4(uint32_t x, uint32_t y, uint32_t z, uint32_t w) { return uint4{x, y, z, w}; }
 static std::vector<int> reads;  // per 16-bit entry of the row
@@ -43,6 +44,7 @@ template <int THREADS, int VECS> static int check(int vocab, int split) {
     for (int t = 0; t < THREADS; ++t) {
       uint4 w[VECS];
       nld::load_logit_vecs<THREADS>(row.data(), v0, v1, t, vocab, w);
+      nld::load_logit_tail<THREADS>(row.data(), v0, v1, t, vocab, w);
       for (int j = 0; j < VECS; ++j)
         for (int e = 0; e < 8; ++e) {
           const long v = v0 + t + (long)j * THREADS, i = v * 8 + e;
@@ -57,7 +59,7 @@ template <int THREADS, int VECS> static int check(int vocab, int split) {
 }
 int main() {
   int n = 0;
-  const int vocabs[] = {1, 2, 7, 8, 9, 15, 16, 2047, 2048, 2050, 8191, 8193, 16383, 16384, 16385, 32766, 32769, 50257};
+  const int vocabs[] = {1, 2, 3, 4, 5, 6, 7, 8, 9, 15, 16, 2047, 2048, 2050, 8191, 8193, 16383, 16384, 16385, 32766, 32769, 50257};
   for (int vocab : vocabs)
     for (int split = 1; split <= 8; split *= 2)
       n += check<256, 8>(vocab, split) + check<512, 8>(vocab, split) + check<256, 4>(vocab, split) + check<512, 4>(vocab, split);
