@@ -140,8 +140,20 @@ void plan_splits_for(const nld_attn_params_t* p, int block_len, int sms, Cluster
     long long s = sms / unsplit_units;
     if (unsplit_units < sms) {  // a single wave: the longest range would set the time
       // at most one slot more than two waves of CTAs have (balanced pieces use
-      // no more, and the combine reads every slot)
-      const long long by_waves = (2 * sms + units - 1) / units + 1;
+      // no more, and the combine reads every slot). Pieces that are not balanced
+      // need more waves to even out while there are few units: 48 units of
+      // 512..32768 tokens 92 us in 2.5 waves, 83 in 4; one sequence of 98304
+      // tokens, 8 units, 95 in 2.05 waves, 89 in 2.5; 128 units 177 in 3.4 waves,
+      // 192 in 4.2. They get them as far as the library's own scratch holds
+      // the partials, so that a call that uses it is not refused for it.
+      long long by_waves = (2 * sms + units - 1) / units + 1;
+      if (!can_balance(p) && 2 * units <= sms) {
+        const long long in_scratch = static_cast<long long>(nld::kStaticScratchBytes - 256) /
+                                     (units * rows * (p->head_dim * 2 + 4));
+        const long long four = (4 * sms + units - 1) / units;
+        const long long more = four < in_scratch ? four : in_scratch;
+        if (more > by_waves) by_waves = more;
+      }
       if (s < by_chunk) s = by_chunk < by_waves ? by_chunk : by_waves;
       // More pieces where they run as one CTA each, not as block-slot halves.
       if (s > 1 && s < sms / units && max_tokens > s * kHalvesChunk) s = sms / units;

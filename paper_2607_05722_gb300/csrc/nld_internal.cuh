@@ -16,6 +16,7 @@ namespace nld {
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr int kMaxSplits = 128;
+constexpr size_t kStaticScratchBytes = size_t(16) << 20;  // nld_block_attn_static_scratch's partials, per device
 constexpr int kModeBlockMask = 2;  // block part of the mask from a per-row table
 constexpr int kMaxBalanced = 32;  // sequences of a launch with balanced pieces
 constexpr int kMaxRows = 256;   // (Hq / Hkv) * block_len handled by one CTA (two 128-row M tiles)

@@ -26,7 +26,7 @@
 
 namespace {
 
-constexpr size_t kStaticScratchBytes = size_t(16) << 20;  // 16 MiB per device
+using nld::kStaticScratchBytes;
 
 __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
 

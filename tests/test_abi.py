@@ -200,6 +200,28 @@ def test_plan_invariants(L, B, Hq, Hkv, D, P, L_, bl):
                 assert plan["splits"] <= S
 
 
+@pytest.mark.parametrize("B,Hkv,max_tokens", [(1, 8, 98304), (1, 8, 200000), (48, 1, 32768), (64, 1, 32768)])
+def test_plan_few_unbalanced_units_fill_their_waves(L, B, Hkv, max_tokens):
+    """Pieces the launch does not balance (one sequence, or more than 32) over
+    few units: cut as finely as 2048 tokens, or into four waves."""
+    plan, tokens = _plan(B, 4 * Hkv, Hkv, 128, 16, max_tokens - 16, 16)
+    units = B * Hkv
+    assert plan["splits"] * units >= min(4 * 152, -(-tokens // 2048) * units)
+    assert plan["splits"] * units < 4 * 152 + units
+
+
+def test_plan_partials_fit_the_static_scratch(L):
+    """The finer plans stay within the 16 MiB of nld_block_attn_static_scratch
+    wherever the two-wave plan does."""
+    for B, Hkv, G, bl in ((1, 8, 4, 32), (48, 1, 4, 32), (40, 1, 8, 16), (1, 1, 4, 32)):
+        for tokens in (65536, 131072, 262144):
+            plan, _ = _plan(B, G * Hkv, Hkv, 128, 16, tokens - bl, bl)
+            units, row_bytes = B * Hkv, G * bl * (128 * 2 + 4)
+            two_waves = min(128, -(-2 * 152 // units) + 1)
+            if two_waves * units * row_bytes + 256 <= 16 << 20:
+                assert plan["splits"] * units * row_bytes + 256 <= 16 << 20
+
+
 def test_plan_without_clusters(L):
     """NLD_ATTN_NO_CLUSTER: every piece of an explicit split count is a
     partial (pieces are whole 16-token groups, so 64 pieces of 32800 tokens
