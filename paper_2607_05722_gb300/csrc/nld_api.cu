@@ -101,10 +101,16 @@ constexpr long long kPairedChunk = 384;
 // all of those fit in one wave: the pair reads every tile twice, but a half's
 // chain is shorter (1.15 us per 128 tokens against 1.67 with two M tiles, Q by
 // TMA, half the rows to store). Automatic plans cut pieces for that up to this
-// length, and else twice as many for one CTA each: one sequence, 14B heads, 1000
-// / 4096 / 16384 tokens take 9.7 / 13.1 / 26.7 us as halves, 12.0 / 13.9 / 24.3
-// with two M tiles.
-constexpr long long kHalvesChunk = 512;
+// length, and else twice as many for one CTA each. Halves / two M tiles, us:
+// one sequence, 8 KV heads, 160 rows 6880 tokens 14.7 / 16.1, 18400 26.4 / 27.1,
+// 27616 35.7 / 34.9; 256 rows 18400 27.4 / 29.8, 36832 45.5 / 45.8; head_dim 64,
+// 2272 9.3 / 9.7, 4576 12.0 / 11.1. Several sequences of a range the longest
+// may not fill: the line lies lower (two of 2000..8000, 224 rows, 26.4 / 24.4;
+// two of 4064, 256 rows, 17.5 / 20.6).
+long long halves_chunk(const nld_attn_params_t* p, int rows) {
+  if (p->head_dim == 64) return 384;
+  return (p->batch == 1 ? 12ll : 6ll) * rows;
+}
 
 // Several sequences share a launch whose pieces the kernel may balance over
 // the SMs, knowing their lengths.
@@ -138,7 +144,8 @@ void plan_splits_for(const nld_attn_params_t* p, int block_len, int sms, Cluster
     // once. With more units than SMs the hardware scheduler balances them.
     const long long by_chunk = (max_tokens + kMaxAutoChunk - 1) / kMaxAutoChunk;
     long long s = sms / unsplit_units;
-    if (unsplit_units < sms) {  // a single wave: the longest range would set the time
+    const bool halves = wide_even && s > 1 && max_tokens <= s * halves_chunk(p, rows);
+    if (unsplit_units < sms && !halves) {  // a single wave: the longest range would set the time
       // at most one slot more than two waves of CTAs have (balanced pieces use
       // no more, and the combine reads every slot). Pieces that are not balanced
       // need more waves to even out while there are few units: 48 units of
@@ -156,7 +163,7 @@ void plan_splits_for(const nld_attn_params_t* p, int block_len, int sms, Cluster
       }
       if (s < by_chunk) s = by_chunk < by_waves ? by_chunk : by_waves;
       // More pieces where they run as one CTA each, not as block-slot halves.
-      if (s > 1 && s < sms / units && max_tokens > s * kHalvesChunk) s = sms / units;
+      if (s > 1 && s < sms / units) s = sms / units;
     }
     const long long by_tiles = (max_tokens + nld::kTileTok - 1) / nld::kTileTok;  // >= one tile per split
     if (s > by_tiles) s = by_tiles;

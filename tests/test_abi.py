@@ -210,6 +210,18 @@ def test_plan_few_unbalanced_units_fill_their_waves(L, B, Hkv, max_tokens):
     assert plan["splits"] * units < 4 * 152 + units
 
 
+@pytest.mark.parametrize("B,Hkv,D,rows,tokens,halves", [
+    (1, 8, 128, 160, 5000, True), (1, 8, 128, 256, 10000, True), (1, 4, 128, 160, 16000, True),
+    (1, 8, 128, 160, 30000, False), (2, 8, 128, 256, 4000, True), (2, 8, 128, 160, 8000, False),
+    (1, 8, 64, 256, 2200, True), (1, 8, 64, 256, 5000, False)])
+def test_plan_wide_pieces_as_halves(L, B, Hkv, D, rows, tokens, halves):
+    """129..256 rows: half as many pieces, each two CTAs of half the block
+    slots, up to a length that grows with the rows (measured on both sides)."""
+    bl = 32
+    plan, _ = _plan(B, rows // bl * Hkv, Hkv, D, 16, tokens - bl, bl)
+    assert (2 * B * Hkv * plan["splits"] <= 152) == halves
+
+
 def test_plan_partials_fit_the_static_scratch(L):
     """The finer plans stay within the 16 MiB of nld_block_attn_static_scratch
     wherever the two-wave plan does."""
