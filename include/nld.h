@@ -132,14 +132,37 @@ int nld_block_attn_kernels(const nld_attn_params_t *params, int block_len);
  * size, plan[3] partials per output row. An explicit params->num_splits
  * divisible by 8, 4 or 2 runs as clusters of that size (plan[2] = 8, 4 or
  * 2), exactly as nld_block_attn launches it. An automatic plan
- * (num_splits = 0) is given as if no cluster were resident: on a device
- * where the plan's 2..8 pieces per (sequence, KV head) fit as resident
- * clusters, the launched plan instead uses one cluster of 2 to 8 per
- * (sequence, KV head) and one partial, and nld_block_attn_num_splits
- * reports that. Returns 0, or -1 for invalid parameters. Touches no device;
- * for tests and capacity planning.
+ * (num_splits = 0) is given as if no cluster were resident; the launch may
+ * differ from it in four ways, which nld_block_attn_route tells:
+ *   - where the plan's 2..8 pieces per (sequence, KV head) fit as resident
+ *     clusters, it uses one cluster of 2 to 8 CTAs per (sequence, KV head) and
+ *     one partial;
+ *   - unsplit (sequence, KV head) units of 129..256 rows may run as cluster
+ *     pairs, each CTA with half of its own sequence;
+ *   - several sequences in more pieces than SMs are cut anew on the device,
+ *     where their lengths are: plan[0] is then the number of partials a row
+ *     has room for, and the tokens per piece differ by sequence;
+ *   - pieces of 129..256 rows may run as two CTAs of half the block slots.
+ * Returns 0, or -1 for invalid parameters. Touches no device; for tests and
+ * capacity planning.
  */
 int nld_block_attn_plan(const nld_attn_params_t *params, int block_len, int sm_count, int32_t plan[4]);
+
+/*
+ * What nld_block_attn (table_mask = 0) or nld_block_attn_masked (1) launches:
+ * route[0] pieces per (sequence, KV head), or the most it may have when they
+ * are balanced; [1] tokens per piece, or of the longest range's pieces; [2]
+ * cluster size; [3] partials per output row; [4] CTAs per piece (2: each half
+ * of the block slots); [5] how CTAs take the pieces: 0 by grid position, 1
+ * longest sequence first (cluster pairs: half of their own sequence each), 2
+ * balanced on the device; [6] CTAs of the launch; [7] tokens per K/V box.
+ * With `resident` NULL for the current device. Otherwise for sm_count SMs on
+ * which resident[c] clusters of c = 2..8 CTAs run at once, without touching a
+ * device. Returns 0, or -1 for invalid parameters or a failed device query;
+ * for tests and capacity planning.
+ */
+int nld_block_attn_route(const nld_attn_params_t *params, int block_len, int table_mask, int sm_count,
+                         const int32_t *resident, int32_t route[8]);
 
 /*
  * Workspace bytes nld_block_attn needs (0 when it runs unsplit). The

@@ -7,6 +7,10 @@ namespace nld {
 
 bool tc_supports(int R, int head_dim) { return R <= 256 && (head_dim == 64 || head_dim == 128); }
 
+bool tc_row_copies(int R, int head_dim, int chunk) {
+  return tc_replication(R) == 2 && (head_dim == 128 ? ring_holds<128>(chunk) : ring_holds<64>(chunk));
+}
+
 int tc_max_active_clusters(int csize, int head_dim, int rows) {
   return head_dim == 128 ? max_active_clusters_d<128>(csize, rows) : max_active_clusters_d<64>(csize, rows);
 }

@@ -1642,6 +1642,10 @@ int max_active_clusters_t(int csize) {
 // packed rows, else one.
 int tc_replication(int rows) { return rows > 32 && rows <= 64 ? 2 : 1; }
 
+// A split of `chunk` tokens sits whole in the ring of the one-M-tile kernels.
+template <int D>
+bool ring_holds(int chunk) { return chunk <= TcLayout<D, 1, 2>::kKStages * kTileTok; }
+
 template <int D>
 int max_active_clusters_d(int csize, int rows) {
   if (rows > 128) return max_active_clusters_t<D, 2, 1, 2, 1>(csize);
@@ -1675,7 +1679,7 @@ cudaError_t launch_tc_d(const AttnArgs& a, const TmaMaps& maps, cudaStream_t str
     return launch_tc_o<D, 1, 1, 2, MASKED, kGridOrder, 2>(a, maps, stream);
   }
   if (a.R > 128) return launch_tc_t<D, 2, 1, 2, MASKED>(a, maps, stream);
-  if (a.chunk <= TcLayout<D, 1, 2>::kKStages * kTileTok) return launch_tc_rep<D, true, MASKED>(a, maps, stream);
+  if (ring_holds<D>(a.chunk)) return launch_tc_rep<D, true, MASKED>(a, maps, stream);
   return launch_tc_rep<D, false, MASKED>(a, maps, stream);
 }
 

@@ -240,6 +240,52 @@ nld_status_t plan_splits(const nld_attn_params_t* p, int block_len, SplitPlan* o
   return NLD_OK;
 }
 
+// What a call launches: its plan, and how the CTAs take the pieces.
+struct Route {
+  SplitPlan plan;
+  int nh;             // CTAs per piece (2: block-slot halves)
+  bool longest_first; // CTAs take the sequences by length; cluster pairs each half of their own
+  int balanced_ctas;  // > 0: pieces balanced on the device over that many CTAs
+};
+
+Route route_for(const nld_attn_params_t* p, int block_len, bool table_mask, int sms, const SplitPlan& plan) {
+  const int rows = (p->num_q_heads / p->num_kv_heads) * block_len;
+  const long long units = static_cast<long long>(p->batch) * p->num_kv_heads;
+  const long long max_tokens = static_cast<long long>(p->max_pages_per_seq) * p->page_size;
+  const long long ctas = units * plan.splits;
+  const bool automatic = p->num_splits == 0;
+  Route r;
+  r.plan = plan;
+  r.nh = rows > 128 && block_len % 2 == 0 && plan.csize == 1 && 2 * ctas <= sms ? 2 : 1;
+  // Longest sequences first when one split each leaves several waves: the last
+  // wave then holds the short sequences. With a table mask only ranges above
+  // 2048 tokens, since the ranking takes about 1 us of a CTA's start (31
+  // sequences of 277..555 tokens: 31.4 us ordered, 30.8 in grid order). And
+  // where the plan made cluster pairs of unsplit units of 129..256 rows, whose
+  // CTAs take half of their own sequence each. Pairs of fewer rows come from a
+  // plan of two pieces, which fills one wave and keeps its pieces (76 units of
+  // 1024 tokens, 32 rows, 12.8 us, as own halves 14.0).
+  const bool waves = plan.splits == 1 && units > sms && (!table_mask || max_tokens > kMaxAutoChunk);
+  const bool pairs = automatic && rows > 128 && plan.csize == 2 && plan.splits == 2 && 2 * units >= sms;
+  r.longest_first = (waves || pairs) && p->batch > 1 && p->batch <= 1024;
+  // Balanced pieces: a plan of several streaming pieces a sequence, none of
+  // them in clusters, more slots than SMs. The launch has CTAs for two waves,
+  // or one per slot. Measured against the plan's own pieces (8B heads, 32 rows):
+  // 8 sequences of 512..8192 tokens 43.4 -> 38.6 us, 8 of 4096 39.8 -> 32.4, 18
+  // of 8192 115 -> 103; 14B heads, 4 of 4096..16384 77 -> 59. A CTA learns its
+  // piece about 2 us later, so a single wave keeps the plan's pieces, and so
+  // does a plan of at most three that fill their last wave to 90% (12 of 4096:
+  // 46.5 us against 50.5).
+  r.balanced_ctas = 0;
+  if (can_balance(p) && plan.csize == 1 && plan.splits > 1 && plan.chunk > kPairedChunk &&
+      !nld::tc_row_copies(rows, p->head_dim, plan.chunk)) {
+    const long long in_waves = (ctas + sms - 1) / sms;
+    if (ctas > sms && units <= 2 * sms && !(plan.splits <= 3 && 10 * ctas >= 9 * in_waves * sms))
+      r.balanced_ctas = static_cast<int>(ctas < 2 * sms ? ctas : 2 * sms);
+  }
+  return r;
+}
+
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 size_t partial_o_bytes(const nld_attn_params_t* p, int block_len, int splits) {
@@ -438,6 +484,29 @@ int nld_block_attn_plan(const nld_attn_params_t* params, int block_len, int sm_c
   return 0;
 }
 
+int nld_block_attn_route(const nld_attn_params_t* params, int block_len, int table_mask, int sm_count,
+                         const int32_t* resident, int32_t route[8]) {
+  if (route == nullptr || (resident != nullptr && sm_count < 1)) return -1;
+  if (check_params(params, block_len) != NLD_OK) return -1;
+  SplitPlan plan;
+  if (resident != nullptr) {
+    plan_splits_for(params, block_len, sm_count, [&](int cs) { return static_cast<long long>(resident[cs]); }, &plan);
+  } else if (plan_splits(params, block_len, &plan) != NLD_OK || device_state(nullptr, &sm_count) != NLD_OK) {
+    return -1;
+  }
+  const Route r = route_for(params, block_len, table_mask != 0, sm_count, plan);
+  const long long ctas = static_cast<long long>(plan.splits) * params->batch * params->num_kv_heads * r.nh;
+  route[0] = plan.splits;
+  route[1] = plan.chunk;
+  route[2] = plan.csize;
+  route[3] = plan.partials;
+  route[4] = r.nh;
+  route[5] = r.balanced_ctas > 0 ? 2 : r.longest_first ? 1 : 0;
+  route[6] = r.balanced_ctas > 0 ? r.balanced_ctas : ctas > INT_MAX ? INT_MAX : static_cast<int32_t>(ctas);
+  route[7] = box_tokens(params, plan);
+  return 0;
+}
+
 int nld_block_attn_num_splits(const nld_attn_params_t* params, int block_len) {
   if (check_params(params, block_len) != NLD_OK) return -1;
   SplitPlan plan;
@@ -490,8 +559,10 @@ nld_status_t block_attn_impl(const nld_attn_params_t* params, const void* q_bloc
   }
   unsigned int* err = nullptr;
   unsigned long long* rescales = nullptr;
-  st = device_state(&err, nullptr, &rescales);
+  int sms = 0;
+  st = device_state(&err, &sms, &rescales);
   if (st != NLD_OK) return st;
+  const Route route = route_for(params, block_len, mode == nld::kModeBlockMask, sms, plan);
 
   nld::TmaMaps maps;
   const int box_tok = box_tokens(params, plan);
@@ -517,13 +588,7 @@ nld_status_t block_attn_impl(const nld_attn_params_t* params, const void* q_bloc
   a.Hkv = params->num_kv_heads;
   a.G = G;
   a.bl = block_len;
-  {
-    int sms = 0;
-    if ((st = device_state(nullptr, &sms)) != NLD_OK) return st;
-    const bool halves = G * block_len > 128 && block_len % 2 == 0 && plan.csize == 1 &&
-                        2ll * a.B * a.Hkv * plan.splits <= sms;
-    a.nh = halves ? 2 : 1;
-  }
+  a.nh = route.nh;
   a.bl_c = block_len / a.nh;
   a.R = G * a.bl_c;
   a.page_size = params->page_size;
@@ -539,42 +604,9 @@ nld_status_t block_attn_impl(const nld_attn_params_t* params, const void* q_bloc
   a.block_mask = mode == nld::kModeBlockMask ? block_mask : nullptr;
   a.scale_log2 = scale * nld::kLog2e;
   a.prefix_ready = (params->flags & NLD_ATTN_PREFIX_READY) ? 1 : 0;
-  {
-    // Longest sequences first when one split (or one cluster pair, whose CTAs
-    // take half of their own sequence) each leaves several waves: the last
-    // wave then holds the short sequences. With a table mask only ranges above
-    // 2048 tokens, since the ranking takes about 1 us of a CTA's start (31
-    // sequences of 277..555 tokens: 31.4 us ordered, 30.8 in grid order).
-    const bool long_enough = mode != nld::kModeBlockMask ||
-                             static_cast<long long>(params->max_pages_per_seq) * params->page_size > kMaxAutoChunk;
-    int sms = 0;
-    if ((st = device_state(nullptr, &sms)) != NLD_OK) return st;
-    const bool halves = params->num_splits == 0 && plan.csize == 2 && plan.splits == 2 &&
-                        static_cast<long long>(a.B) * a.Hkv * 2 >= sms;
-    a.order_by_length = (((plan.splits == 1 && static_cast<long long>(a.B) * a.Hkv > sms) || halves) && a.B > 1 &&
-                         a.B <= 1024 && long_enough)
-                            ? 1
-                            : 0;
-  }
-  // Balanced pieces: a plan of several streaming pieces a sequence, none of
-  // them in clusters, more slots than SMs. The launch has CTAs for two waves,
-  // or one per slot. Measured against the plan's own pieces (8B heads, 32 rows):
-  // 8 sequences of 512..8192 tokens 43.4 -> 38.6 us, 8 of 4096 39.8 -> 32.4, 18
-  // of 8192 115 -> 103; 14B heads, 4 of 4096..16384 77 -> 59. A CTA learns its
-  // piece about 2 us later, so a single wave keeps the plan's pieces, and so
-  // does a plan of at most three that fill their last wave to 90% (12 of 4096:
-  // 46.5 us against 50.5).
-  if (can_balance(params) && plan.csize == 1 && plan.splits > 1 && plan.chunk > kPairedChunk) {
-    int sms = 0;
-    if ((st = device_state(nullptr, &sms)) != NLD_OK) return st;
-    const long long units = static_cast<long long>(a.B) * a.Hkv;
-    const long long ctas = units * plan.splits;
-    const long long waves = (ctas + sms - 1) / sms;
-    if (ctas > sms && units <= 2 * sms && !(plan.splits <= 3 && 10 * ctas >= 9 * waves * sms)) {
-      a.sms = sms;
-      a.balanced_ctas = static_cast<int>(ctas < 2 * sms ? ctas : 2 * sms);
-    }
-  }
+  a.order_by_length = route.longest_first ? 1 : 0;
+  a.balanced_ctas = route.balanced_ctas;
+  a.sms = sms;
   if (plan.partials > 1) {
     a.o_part = static_cast<__nv_bfloat16*>(workspace);
     a.lse_part = reinterpret_cast<float*>(static_cast<char*>(workspace) + o_bytes);
@@ -583,8 +615,6 @@ nld_status_t block_attn_impl(const nld_attn_params_t* params, const void* q_bloc
   if ((st = encode_block_map(&maps.q, q_block, a, params->head_dim)) != NLD_OK) return st;
   if (nld::launch_block_attn_tc(a, maps, params->head_dim, stream) != cudaSuccess) return NLD_ERR_CUDA;
   if (plan.partials > 1 && run_combine) {
-    int sms = 0;
-    if ((st = device_state(nullptr, &sms)) != NLD_OK) return st;
     if (nld::launch_combine(a.o_part, a.lse_part, plan.partials, a.B, a.Hq, block_len, params->head_dim, a.out, lse,
                             sms, stream) != cudaSuccess)
       return NLD_ERR_CUDA;

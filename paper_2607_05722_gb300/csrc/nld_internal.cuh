@@ -54,6 +54,9 @@ struct AttnArgs {
 // Launchers (defined next to their kernels). Return a CUDA error code.
 // tcgen05 kernel: query rows R <= 256 (one or two 128-row MMA tiles).
 bool tc_supports(int R, int head_dim);
+// Whether pieces of `chunk` tokens run on the kernel with row copies (which
+// takes no balanced pieces).
+bool tc_row_copies(int R, int head_dim, int chunk);
 // Tensor maps of one call: k/v the K/V page pools; q the query block and o
 // the output or, with split partials, the partial rows (bf16 both), in
 // boxes of one CTA's rows.

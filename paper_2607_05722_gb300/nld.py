@@ -99,6 +99,8 @@ def lib(path: Optional[str] = None):
     L.nld_block_attn_kernels.restype = I
     L.nld_block_attn_plan.argtypes = [PP, I, I, ctypes.POINTER(ctypes.c_int32)]
     L.nld_block_attn_plan.restype = I
+    L.nld_block_attn_route.argtypes = [PP, I, I, I, V, V]
+    L.nld_block_attn_route.restype = I
     if path is None:
         _lib = L
     return L
@@ -401,6 +403,18 @@ def nld_block_attn_plan(params: AttnParams, block_len: int, sm_count: int) -> di
     if lib().nld_block_attn_plan(ctypes.byref(params), block_len, sm_count, out) != 0:
         raise NldError(1, "nld_block_attn_plan")
     return {"splits": out[0], "chunk": out[1], "cluster": out[2], "partials": out[3]}
+
+
+def nld_block_attn_route(params: AttnParams, block_len: int, table_mask: bool = False, sm_count: int = 0,
+                         resident=None) -> dict:
+    """What a call launches on the current device, or, given resident[c] (clusters
+    of c = 2..8 CTAs that run at once on sm_count SMs), on one like it, host only."""
+    out = (ctypes.c_int32 * 8)()
+    res = None if resident is None else (ctypes.c_int32 * 9)(*resident)
+    if lib().nld_block_attn_route(ctypes.byref(params), block_len, int(table_mask), sm_count, res, out) != 0:
+        raise NldError(1, "nld_block_attn_route")
+    keys = ("pieces", "chunk", "cluster", "partials", "halves", "order", "ctas", "box")
+    return dict(zip(keys, out))
 
 
 def nld_check_wait_timeout(limit_ns: int, stream=None) -> None:

@@ -222,6 +222,45 @@ def test_plan_wide_pieces_as_halves(L, B, Hkv, D, rows, tokens, halves):
     assert (2 * B * Hkv * plan["splits"] <= 152) == halves
 
 
+# clusters of 2..8 CTAs that run at once on 152 SMs
+RESIDENT = [0, 0, 76, 48, 36, 28, 24, 20, 18]
+
+
+def _route(B, Hq, Hkv, D, P, prefix_max, bl, splits=0, flags=0, mask=False, resident=RESIDENT):
+    pages = (prefix_max + bl + P - 1) // P
+    p = nld.make_params(B, Hq, Hkv, D, P, B * pages, pages, splits, 0.0, flags)
+    return nld.nld_block_attn_route(p, bl, mask, 152, resident)
+
+
+@pytest.mark.parametrize("G,bl", [(4, 8), (4, 16), (4, 32)])
+def test_route_pairs_of_one_wave_keep_the_plan(L, G, bl):
+    """76 units in pairs fill one wave: up to 128 rows they take the plan's two
+    pieces in grid order, with more rows half of their own sequence each."""
+    r = _route(19, 4 * G, 4, 128, 16, 4000, bl)
+    assert (r["pieces"], r["cluster"], r["partials"], r["order"], r["ctas"]) == (2, 2, 1, 0, 152)
+    assert _route(19, 20, 4, 128, 16, 8192, 32)["order"] == 1
+
+
+@pytest.mark.parametrize("B,Hkv,G,bl,prefix", [(1, 8, 4, 16, 4096), (8, 8, 4, 8, 8192), (3, 8, 4, 16, 4000),
+                                              (16, 8, 5, 32, 16384), (24, 8, 4, 16, 4096), (2, 8, 8, 32, 3000)])
+@pytest.mark.parametrize("D", [64, 128])
+def test_route_invariants(L, B, Hkv, G, bl, prefix, D):
+    """A route uses one way to take its pieces, and clusters only where they
+    are resident; without resident clusters it is the plan."""
+    for flags in (0, nld.NLD_ATTN_NO_CLUSTER):
+        for resident in (RESIDENT, [0] * 9):
+            for splits in (0, 2, 3):
+                r = _route(B, G * Hkv, Hkv, D, 16, prefix, bl, splits, flags, resident=resident)
+                assert r["pieces"] == r["cluster"] * r["partials"] and r["box"] == 16
+                assert r["halves"] == 1 or (r["order"] == 0 and r["cluster"] == 1)
+                assert r["order"] != 2 or (r["cluster"] == 1 and 152 < r["ctas"] <= 304)
+                if splits == 0 and r["cluster"] > 1:
+                    assert B * Hkv <= resident[r["cluster"]] or r["order"] == 1
+                if splits == 0 and not any(resident):
+                    plan, _ = _plan(B, G * Hkv, Hkv, D, 16, prefix, bl)
+                    assert (r["pieces"], r["chunk"], r["cluster"]) == (plan["splits"], plan["chunk"], plan["cluster"])
+
+
 def test_plan_partials_fit_the_static_scratch(L):
     """The finer plans stay within the 16 MiB of nld_block_attn_static_scratch
     wherever the two-wave plan does."""
