@@ -142,7 +142,8 @@ int nld_block_attn_kernels(const nld_attn_params_t *params, int block_len);
  *   - several sequences in more pieces than SMs are cut anew on the device,
  *     where their lengths are: plan[0] is then the number of partials a row
  *     has room for, and the tokens per piece differ by sequence;
- *   - pieces of 129..256 rows may run as two CTAs of half the block slots.
+ *   - pieces of 129..256 rows may run as two CTAs of half the block slots,
+ *     of unsplit sequences only the longer ones.
  * Returns 0, or -1 for invalid parameters. Touches no device; for tests and
  * capacity planning.
  */
@@ -155,7 +156,8 @@ int nld_block_attn_plan(const nld_attn_params_t *params, int block_len, int sm_c
  * cluster size; [3] partials per output row; [4] CTAs per piece (2: each half
  * of the block slots); [5] how CTAs take the pieces: 0 by grid position, 1
  * longest sequence first (cluster pairs: half of their own sequence each), 2
- * balanced on the device; [6] CTAs of the launch; [7] tokens per K/V box.
+ * balanced on the device, 3 the longest sequences as block-slot halves and the
+ * others whole; [6] CTAs of the launch; [7] tokens per K/V box.
  * With `resident` NULL for the current device. Otherwise for sm_count SMs on
  * which resident[c] clusters of c = 2..8 CTAs run at once, without touching a
  * device. Returns 0, or -1 for invalid parameters or a failed device query;

@@ -20,4 +20,11 @@ cudaError_t launch_block_attn_tc(const AttnArgs& a, const TmaMaps& maps, int hea
   return head_dim == 128 ? launch_tc_d<128, false>(a, maps, stream) : launch_tc_d<64, false>(a, maps, stream);
 }
 
+cudaError_t launch_block_attn_tc_mixed(const AttnArgs& a, const TmaMaps& maps, const AttnArgs& half,
+                                       const TmaMaps& half_maps, int head_dim, cudaStream_t stream) {
+  if (a.mode == kModeBlockMask) return launch_block_attn_tc_mixed_masked(a, maps, half, half_maps, head_dim, stream);
+  return head_dim == 128 ? launch_tc_mixed<128, false>(a, maps, half, half_maps, stream)
+                         : launch_tc_mixed<64, false>(a, maps, half, half_maps, stream);
+}
+
 }  // namespace nld

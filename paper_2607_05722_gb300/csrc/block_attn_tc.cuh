@@ -164,10 +164,9 @@ struct TcLayout {
   static_assert(D / 64 * kMergeRows * 128 <= kPOff, "output staging");
 };
 
-// The sequence of rank blockIdx.z by prefix length (descending, ties by
-// index), computed by the whole CTA in `scratch` (2 * B ints of shared
+// The sequence of a rank by prefix length (descending, ties by index), computed by the whole CTA in `scratch` (2 * B ints of shared
 // memory). Out of line, so that kernels that never take it keep their code.
-__device__ __noinline__ int sequence_by_length_rank(const AttnArgs& a, int* scratch) {
+__device__ __noinline__ int sequence_by_length_rank(const AttnArgs& a, int* scratch, int wanted) {
   int* lens = scratch;
   int* order = scratch + a.B;
   for (int t = threadIdx.x; t < a.B; t += blockDim.x) lens[t] = __ldg(a.prefix_lens + t);
@@ -182,12 +181,13 @@ __device__ __noinline__ int sequence_by_length_rank(const AttnArgs& a, int* scra
     order[rank] = t;
   }
   __syncthreads();
-  return order[blockIdx.z];
+  return order[wanted];
 }
 
 // Which (split, KV head, sequence) a CTA takes: its grid position, with the
 // sequences in grid order or longest first, or a piece of balanced_piece().
-constexpr int kGridOrder = 0, kLongestFirst = 1, kBalanced = 2;
+// kPicked: the kernel has picked it before.
+constexpr int kGridOrder = 0, kLongestFirst = 1, kBalanced = 2, kPicked = 3;
 
 // Pieces of one launch over sequences of different lengths, chosen on the
 // device, where the lengths are. Sequence b is cut into n_b equal pieces of at
@@ -261,8 +261,7 @@ __device__ __noinline__ void balanced_piece(const AttnArgs& a, Piece* out) {
 }
 
 template <int D, int MT, int REP, int TPS, bool MASKED, int ORDER, int CG>
-__global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
-    block_attn_tc_kernel(const __grid_constant__ TmaMaps maps, const AttnArgs a) {
+__device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const AttnArgs& a, Piece piece) {
   static_assert(REP == 1 || REP == 2, "replication of 1 or 2 (up to 32 rows run on two softmax groups)");
   static_assert(MT == 1 || REP == 1, "replication only with one M tile");
   static_assert(CG == 1 || REP == 1, "softmax groups without row copies");
@@ -312,7 +311,6 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
   // With NLD_ATTN_PREFIX_READY the prefix lengths, the page table and
   // prefix-only K/V tiles are read before the dependency wait.
   const bool early = a.prefix_ready != 0;
-  Piece piece = {static_cast<int>(blockIdx.z), static_cast<int>(blockIdx.y), static_cast<int>(blockIdx.x), a.chunk, 0};
   Piece* picked = reinterpret_cast<Piece*>(reinterpret_cast<uint8_t*>(bars) + Lay::kPieceOff);
   if constexpr (ORDER == kBalanced) {
     grid_launch_dependents();
@@ -377,14 +375,14 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
   // Block-slot halves (a.nh = 2: short pieces of 129..256 packed rows): the two
   // CTAs of a (split, KV head, sequence) are adjacent along x and hold block
   // slots [hc*bl_c, (hc+1)*bl_c) of the G heads each, R = G*bl_c rows.
-  constexpr bool kHalves = CG == 2 && ORDER == kGridOrder;
+  constexpr bool kHalves = CG == 2 && (ORDER == kGridOrder || ORDER == kPicked);
   const int split = kHalves ? piece.split >> (a.nh - 1) : piece.split, g = piece.g;
   const int slot0 = kHalves ? (piece.split & (a.nh - 1)) * a.bl_c : 0;  // first block slot of this CTA
   // Without NLD_ATTN_PREFIX_READY nothing global is read before the
   // dependency wait. With it, the page table, the prefix lengths and
   // prefix-only K/V tiles are read first, and only the block slots, Q and the
   // outputs wait (producers: in produce_kv; softmax warps: before Q).
-  if constexpr (ORDER != kBalanced) {
+  if constexpr (ORDER == kGridOrder || ORDER == kLongestFirst) {
     grid_launch_dependents();  // dependents launch early; they wait on this grid themselves
     if (!early) grid_dependency_wait();
   }
@@ -395,7 +393,7 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
   // instantiation, so the other kernels keep b = blockIdx.z.
   // Two CTAs of a cluster take half of their sequence each.
   if constexpr (ORDER == kLongestFirst) {
-    piece.b = sequence_by_length_rank(a, reinterpret_cast<int*>(smem));
+    piece.b = sequence_by_length_rank(a, reinterpret_cast<int*>(smem), piece.b);
     if (a.num_splits == 2) {
       const int tokens = min(max(reinterpret_cast<const int*>(smem)[piece.b], 0), a.max_pages * a.page_size - a.bl) + a.bl;
       piece.chunk = ((tokens + 1) / 2 + kTileTok - 1) & ~(kTileTok - 1);
@@ -1567,6 +1565,71 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
     tc_fence_after();
     tmem_dealloc(tmem, Cfg::kTmemCols);
   }
+}
+
+template <int D, int MT, int REP, int TPS, bool MASKED, int ORDER, int CG>
+__global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
+    block_attn_tc_kernel(const __grid_constant__ TmaMaps maps, const AttnArgs a) {
+  block_attn_tc_body<D, MT, REP, TPS, MASKED, ORDER, CG>(
+      maps, a,
+      {static_cast<int>(blockIdx.z), static_cast<int>(blockIdx.y), static_cast<int>(blockIdx.x), a.chunk, 0});
+}
+
+// Unsplit sequences of 129..256 rows, an even block length, more than half as
+// many (sequence, KV head) units as SMs but fewer than SMs: one wave in which
+// the a.halved longest sequences run as block-slot halves in two CTAs
+// (half_maps, half: as for a.nh = 2), as many as SMs are left for, and the
+// others whole, with two M tiles. Blocks: y < B takes the sequence of rank y,
+// whole or its first half, y >= B the second half of rank y - B. A half ends
+// sooner (5.5 us and 1.15 us per 128 tokens against 9.4 and 1.72), so the
+// longest sequence no longer sets the time alone. us, all whole / mixed: 160
+// rows, 8 KV heads, 10 sequences of 512..1900 tokens 32.3 / 23.1, 14 of 100..2000
+// 34.2 / 31.5, 10 of 1900 35.3 / 37.5 (the ranking); in cluster pairs of half
+// sequences / mixed: 12 of 512..4096 51.0 / 42.1, 14 of 3000 69.6 / 51.3.
+template <int D, bool MASKED>
+__global__ void __launch_bounds__(TcCfg<2, 2>::kThreads, 1)
+    block_attn_tc_mixed_kernel(const __grid_constant__ TmaMaps maps, const AttnArgs a,
+                               const __grid_constant__ TmaMaps half_maps, const AttnArgs half) {
+  static_assert(TcCfg<2, 2>::kThreads == TcCfg<1, 2, 2>::kThreads, "one block shape for both");
+  extern __shared__ uint8_t smem_raw[];
+  grid_launch_dependents();
+  if (a.prefix_ready == 0) grid_dependency_wait();
+  // The scratch lies where the K/V rings will, as with kLongestFirst.
+  int* scratch = reinterpret_cast<int*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int y = static_cast<int>(blockIdx.y);
+  const int second = y >= a.B ? 1 : 0, rank = second ? y - a.B : y;
+  const Piece piece = {sequence_by_length_rank(a, scratch, rank), static_cast<int>(blockIdx.x), second, a.chunk, 0};
+  // Halves read every tile twice; they pay where they take an eighth off the
+  // longest whole sequence.
+  const int* order = scratch + a.B;
+  const int rest = a.halved < a.B ? scratch[order[a.halved]] : 0;
+  const bool halves = rest < scratch[order[0]] - scratch[order[0]] / 8;
+  if (second && !halves) return;
+  if (halves && rank < a.halved)
+    block_attn_tc_body<D, 1, 1, 2, MASKED, kPicked, 2>(half_maps, half, piece);
+  else
+    block_attn_tc_body<D, 2, 1, 2, MASKED, kPicked, 1>(maps, a, piece);
+}
+
+template <int D, bool MASKED>
+cudaError_t launch_tc_mixed(const AttnArgs& a, const TmaMaps& maps, const AttnArgs& half, const TmaMaps& half_maps,
+                            cudaStream_t stream) {
+  constexpr int kBytes =
+      (TcLayout<D, 2, 2>::kBytes > TcLayout<D, 1, 2>::kBytes ? TcLayout<D, 2, 2>::kBytes : TcLayout<D, 1, 2>::kBytes) + 1024;
+  static int configured[64] = {0};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (!__atomic_load_n(&configured[dev], __ATOMIC_ACQUIRE)) {
+    e = cudaFuncSetAttribute(block_attn_tc_mixed_kernel<D, MASKED>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
+    if (e != cudaSuccess) return e;
+    __atomic_store_n(&configured[dev], 1, __ATOMIC_RELEASE);
+  }
+  if (a.R <= 128 || a.R > 256 || a.num_splits != 1 || half.nh != 2 || half.R <= 64 || half.R > 128 || a.B > 1024 || a.halved > a.B)
+    return cudaErrorInvalidValue;
+  return launch_kernel(block_attn_tc_mixed_kernel<D, MASKED>, dim3(a.Hkv, a.B + a.halved), dim3(TcCfg<2, 2>::kThreads), kBytes,
+                       stream, maps, a, half_maps, half);
 }
 
 template <int D, int MT, int REP, int TPS, bool MASKED, int ORDER, int CG>

@@ -10,4 +10,10 @@ cudaError_t launch_block_attn_tc_masked(const AttnArgs& a, const TmaMaps& maps, 
   return head_dim == 128 ? launch_tc_d<128, true>(a, maps, stream) : launch_tc_d<64, true>(a, maps, stream);
 }
 
+cudaError_t launch_block_attn_tc_mixed_masked(const AttnArgs& a, const TmaMaps& maps, const AttnArgs& half,
+                                              const TmaMaps& half_maps, int head_dim, cudaStream_t stream) {
+  return head_dim == 128 ? launch_tc_mixed<128, true>(a, maps, half, half_maps, stream)
+                         : launch_tc_mixed<64, true>(a, maps, half, half_maps, stream);
+}
+
 }  // namespace nld

@@ -112,6 +112,14 @@ long long halves_chunk(const nld_attn_params_t* p, int rows) {
   return (p->batch == 1 ? 12ll : 6ll) * rows;
 }
 
+// Unsplit units of 129..256 rows, fewer than SMs, take cluster pairs of half
+// sequences above this many tokens (10 sequences of 100..9000 tokens 71 us, whole
+// or as halves 86; head_dim 64, 16 of 512..4096 48, 54), below that whole
+// sequences and block-slot halves mixed, and whole sequences alone below
+// kMixedMinTokens (the ranking is 1 us).
+long long pair_tokens(const nld_attn_params_t* p) { return p->head_dim == 64 ? 2048 : 4352; }
+constexpr long long kMixedMinTokens = 512;
+
 // Several sequences share a launch whose pieces the kernel may balance over
 // the SMs, knowing their lengths.
 bool can_balance(const nld_attn_params_t* p) {
@@ -193,7 +201,7 @@ void plan_splits_for(const nld_attn_params_t* p, int block_len, int sms, Cluster
     // up to 128 rows, whole sequences measured faster (24 sequences of 64 rows,
     // 192 units: 60 us against 64; 32 of 32 rows, 256 units: 96 against 111).
     if (want == 1 && rows > 128 && units < sms && unsplit_units >= sms && p->batch > 1 && p->batch <= 1024 &&
-        max_tokens > kMaxAutoChunk && !(p->flags & NLD_ATTN_NO_CLUSTER) && 2 * clusters_resident(2) >= sms - 1) {
+        max_tokens > pair_tokens(p) && !(p->flags & NLD_ATTN_NO_CLUSTER) && 2 * clusters_resident(2) >= sms - 1) {
       want = 2;
       csize = 2;
     }
@@ -244,6 +252,7 @@ nld_status_t plan_splits(const nld_attn_params_t* p, int block_len, SplitPlan* o
 struct Route {
   SplitPlan plan;
   int nh;             // CTAs per piece (2: block-slot halves)
+  int halved;         // > 0: unsplit sequences, that many as block-slot halves, the longest
   bool longest_first; // CTAs take the sequences by length; cluster pairs each half of their own
   int balanced_ctas;  // > 0: pieces balanced on the device over that many CTAs
 };
@@ -265,6 +274,14 @@ Route route_for(const nld_attn_params_t* p, int block_len, bool table_mask, int 
   // CTAs take half of their own sequence each. Pairs of fewer rows come from a
   // plan of two pieces, which fills one wave and keeps its pieces (76 units of
   // 1024 tokens, 32 rows, 12.8 us, as own halves 14.0).
+  // Whole sequences and block-slot halves mixed in one wave, where the longest
+  // sequence sets the time and there are SMs left for the halves of a fifth of
+  // them (18 sequences of 100..2000 tokens, one of which could be: 34.5 us all
+  // whole, 37.0).
+  const long long spare = (sms - units) / p->num_kv_heads;  // sequences that can run as halves
+  const bool mixed = plan.splits == 1 && rows > 128 && block_len % 2 == 0 && r.nh == 1 && 5 * spare >= p->batch && p->batch > 1 &&
+                     p->batch <= 1024 && max_tokens >= kMixedMinTokens;
+  r.halved = !mixed ? 0 : spare < p->batch ? static_cast<int>(spare) : p->batch;
   const bool waves = plan.splits == 1 && units > sms && (!table_mask || max_tokens > kMaxAutoChunk);
   const bool pairs = automatic && rows > 128 && plan.csize == 2 && plan.splits == 2 && 2 * units >= sms;
   r.longest_first = (waves || pairs) && p->batch > 1 && p->batch <= 1024;
@@ -495,13 +512,13 @@ int nld_block_attn_route(const nld_attn_params_t* params, int block_len, int tab
     return -1;
   }
   const Route r = route_for(params, block_len, table_mask != 0, sm_count, plan);
-  const long long ctas = static_cast<long long>(plan.splits) * params->batch * params->num_kv_heads * r.nh;
+  const long long ctas = (static_cast<long long>(plan.splits) * params->batch * r.nh + r.halved) * params->num_kv_heads;
   route[0] = plan.splits;
   route[1] = plan.chunk;
   route[2] = plan.csize;
   route[3] = plan.partials;
   route[4] = r.nh;
-  route[5] = r.balanced_ctas > 0 ? 2 : r.longest_first ? 1 : 0;
+  route[5] = r.halved > 0 ? 3 : r.balanced_ctas > 0 ? 2 : r.longest_first ? 1 : 0;
   route[6] = r.balanced_ctas > 0 ? r.balanced_ctas : ctas > INT_MAX ? INT_MAX : static_cast<int32_t>(ctas);
   route[7] = box_tokens(params, plan);
   return 0;
@@ -606,6 +623,7 @@ nld_status_t block_attn_impl(const nld_attn_params_t* params, const void* q_bloc
   a.prefix_ready = (params->flags & NLD_ATTN_PREFIX_READY) ? 1 : 0;
   a.order_by_length = route.longest_first ? 1 : 0;
   a.balanced_ctas = route.balanced_ctas;
+  a.halved = route.halved;
   a.sms = sms;
   if (plan.partials > 1) {
     a.o_part = static_cast<__nv_bfloat16*>(workspace);
@@ -613,7 +631,19 @@ nld_status_t block_attn_impl(const nld_attn_params_t* params, const void* q_bloc
   }
   if ((st = encode_out_map(&maps.o, a, params->head_dim)) != NLD_OK) return st;
   if ((st = encode_block_map(&maps.q, q_block, a, params->head_dim)) != NLD_OK) return st;
-  if (nld::launch_block_attn_tc(a, maps, params->head_dim, stream) != cudaSuccess) return NLD_ERR_CUDA;
+  if (route.halved > 0) {
+    AttnArgs half = a;
+    half.nh = 2;
+    half.bl_c = block_len / 2;
+    half.R = G * half.bl_c;
+    nld::TmaMaps half_maps = maps;
+    if ((st = encode_out_map(&half_maps.o, half, params->head_dim)) != NLD_OK) return st;
+    if ((st = encode_block_map(&half_maps.q, q_block, half, params->head_dim)) != NLD_OK) return st;
+    if (nld::launch_block_attn_tc_mixed(a, maps, half, half_maps, params->head_dim, stream) != cudaSuccess)
+      return NLD_ERR_CUDA;
+  } else if (nld::launch_block_attn_tc(a, maps, params->head_dim, stream) != cudaSuccess) {
+    return NLD_ERR_CUDA;
+  }
   if (plan.partials > 1 && run_combine) {
     if (nld::launch_combine(a.o_part, a.lse_part, plan.partials, a.B, a.Hq, block_len, params->head_dim, a.out, lse,
                             sms, stream) != cudaSuccess)

@@ -45,6 +45,7 @@ struct AttnArgs {
   float scale_log2;            // softmax scale * log2(e)
   int prefix_ready;            // NLD_ATTN_PREFIX_READY: prefix K/V may be read before the dependency wait
   int order_by_length;         // CTA z takes the sequence of rank z by prefix length (longest first)
+  int halved;                  // > 0: sequences that run as block-slot halves, the longest (mixed launch)
   int balanced_ctas;           // > 0: CTAs of a launch whose pieces are balanced on the device (else 0)
   int sms;                     // SMs, for that
   int csize;                   // thread-block cluster size along the splits (1 = no cluster)
@@ -66,6 +67,12 @@ struct TmaMaps {
 cudaError_t launch_block_attn_tc(const AttnArgs& a, const TmaMaps& maps, int head_dim, cudaStream_t stream);
 // The same for a table mask (a.mode == kModeBlockMask; block_attn_tc_masked.cu).
 cudaError_t launch_block_attn_tc_masked(const AttnArgs& a, const TmaMaps& maps, int head_dim, cudaStream_t stream);
+// Unsplit sequences, the a.halved longest as block-slot halves in two CTAs (half,
+// half_maps), the others whole in one (a, maps).
+cudaError_t launch_block_attn_tc_mixed(const AttnArgs& a, const TmaMaps& maps, const AttnArgs& half,
+                                       const TmaMaps& half_maps, int head_dim, cudaStream_t stream);
+cudaError_t launch_block_attn_tc_mixed_masked(const AttnArgs& a, const TmaMaps& maps, const AttnArgs& half,
+                                              const TmaMaps& half_maps, int head_dim, cudaStream_t stream);
 // A kernel whose one mbarrier wait can never complete (decide.cu).
 cudaError_t launch_wait_timeout_check(uint64_t limit_ns, unsigned int* err, cudaStream_t stream);
 cudaError_t launch_combine(const __nv_bfloat16* o_part, const float* lse_part, int S, int B, int Hq, int bl,

@@ -261,6 +261,25 @@ def test_route_invariants(L, B, Hkv, G, bl, prefix, D):
                     assert (r["pieces"], r["chunk"], r["cluster"]) == (plan["splits"], plan["chunk"], plan["cluster"])
 
 
+@pytest.mark.parametrize("B,prefix,D,flags,order,cluster,ctas", [
+    (10, 1900, 128, 0, 3, 1, 152),           # 9 of 10 sequences may run as halves
+    (14, 4096, 128, 0, 3, 1, 152),
+    (16, 4096, 128, 0, 0, 1, 128),           # too few SMs left for halves
+    (10, 400, 128, 0, 0, 1, 80),             # short: whole
+    (10, 9000, 128, 0, 1, 2, 160),           # long: cluster pairs
+    (10, 9000, 128, 4, 3, 1, 152),           # ... which NLD_ATTN_NO_CLUSTER forbids
+    (10, 3000, 64, 0, 1, 2, 160), (10, 1900, 64, 0, 3, 1, 152),
+    (19, 1900, 128, 0, 0, 1, 152), (20, 1900, 128, 0, 1, 1, 160)])
+def test_route_unsplit_wide_sequences(L, B, prefix, D, flags, order, cluster, ctas):
+    """160 rows over 8 KV heads, unsplit: whole sequences, some of them as
+    block-slot halves, or cluster pairs."""
+    for mask in (False, True):
+        if mask and order == 1 and cluster == 1:
+            continue  # with a table mask only ranges above 2048 tokens are ordered
+        r = _route(B, 40, 8, D, 16, prefix, 32, 0, flags, mask)
+        assert (r["order"], r["cluster"], r["ctas"], r["partials"]) == (order, cluster, ctas, 1)
+
+
 def test_plan_partials_fit_the_static_scratch(L):
     """The finer plans stay within the 16 MiB of nld_block_attn_static_scratch
     wherever the two-wave plan does."""

@@ -912,6 +912,39 @@ def test_attention_halves_of_ragged_sequences(orc):
             compare_attn(out, lse, ro, rl, f"halves mode={mode} flags={flags}")
 
 
+MIXED_LENS = {
+    "ragged": lambda b, n: 900 * (b * b % n) // n,         # the longest as halves, some whole
+    "equal": lambda b, n: 700,                             # whole, all of them
+    "one long": lambda b, n: 899 if b == n // 2 else b % 3,
+}
+
+
+@pytest.mark.parametrize("name", sorted(MIXED_LENS))
+@pytest.mark.parametrize("G,bl,D", [(10, 16, 64), (5, 32, 128), (8, 32, 128), (13, 10, 128)])
+def test_attention_mixed_whole_and_halves(orc, name, G, bl, D):
+    """Unsplit sequences of 129..256 rows in one wave: the longest as block-slot
+    halves, the others whole, both in one launch; the passes and the causal
+    table, whose mask is the verify pass's."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    B = sms // 8 + 1  # 4 KV heads: a few more units than half the SMs
+    lens = [MIXED_LENS[name](b, B) for b in range(B)]
+    case = W.make_block_attn_case("mixed", B, G * 4, 4, D, block_len=bl, page_size=32, prefix_lens=lens, seed=12)
+    dc = DeviceCase(case)
+    route = nld.nld_block_attn_route(dc.params(), bl)
+    assert route["order"] == 3 and route["partials"] == 1
+    rows = rows_per_unit(case, 3, 13)
+    kv = case.kv
+    for mode in (DIFF, VER):
+        ro, rl = orc.block_attn_rows(dc.q_bits(mode), kv.k_bits, kv.v_bits, kv.page_table, kv.prefix_lens,
+                                     case.num_q_heads, case.num_kv_heads, bl, mode, case.scale, rows)
+        runs = [dc.run(mode, flags=flags) for flags in (0, nld.NLD_ATTN_PREFIX_READY)]
+        if mode == VER:
+            runs.append(run_masked(dc, [(2 << i) - 1 & 0xFFFFFFFF for i in range(bl)], q=dc.q[VER]))
+        for i, (out, lse) in enumerate(runs):
+            compare_attn(out[rows[:, 0], rows[:, 1], rows[:, 2]], lse[rows[:, 0], rows[:, 2], rows[:, 1]], ro, rl,
+                         f"mixed {name} G={G} bl={bl} D={D} mode={mode} run {i}")
+
+
 BALANCED_LENS = {
     "equal": [5000] * 7,
     "one long": [9000, 0, 1, 2, 40],
