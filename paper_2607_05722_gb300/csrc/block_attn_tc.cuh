@@ -55,6 +55,8 @@
 // max grows by more than 2^8 (P then stays below 256, exact enough in bf16);
 // the final division by the matching sum removes the reference max.
 #pragma once
+#include <type_traits>
+
 #include "nld_internal.cuh"
 
 namespace nld {
@@ -811,19 +813,20 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
     if constexpr (MT == 2) {
       // Two M tiles, a softmax group each: its step is a whole product, 128
       // columns a thread. P goes over the S columns it has read.
-      const int nprod = (ntiles + 1) / 2;
       const int row_warps = tile_row_warps(mt);
-      for (int j = 0; warp_rows && j < nprod; ++j) {
+      // one product of TILES tiles
+      auto step = [&](int j, auto tiles) -> bool {
+        constexpr int kTiles = decltype(tiles)::value;
         const int t_own = t_begin + 2 * j * kTileTok;
-        if (!warp_wait(&s_full[mt], j & 1)) {
-          ok = false;
-          break;
-        }
+        if (!warp_wait(&s_full[mt], j & 1)) return false;
         tc_fence_after();
-        float s[2 * kTileTok];
-        tmem_ld128(tS(mt, 0) + lane_off, s);
+        float s[kTiles * kTileTok];
+        if constexpr (kTiles == 2)
+          tmem_ld128(tS(mt, 0) + lane_off, s);
+        else
+          tmem_ld64(tS(mt, 0) + lane_off, s);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < kTiles; ++h) {
           uint64_t vis;
           if constexpr (MASKED) {
             vis = column_mask(t_own + h * kTileTok);
@@ -839,7 +842,7 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
         }
         float pm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-        for (int e = 0; e < 2 * kTileTok; e += 8) {
+        for (int e = 0; e < kTiles * kTileTok; e += 8) {
 #pragma unroll
           for (int q = 0; q < 4; ++q) pm[q] = fmax3(pm[q], s[e + 2 * q], s[e + 2 * q + 1]);
         }
@@ -874,7 +877,7 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
           float2 ls[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
           const uint32_t tp = tS(mt, 0) + lane_off;
 #pragma unroll
-          for (int c = 0; c < 2 * kTileTok / 16; ++c) {
+          for (int c = 0; c < kTiles * kTileTok / 16; ++c) {
             uint32_t w[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
@@ -894,10 +897,7 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
           // zeroes them before its PV product (P is 0 there, but 0 * NaN =
           // NaN; the other group's PV reads the same zeros).
           const int kz = 2 * j + valid / kTileTok, st = kz % kVStages;
-          if (!warp_wait(&v_full[j % kVSlots], (j / kVSlots) & 1)) {
-            ok = false;
-            break;
-          }
+          if (!warp_wait(&v_full[j % kVSlots], (j / kVSlots) & 1)) return false;
           const int r0 = valid % kTileTok, r1 = (r0 + a.box_tok - 1) & ~(a.box_tok - 1);
           uint8_t* vt = smem + Lay::kVOff + st * Geo::kTileBytes;
           for (int idx = sm_tid - mt * 128; idx < (r1 - r0) * (D / 8); idx += 32 * row_warps) {
@@ -909,6 +909,12 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&p_full[mt]);
+        return true;
+      };
+      if (warp_rows) {
+        const int whole = ntiles / 2;
+        for (int j = 0; ok && j < whole; ++j) ok = step(j, std::integral_constant<int, 2>{});
+        if (ok && (ntiles & 1)) ok = step(whole, std::integral_constant<int, 1>{});
       }
     } else if constexpr (CG == 2) {
       // Two softmax groups over every score product j: group c takes tile
