@@ -187,8 +187,17 @@ void plan_splits_for(const nld_attn_params_t* p, int block_len, int sms, Cluster
       // of two score products or more (28 units of 912 tokens: 5 pieces 10.5
       // us, 4 pieces 10.1).
       const int floor2 = want >= 8 ? 8 : want >= 4 ? 4 : 2;
+      // With two M tiles a piece's time goes by its products of 128 tokens: the
+      // fewest CTAs with the fewest products (20 units of 721 tokens, 168 rows, 6
+      // pieces of one product 13.4 us, 4 of one and a half 14.7).
       int cs = want;
-      while (cs >= floor2 && (units > clusters_resident(cs) || (!is_pow2(cs) && max_tokens < 256 * cs))) --cs;
+      if (rows > 128) {
+        const auto products = [&](int n) { return (max_tokens + 128ll * n - 1) / (128ll * n); };
+        while (cs >= floor2 && units > clusters_resident(cs)) --cs;
+        for (int n = cs - 1; n >= floor2; --n)
+          if (products(n) <= products(cs)) cs = n;
+      }
+      while (rows <= 128 && cs >= floor2 && (units > clusters_resident(cs) || (!is_pow2(cs) && max_tokens < 256 * cs))) --cs;
       if (cs >= floor2) {
         want = cs;
         csize = cs;

@@ -261,6 +261,14 @@ def test_route_invariants(L, B, Hkv, G, bl, prefix, D):
                     assert (r["pieces"], r["chunk"], r["cluster"]) == (plan["splits"], plan["chunk"], plan["cluster"])
 
 
+@pytest.mark.parametrize("B,prefix,cluster", [(5, 700, 6), (5, 1000, 4), (1, 224, 4), (7, 700, 4)])
+def test_route_two_tile_clusters_by_products(L, B, prefix, cluster):
+    """168 rows, an odd block length, 4 KV heads: the fewest CTAs a cluster with
+    the fewest 128-token products each."""
+    r = _route(B, 32, 4, 128, 16, prefix, 21)
+    assert (r["cluster"], r["partials"], r["halves"]) == (cluster, 1, 1)
+
+
 @pytest.mark.parametrize("B,prefix,D,flags,order,cluster,ctas", [
     (10, 1900, 128, 0, 3, 1, 152),           # 9 of 10 sequences may run as halves
     (14, 4096, 128, 0, 3, 1, 152),
