@@ -400,6 +400,7 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
       const int tokens = min(max(reinterpret_cast<const int*>(smem)[piece.b], 0), a.max_pages * a.page_size - a.bl) + a.bl;
       piece.chunk = ((tokens + 1) / 2 + kTileTok - 1) & ~(kTileTok - 1);
     }
+    fence_proxy_async_smem();  // the ranks' accesses before the copies into the ring
   }
   const int b = piece.b;
   const int t_begin = split * piece.chunk;
@@ -1610,6 +1611,7 @@ __global__ void __launch_bounds__(TcCfg<2, 2>::kThreads, 1)
   const int* order = scratch + a.B;
   const int rest = a.halved < a.B ? scratch[order[a.halved]] : 0;
   const bool halves = rest < scratch[order[0]] - scratch[order[0]] / 8;
+  fence_proxy_async_smem();
   if (second && !halves) return;
   if (halves && rank < a.halved)
     block_attn_tc_body<D, 1, 1, 2, MASKED, kPicked, 2>(half_maps, half, piece);
