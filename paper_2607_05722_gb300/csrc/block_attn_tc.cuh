@@ -14,13 +14,13 @@
 //             refills once its score product is done.
 //   warp 3    allocates the TMEM columns; lane 0 loads Q by TMA (one M tile)
 //             and issues every MMA:
-//               S_j = Q K^T     (M=128 rows, N=64*TPS tokens, K=D; double-buffered in TMEM)
+//               S_j = Q K^T     (M=128 rows, N=128 tokens, K=D; double-buffered in TMEM)
 //               O  += P_k V_k   (M=128 rows, N=D, K=64 tokens; V read MN-major)
 //             S_{j+1} is issued before the PV products of S_j so the tensor
 //             core computes the next scores while the softmax warps work.
-//             Each MMA or commit instruction holds the issuing thread ~50
-//             cycles (measured), so the one issuing thread is a serial
-//             resource of the chain.
+//             Each instruction holds the issuing thread (a commit ~50 cycles,
+//             an MMA 70 to 98 with two M tiles, measured), so the one issuing
+//             thread is a serial resource of the chain.
 //   warps 4.. softmax: thread t owns TMEM lane 32*(warp%4)+lane, one query
 //             row. It loads its S row, applies the mask and the base-2 scale,
 //             keeps the running max and sum, writes P (bf16) back to TMEM
@@ -31,10 +31,10 @@
 //             split partials, in packed row order).
 //             With 33..64 packed rows and a split that fits in the ring, Q
 //             is replicated into the idle lane quadrants (REP = 2): each copy
-//             of a row takes a 32-token slice of every tile with its own
-//             running max and sum, so every softmax warp works and each does
-//             half of the exponentials; the copies are merged once, each
-//             finalising half of the columns.
+//             of a row takes one of the two tiles of every score product with
+//             its own running max and sum, so every softmax warp works and
+//             each does half of the exponentials; the copies are merged once,
+//             each finalising half of the columns.
 //             With two M tiles each has a softmax group of its own, and the
 //             tensor core works on one tile while the other's group turns its
 //             scores into P.
@@ -67,7 +67,7 @@ constexpr int kMmaWarp = 3;
 constexpr int kSoftmaxWarp0 = 4;
 
 // MT 128-row M tiles per CTA (MT = 2 for 129..256 packed rows); 4*MT
-// softmax warps; TPS = 2 64-token K/V tiles per score product: N = 128
+// softmax warps; two 64-token K/V tiles per score product: N = 128
 // products, which the tensor core runs at full rate (N = 64 at about half), and
 // half as many steps in the chain S -> softmax -> PV. The ring takes what
 // shared memory the Q tiles leave (up to 8 stages): a streaming CTA's bandwidth
@@ -96,11 +96,10 @@ constexpr int kSoftmaxWarp0 = 4;
 // PV MMAs, each softmax thread exponentiates one 64-column tile, and a score
 // product waits only for the softmax warps to have read its S buffer: the
 // chain S -> softmax -> PV no longer holds the next score products back.
-template <int MT, int TPS, int CG = 1>
+template <int MT, int CG = 1>
 struct TcCfg {
-  static_assert(TPS == 2, "paired score products");
   static_assert(CG == 1 || (CG == 2 && MT == 1), "two softmax groups: one M tile");
-  static constexpr int kTPS = TPS;               // K/V tiles per score product
+  static constexpr int kTPS = 2;                 // K/V tiles per score product
   static constexpr int kSTok = kTPS * kTileTok;  // tokens (N) of a score product
   static constexpr int kPBufs = 2 * kTPS;        // tiles in flight between the softmax and PV (barrier slots)
   static constexpr int kSmWarps = 4 * MT * CG;   // softmax warps
@@ -122,23 +121,23 @@ __host__ __device__ constexpr int merge_pitch() { return D * 4 + 16; }
 // K/V ring: the K tiles (the tiles of consecutive stages follow one another
 // with the same 8-token group stride, so two form one operand of 128 rows),
 // then the V tiles.
-template <int D, int MT, int TPS>
+template <int D, int MT>
 struct TcLayout {
   using Geo = TileGeom<D>;
-  static constexpr int kPBufs = TcCfg<MT, TPS>::kPBufs;
+  static constexpr int kPBufs = TcCfg<MT>::kPBufs;
   static constexpr int kQBytes = Geo::kColBlocks * 128 * 128;  // one 128-row Q tile, bf16
   // K and V stages: what is left of 227 KB after Q, 512 bytes of barriers, the
   // 1024-byte alignment slack and the row maxima that two softmax groups
-  // exchange, a multiple of TPS, at most 8 (P lives in TMEM). With two M tiles
+  // exchange, even, at most 8 (P lives in TMEM). With two M tiles
   // and D = 128 the K ring takes the odd product that fits: its slots are free
   // only when both tiles' score products have completed.
   static constexpr int kXmBytes = MT == 2 ? 0 : 1536;
   static constexpr int kFree = 232448 - 1024 - 512 - kXmBytes - MT * kQBytes;
   static constexpr int kFitStages = kFree / Geo::kStageBytes;
-  static constexpr int kVStages = (kFitStages < 8 ? kFitStages : 8) / TPS * TPS;
+  static constexpr int kVStages = (kFitStages < 8 ? kFitStages : 8) / 2 * 2;
   static constexpr int kKFit = (kFree - kVStages * Geo::kTileBytes) / Geo::kTileBytes;
-  static constexpr int kKStages = MT == 2 ? (kKFit < 8 ? kKFit : 8) / TPS * TPS : kVStages;
-  static_assert(kVStages >= 2 * TPS, "at least two score products in the ring");
+  static constexpr int kKStages = MT == 2 ? (kKFit < 8 ? kKFit : 8) / 2 * 2 : kVStages;
+  static_assert(kVStages >= 4, "at least two score products in the ring");
   static constexpr int kVOff = kKStages * Geo::kTileBytes;      // V tiles after the K tiles
   static constexpr int kQOff = kVOff + kVStages * Geo::kTileBytes;
   static constexpr int kPOff = kQOff + MT * kQBytes;  // end of the ring and Q tiles
@@ -262,14 +261,14 @@ __device__ __noinline__ void balanced_piece(const AttnArgs& a, Piece* out) {
   if (__ballot_sync(kFull, hit) == 0u && lane == 0) out->b = -1;
 }
 
-template <int D, int MT, int REP, int TPS, bool MASKED, int ORDER, int CG>
+template <int D, int MT, int REP, bool MASKED, int ORDER, int CG>
 __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const AttnArgs& a, Piece piece) {
   static_assert(REP == 1 || REP == 2, "replication of 1 or 2 (up to 32 rows run on two softmax groups)");
   static_assert(MT == 1 || REP == 1, "replication only with one M tile");
   static_assert(CG == 1 || REP == 1, "softmax groups without row copies");
   using Geo = TileGeom<D>;
-  using Cfg = TcCfg<MT, TPS, CG>;
-  using Lay = TcLayout<D, MT, TPS>;
+  using Cfg = TcCfg<MT, CG>;
+  using Lay = TcLayout<D, MT>;
   constexpr int kTcStages = Lay::kKStages;  // K ring; V ring the same but with two M tiles
   constexpr int kVStages = Lay::kVStages;
   // Ring barriers. With two softmax groups or two M tiles K and V slots fill
@@ -299,9 +298,9 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
   uint64_t* q_ready = o_done + Cfg::kPBufs;
   uint64_t* q_full = q_ready + 1;  // the Q tiles' TMA copies (one M tile)
   uint64_t* drain = q_full + 1;
-  // o_fin (two softmax groups): every PV product has completed (committed
-  // once, after the last). With one group every softmax warp waits on the
-  // last o_done phase.
+  // o_fin (two softmax groups or two M tiles): every PV product has completed
+  // (committed once, after the last). With row copies every softmax warp waits
+  // on the last o_done phase.
   uint64_t* o_fin = drain + 1;
   // xm_full[b] (two softmax groups): every softmax warp has written its rows'
   // score maxima of the step with parity b
@@ -563,17 +562,14 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
       auto issue_s = [&](int j) {
         const int st = (j * kTPS) % kTcStages;
         const uint32_t k_addr = smem_u32(smem) + static_cast<uint32_t>(st * Geo::kTileBytes);
+        const uint32_t d = tS(0, j & 1);
 #pragma unroll
-        for (int mt = 0; mt < MT; ++mt) {
-          const uint32_t d = tS(mt, j & 1);
-#pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) {
-            const uint32_t koff = (kk & 3) * 32;  // 16 elements along the 128-byte row
-            const int cb = kk >> 2;               // 64-dim column block
-            const uint64_t ad = sw128_desc(q_addr + mt * Lay::kQBytes + cb * (128 * 128) + koff, 0, 1024);
-            const uint64_t bd = sw128_desc(k_addr + cb * 1024 + koff, 0, Geo::kGroup8Bytes);
-            umma_bf16(d, ad, bd, idesc_s, kk > 0 ? 1u : 0u);
-          }
+        for (int kk = 0; kk < D / 16; ++kk) {
+          const uint32_t koff = (kk & 3) * 32;  // 16 elements along the 128-byte row
+          const int cb = kk >> 2;               // 64-dim column block
+          const uint64_t ad = sw128_desc(q_addr + cb * (128 * 128) + koff, 0, 1024);
+          const uint64_t bd = sw128_desc(k_addr + cb * 1024 + koff, 0, Geo::kGroup8Bytes);
+          umma_bf16(d, ad, bd, idesc_s, kk > 0 ? 1u : 0u);
         }
         umma_commit(&s_full[j & 1]);
         if (kSplitKV) umma_commit(&k_empty[j % kKSlots]);  // the K slot is free once the product completes
@@ -584,18 +580,14 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
       auto issue_pv = [&](int k) {
         const int st = k % kTcStages;
         const uint32_t v_addr = smem_u32(smem + Lay::kVOff + st * Geo::kTileBytes);
+        // A = P in TMEM (bf16 pairs, 32 columns per 64-token tile, over S
+        // columns its tile's softmax has consumed); B = V (MN-major: 64-dim
+        // atoms LBO apart, 8-token row groups SBO apart).
+        const uint32_t p_tmem = tS(0, (k / kTPS) & 1) + static_cast<uint32_t>((k % kTPS) * kPCols);
 #pragma unroll
-        for (int mt = 0; mt < MT; ++mt) {
-          // A = P in TMEM (bf16 pairs, 32 columns per 64-token tile, over S
-          // columns its tile's softmax has consumed); B = V (MN-major: 64-dim
-          // atoms LBO apart, 8-token row groups SBO apart).
-          const uint32_t p_tmem = tS(mt, (k / kTPS) & 1) + static_cast<uint32_t>((k % kTPS) * kPCols);
-          const uint32_t o_acc = tO(mt);
-#pragma unroll
-          for (int kt = 0; kt < kTileTok / 16; ++kt) {
-            const uint64_t bd = sw128_desc(v_addr + kt * 2 * Geo::kGroup8Bytes, 1024, Geo::kGroup8Bytes);
-            umma_bf16_ts(o_acc, p_tmem + kt * 8, bd, idesc_o, (k > 0 || kt > 0) ? 1u : 0u);
-          }
+        for (int kt = 0; kt < kTileTok / 16; ++kt) {
+          const uint64_t bd = sw128_desc(v_addr + kt * 2 * Geo::kGroup8Bytes, 1024, Geo::kGroup8Bytes);
+          umma_bf16_ts(tO(0), p_tmem + kt * 8, bd, idesc_o, (k > 0 || kt > 0) ? 1u : 0u);
         }
         umma_commit(&o_done[k % kPBufs]);
         umma_commit(&k_empty[st]);
@@ -706,24 +698,16 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
   } else if (warp >= kSoftmaxWarp0) {  // warp 2 has no role
     // ---------------- softmax warps ----------------
     // Warp `quad` reads TMEM lanes 32*quad..+31. With REP > 1 those lanes hold
-    // a copy of row block rq = quad % kRowQuads and the warp takes the token
-    // slice cp = quad / kRowQuads (columns c0u .. c0u+kColsU-1) of every step.
+    // a copy of row block rq = quad % kRowQuads and the warp takes tile
+    // 2j + cp of every product j, cp = quad / kRowQuads.
     constexpr int kRowQuads = 4 / REP;
-    // Softmax steps: one tile, or with paired score products and copies
-    // (TPS = 2, REP >= 2) the whole product, so that a step's columns per
-    // thread stay at most 64 and its work is one max and one exponential pass.
-    constexpr int kU = (kTPS == 2 && REP >= 2) ? 2 : 1;  // tiles per softmax step
-    constexpr int kColsU = kU * kTileTok / REP;          // S columns per thread and step
     const int quad = warp & 3;
     const int wg = (warp - kSoftmaxWarp0) >> 2;
     const int mt = CG == 1 ? wg : 0;                // M tile of this warp
     const int cg = CG == 1 ? 0 : wg;                // softmax group: tile 2j + cg of score product j
     const int part = CG == 1 ? quad / kRowQuads : cg;  // this thread's share of a row's state (copy or group)
     const int rq = quad % kRowQuads;                // row block
-    const int cp = quad / kRowQuads;                // token slice
-    const int c0u = cp * kColsU;           // first column of this thread's slice of a step
-    const int h_own = c0u / kTileTok;      // the step's tile holding the slice
-    const int lc0 = c0u % kTileTok;        // first column of the slice within that tile
+    const int cp = quad / kRowQuads;                // copy of the row: its tile of each product
     const int r_loc = quad * 32 + lane;             // TMEM lane == row of the Q and P tiles
     const int r = mt * 128 + rq * 32 + lane;        // packed query row
     const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
@@ -738,8 +722,8 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
 
     // Q rows in shared memory, 128-byte-swizzled K-major (padding rows zero).
     // One M tile: the MMA warp brings Q by TMA and the rows past R are zeroed
-    // here, before the dependency wait. Two M tiles: slice 0 of each row loads
-    // it here after the wait and writes every copy.
+    // here, before the dependency wait. Two M tiles: each thread loads its row
+    // here after the wait.
     if (MT == 1 && !row_ok && cg == 0) {
 #pragma unroll
       for (int c = 0; c < D / 8; ++c)
@@ -748,19 +732,15 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
     }
     if (MT == 2 && early) grid_dependency_wait();
     {
-      if (MT == 2 && cp == 0) {
+      if (MT == 2) {
         const uint4* qrow = reinterpret_cast<const uint4*>(
             a.q + ((static_cast<size_t>(b) * a.bl + row_i) * a.Hq + row_h) * D);
         uint4 v[D / 8];
 #pragma unroll
         for (int c = 0; c < D / 8; ++c) v[c] = row_ok ? __ldg(qrow + c) : make_uint4(0, 0, 0, 0);
 #pragma unroll
-        for (int q = 0; q < REP; ++q) {
-          const int rl = r_loc + q * kRowQuads * 32;  // TMEM lane of copy q (same swizzle phase)
-#pragma unroll
-          for (int c = 0; c < D / 8; ++c)
-            *reinterpret_cast<uint4*>(q_tile + (c >> 3) * (128 * 128) + rl * 128 + (((c & 7) ^ swz) << 4)) = v[c];
-        }
+        for (int c = 0; c < D / 8; ++c)
+          *reinterpret_cast<uint4*>(q_tile + (c >> 3) * (128 * 128) + r_loc * 128 + (((c & 7) ^ swz) << 4)) = v[c];
       }
       fence_proxy_async_smem();
       __syncwarp();
@@ -793,12 +773,12 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
     if constexpr (MASKED) rowbits = row_ok ? __ldg(a.block_mask + row_i) : 0u;
     const int plim = min(t_end, L);  // prefix keys of this split end here
     auto column_mask = [&](int col0) -> uint64_t {  // col0: token of this thread's first column
-      const int np = min(max(plim - col0, 0), kColsU);
+      const int np = min(max(plim - col0, 0), kTileTok);
       uint64_t vis = np >= 64 ? ~0ull : (1ull << np) - 1ull;
       const int off = col0 - L;  // block slot of column 0
-      if (off < a.bl && off + kColsU > 0) {
+      if (off < a.bl && off + kTileTok > 0) {
         uint64_t bb = off >= 0 ? static_cast<uint64_t>(rowbits) >> off : static_cast<uint64_t>(rowbits) << -off;
-        const int nvalid = min(max(t_end - col0, 0), kColsU);
+        const int nvalid = min(max(t_end - col0, 0), kTileTok);
         bb &= nvalid >= 64 ? ~0ull : (1ull << nvalid) - 1ull;
         vis |= bb;
       }
@@ -1083,32 +1063,21 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
         if (lane == 0) mbar_arrive(&p_full[j & 1]);
       }
     }
-    // One softmax group: a step is one tile, or the whole product with row
-    // copies and paired products.
-    for (int k0 = 0; CG == 1 && MT == 1 && k0 < ntiles; k0 += kU) {  // k0: first tile of the step
-      const int j = k0 / kTPS, half = k0 % kTPS;  // score product and the step's first 64-token half
-      const int step_t0 = t_begin + k0 * kTileTok;
-      const int k_own = k0 + h_own;               // the tile holding this thread's columns
-      if (half == 0 && !warp_wait(&s_full[j & 1], (j >> 1) & 1)) {
+    // Row copies: a step is a whole product, one tile of it for each copy.
+    for (int k0 = 0; CG == 1 && MT == 1 && k0 < ntiles; k0 += kTPS) {  // k0: first tile of the product
+      const int j = k0 / kTPS;
+      const int k_own = k0 + cp;  // this copy's tile
+      const int t_own = t_begin + k_own * kTileTok;
+      if (!warp_wait(&s_full[j & 1], (j >> 1) & 1)) {
         ok = false;
         break;
       }
       tc_fence_after();
-      float s[kColsU];
-      if (warp_rows) {
-        const uint32_t ts = tS(mt, j & 1) + lane_off + static_cast<uint32_t>(half * kTileTok + c0u);
-        if constexpr (kColsU == 64) {
-          tmem_ld64(ts, s);
-        } else if constexpr (kColsU == 32) {
-          tmem_ld32(ts, s);
-        } else {
-          tmem_ld16(ts, s);
-        }
-      }
+      float s[kTileTok];
+      if (warp_rows) tmem_ld64(tS(0, j & 1) + lane_off + static_cast<uint32_t>(cp * kTileTok), s);
       tc_fence_before();
       __syncwarp();
-      const int k_last = min(k0 + kU - 1, ntiles - 1);  // last tile of the step
-      if (lane == 0 && (k_last % kTPS == kTPS - 1 || k_last == ntiles - 1)) mbar_arrive(&s_free[j & 1]);
+      if (lane == 0) mbar_arrive(&s_free[j & 1]);
 
       float alpha = 1.f;
       bool rescale = false;
@@ -1119,19 +1088,18 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
         // warp sees in full (nearly every prefix step) takes no mask.
         uint64_t vis = ~0ull;
         if constexpr (MASKED) {
-          vis = column_mask(step_t0 + c0u);
+          vis = column_mask(t_own);
         } else {
-          const int nv = lim - (step_t0 + c0u);
+          const int nv = lim - t_own;
           vis = nv >= 64 ? ~0ull : nv <= 0 ? 0ull : (1ull << nv) - 1ull;
         }
-        constexpr uint64_t kAll = kColsU >= 64 ? ~0ull : (1ull << kColsU) - 1ull;
-        if (!__all_sync(0xffffffffu, (vis & kAll) == kAll)) {
+        if (!__all_sync(0xffffffffu, vis == ~0ull)) {
 #pragma unroll
-          for (int e = 0; e < kColsU; ++e) s[e] = ((vis >> e) & 1ull) ? s[e] : -INFINITY;
+          for (int e = 0; e < kTileTok; ++e) s[e] = ((vis >> e) & 1ull) ? s[e] : -INFINITY;
         }
         float pm[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-        for (int e = 0; e < kColsU; e += 8) {
+        for (int e = 0; e < kTileTok; e += 8) {
 #pragma unroll
           for (int q = 0; q < 4; ++q) pm[q] = fmax3(pm[q], s[e + 2 * q], s[e + 2 * q + 1]);
         }
@@ -1157,18 +1125,17 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
 #pragma unroll 1
         for (int c = 0; c < D / 32; ++c) {
           float o[32];
-          tmem_ld32(tO(mt) + lane_off + c * 32, o);
+          tmem_ld32(tO(0) + lane_off + c * 32, o);
 #pragma unroll
           for (int e = 0; e < 32; ++e) o[e] *= alpha;
-          tmem_st32(tO(mt) + lane_off + c * 32, o);
+          tmem_st32(tO(0) + lane_off + c * 32, o);
         }
       }
       if (warp_rows) {
         // P goes to TMEM over the consumed S columns: tile k of the product
-        // takes columns (k % TPS) * 32 .. +31 of its S buffer, bf16 pairs.
-        // This thread writes its slice of the tile k_own and zeros over the
-        // rest of the step's tiles (other copies' slices).
-        const uint32_t tbuf = tS(mt, j & 1) + lane_off;
+        // takes columns (k % 2) * 32 .. +31 of its S buffer, bf16 pairs. This
+        // thread writes its copy's tile and zeros over the other copy's.
+        const uint32_t tbuf = tS(0, j & 1) + lane_off;
         constexpr int kPColsS = kTileTok / 2;
         if (k_own < ntiles) {
           // p = 2^(s * scale * log2(e) - m): per pair of elements one paired
@@ -1176,9 +1143,9 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
           const float nmu = m_run == -INFINITY ? 0.f : -m_run;
           const float2 sc2 = make_float2(scl, scl), nm2 = make_float2(nmu, nmu);
           float2 ls[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-          const uint32_t tp = tbuf + static_cast<uint32_t>((k_own % kTPS) * kPColsS);
+          const uint32_t tp = tbuf + static_cast<uint32_t>(cp * kPColsS);
 #pragma unroll
-          for (int c = 0; c < kColsU / 16; ++c) {  // 16 columns (8 TMEM columns) per store
+          for (int c = 0; c < kTileTok / 16; ++c) {  // 16 columns (8 TMEM columns) per store
             uint32_t w[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
@@ -1187,28 +1154,18 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
               ls[e & 1] = add2(ls[e & 1], pp);
               w[e] = pack_bf16(pp.x, pp.y);
             }
-            tmem_st_u32<8>(tp + static_cast<uint32_t>(lc0 / 2 + c * 8), w);
+            tmem_st_u32<8>(tp + static_cast<uint32_t>(c * 8), w);
           }
           l_run += (ls[0].x + ls[0].y) + (ls[1].x + ls[1].y);
-          if constexpr (kColsU < kTileTok) {
-#pragma unroll
-            for (int q = 0; q < kTileTok / kColsU; ++q)
-              if (q != lc0 / kColsU) tmem_st_zero<kColsU / 2>(tp + static_cast<uint32_t>(q * (kColsU / 2)));
-          }
         }
-        if constexpr (kU > 1) {
-#pragma unroll
-          for (int h = 0; h < kU; ++h)
-            if (h != h_own && k0 + h < ntiles)
-              tmem_st_zero<32>(tbuf + static_cast<uint32_t>(((k0 + h) % kTPS) * 32));
-        }
+        if (k0 + (cp ^ 1) < ntiles) tmem_st_zero<kPColsS>(tbuf + static_cast<uint32_t>((cp ^ 1) * kPColsS));
         tmem_wait_st();
       }
-      // Hand the step's tiles to the MMA warp (every softmax warp arrives
-      // for every tile; the P columns of other copies' slices are zero).
+      // Hand the product's tiles to the MMA warp (every softmax warp arrives
+      // for both; the P columns of the other copy's tile are zero).
       bool step_ok = true;
 #pragma unroll
-      for (int h = 0; h < kU; ++h) {
+      for (int h = 0; h < kTPS; ++h) {
         const int k = k0 + h;
         if (k >= ntiles) break;
         const int valid = t_end - (t_begin + k * kTileTok);
@@ -1223,7 +1180,7 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
           }
           const int r0 = valid, r1 = (valid + a.box_tok - 1) & ~(a.box_tok - 1);
           uint8_t* vt = smem + Lay::kVOff + st * Geo::kTileBytes;
-          for (int idx = grp_tid; idx < (r1 - r0) * (D / 8); idx += 128 * MT) {
+          for (int idx = grp_tid; idx < (r1 - r0) * (D / 8); idx += 128) {
             const int row = r0 + idx / (D / 8), c = idx % (D / 8);
             *reinterpret_cast<uint4*>(vt + kv_swz<D>(row, c)) = make_uint4(0, 0, 0, 0);
           }
@@ -1240,7 +1197,7 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
     }
 
     // ---------------- epilogue ----------------
-    // Every PV has completed once o_fin (one group: the last o_done phase)
+    // Every PV has completed once o_fin (row copies: the last o_done phase)
     // fires, so the K/V ring is free for staging. Warp-uniform, like every condition around the warp-collective
     // TMEM loads and stores below.
     const bool o_ready = __all_sync(
@@ -1574,10 +1531,10 @@ __device__ __forceinline__ void block_attn_tc_body(const TmaMaps& maps, const At
   }
 }
 
-template <int D, int MT, int REP, int TPS, bool MASKED, int ORDER, int CG>
-__global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
+template <int D, int MT, int REP, bool MASKED, int ORDER, int CG>
+__global__ void __launch_bounds__(TcCfg<MT, CG>::kThreads, 1)
     block_attn_tc_kernel(const __grid_constant__ TmaMaps maps, const AttnArgs a) {
-  block_attn_tc_body<D, MT, REP, TPS, MASKED, ORDER, CG>(
+  block_attn_tc_body<D, MT, REP, MASKED, ORDER, CG>(
       maps, a,
       {static_cast<int>(blockIdx.z), static_cast<int>(blockIdx.y), static_cast<int>(blockIdx.x), a.chunk, 0});
 }
@@ -1594,10 +1551,10 @@ __global__ void __launch_bounds__(TcCfg<MT, TPS, CG>::kThreads, 1)
 // 34.2 / 31.5, 10 of 1900 35.3 / 37.5 (the ranking); in cluster pairs of half
 // sequences / mixed: 12 of 512..4096 51.0 / 42.1, 14 of 3000 69.6 / 51.3.
 template <int D, bool MASKED>
-__global__ void __launch_bounds__(TcCfg<2, 2>::kThreads, 1)
+__global__ void __launch_bounds__(TcCfg<2>::kThreads, 1)
     block_attn_tc_mixed_kernel(const __grid_constant__ TmaMaps maps, const AttnArgs a,
                                const __grid_constant__ TmaMaps half_maps, const AttnArgs half) {
-  static_assert(TcCfg<2, 2>::kThreads == TcCfg<1, 2, 2>::kThreads, "one block shape for both");
+  static_assert(TcCfg<2>::kThreads == TcCfg<1, 2>::kThreads, "one block shape for both");
   extern __shared__ uint8_t smem_raw[];
   grid_launch_dependents();
   if (a.prefix_ready == 0) grid_dependency_wait();
@@ -1614,16 +1571,16 @@ __global__ void __launch_bounds__(TcCfg<2, 2>::kThreads, 1)
   fence_proxy_async_smem();
   if (second && !halves) return;
   if (halves && rank < a.halved)
-    block_attn_tc_body<D, 1, 1, 2, MASKED, kPicked, 2>(half_maps, half, piece);
+    block_attn_tc_body<D, 1, 1, MASKED, kPicked, 2>(half_maps, half, piece);
   else
-    block_attn_tc_body<D, 2, 1, 2, MASKED, kPicked, 1>(maps, a, piece);
+    block_attn_tc_body<D, 2, 1, MASKED, kPicked, 1>(maps, a, piece);
 }
 
 template <int D, bool MASKED>
 cudaError_t launch_tc_mixed(const AttnArgs& a, const TmaMaps& maps, const AttnArgs& half, const TmaMaps& half_maps,
                             cudaStream_t stream) {
   constexpr int kBytes =
-      (TcLayout<D, 2, 2>::kBytes > TcLayout<D, 1, 2>::kBytes ? TcLayout<D, 2, 2>::kBytes : TcLayout<D, 1, 2>::kBytes) + 1024;
+      (TcLayout<D, 2>::kBytes > TcLayout<D, 1>::kBytes ? TcLayout<D, 2>::kBytes : TcLayout<D, 1>::kBytes) + 1024;
   static int configured[64] = {0};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -1636,50 +1593,50 @@ cudaError_t launch_tc_mixed(const AttnArgs& a, const TmaMaps& maps, const AttnAr
   }
   if (a.R <= 128 || a.R > 256 || a.num_splits != 1 || half.nh != 2 || half.R <= 64 || half.R > 128 || a.B > 1024 || a.halved > a.B)
     return cudaErrorInvalidValue;
-  return launch_kernel(block_attn_tc_mixed_kernel<D, MASKED>, dim3(a.Hkv, a.B + a.halved), dim3(TcCfg<2, 2>::kThreads), kBytes,
+  return launch_kernel(block_attn_tc_mixed_kernel<D, MASKED>, dim3(a.Hkv, a.B + a.halved), dim3(TcCfg<2>::kThreads), kBytes,
                        stream, maps, a, half_maps, half);
 }
 
-template <int D, int MT, int REP, int TPS, bool MASKED, int ORDER, int CG>
+template <int D, int MT, int REP, bool MASKED, int ORDER, int CG>
 cudaError_t configure_tc(int dev) {
   static int configured[64] = {0};
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!__atomic_load_n(&configured[dev], __ATOMIC_ACQUIRE)) {
-    cudaError_t e = cudaFuncSetAttribute(block_attn_tc_kernel<D, MT, REP, TPS, MASKED, ORDER, CG>,
+    cudaError_t e = cudaFuncSetAttribute(block_attn_tc_kernel<D, MT, REP, MASKED, ORDER, CG>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(TcLayout<D, MT, TPS>::kBytes + 1024));
+                                         static_cast<int>(TcLayout<D, MT>::kBytes + 1024));
     if (e != cudaSuccess) return e;
     __atomic_store_n(&configured[dev], 1, __ATOMIC_RELEASE);
   }
   return cudaSuccess;
 }
 
-template <int D, int MT, int REP, int TPS, bool MASKED, int ORDER, int CG>
+template <int D, int MT, int REP, bool MASKED, int ORDER, int CG>
 cudaError_t launch_tc_o(const AttnArgs& a, const TmaMaps& maps, cudaStream_t stream) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  if ((e = configure_tc<D, MT, REP, TPS, MASKED, ORDER, CG>(dev)) != cudaSuccess) return e;
+  if ((e = configure_tc<D, MT, REP, MASKED, ORDER, CG>(dev)) != cudaSuccess) return e;
   const dim3 grid = ORDER == kBalanced ? dim3(a.balanced_ctas) : dim3(a.num_splits * a.nh, a.Hkv, a.B);
-  return launch_kernel_cluster(block_attn_tc_kernel<D, MT, REP, TPS, MASKED, ORDER, CG>, grid,
-                               dim3(TcCfg<MT, TPS, CG>::kThreads), TcLayout<D, MT, TPS>::kBytes + 1024, stream,
+  return launch_kernel_cluster(block_attn_tc_kernel<D, MT, REP, MASKED, ORDER, CG>, grid,
+                               dim3(TcCfg<MT, CG>::kThreads), TcLayout<D, MT>::kBytes + 1024, stream,
                                a.csize, maps, a);
 }
 
-template <int D, int MT, int REP, int TPS, bool MASKED, int CG = 1>
+template <int D, int MT, int REP, bool MASKED, int CG = 1>
 cudaError_t launch_tc_t(const AttnArgs& a, const TmaMaps& maps, cudaStream_t stream) {
-  if (a.order_by_length) return launch_tc_o<D, MT, REP, TPS, MASKED, kLongestFirst, CG>(a, maps, stream);
+  if (a.order_by_length) return launch_tc_o<D, MT, REP, MASKED, kLongestFirst, CG>(a, maps, stream);
   if constexpr (REP == 1) {  // balanced pieces stream; row copies take short splits
-    if (a.balanced_ctas > 0) return launch_tc_o<D, MT, REP, TPS, MASKED, kBalanced, CG>(a, maps, stream);
+    if (a.balanced_ctas > 0) return launch_tc_o<D, MT, REP, MASKED, kBalanced, CG>(a, maps, stream);
   }
-  return launch_tc_o<D, MT, REP, TPS, MASKED, kGridOrder, CG>(a, maps, stream);
+  return launch_tc_o<D, MT, REP, MASKED, kGridOrder, CG>(a, maps, stream);
 }
 
 // Resident clusters of the kernel a plan would launch (one CTA per SM
 // either way; row copies and score-product width do not change residency,
 // the thread count of two softmax groups does not either, but the query
 // uses the instantiation that runs).
-template <int D, int MT, int REP, int TPS, int CG>
+template <int D, int MT, int REP, int CG>
 int max_active_clusters_t(int csize) {
   static int cache[64][9];  // [device][cluster size] + 1 (0 = not queried)
   int dev = 0;
@@ -1687,11 +1644,11 @@ int max_active_clusters_t(int csize) {
     return 0;
   int v = __atomic_load_n(&cache[dev][csize], __ATOMIC_ACQUIRE);
   if (v) return v - 1;
-  if (configure_tc<D, MT, REP, TPS, false, kGridOrder, CG>(dev) != cudaSuccess) return 0;
+  if (configure_tc<D, MT, REP, false, kGridOrder, CG>(dev) != cudaSuccess) return 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(csize, 1, 1);
-  cfg.blockDim = dim3(TcCfg<MT, TPS, CG>::kThreads);
-  cfg.dynamicSmemBytes = TcLayout<D, MT, TPS>::kBytes + 1024;
+  cfg.blockDim = dim3(TcCfg<MT, CG>::kThreads);
+  cfg.dynamicSmemBytes = TcLayout<D, MT>::kBytes + 1024;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = csize;
@@ -1700,7 +1657,7 @@ int max_active_clusters_t(int csize) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, block_attn_tc_kernel<D, MT, REP, TPS, false, kGridOrder, CG>, &cfg) !=
+  if (cudaOccupancyMaxActiveClusters(&n, block_attn_tc_kernel<D, MT, REP, false, kGridOrder, CG>, &cfg) !=
       cudaSuccess) {
     cudaGetLastError();
     n = 0;
@@ -1715,14 +1672,14 @@ int tc_replication(int rows) { return rows > 32 && rows <= 64 ? 2 : 1; }
 
 // A split of `chunk` tokens sits whole in the ring of the one-M-tile kernels.
 template <int D>
-bool ring_holds(int chunk) { return chunk <= TcLayout<D, 1, 2>::kKStages * kTileTok; }
+bool ring_holds(int chunk) { return chunk <= TcLayout<D, 1>::kKStages * kTileTok; }
 
 template <int D>
 int max_active_clusters_d(int csize, int rows) {
-  if (rows > 128) return max_active_clusters_t<D, 2, 1, 2, 1>(csize);
+  if (rows > 128) return max_active_clusters_t<D, 2, 1, 1>(csize);
   switch (tc_replication(rows)) {
-    case 2: return max_active_clusters_t<D, 1, 2, 2, 1>(csize);
-    default: return max_active_clusters_t<D, 1, 1, 2, 2>(csize);
+    case 2: return max_active_clusters_t<D, 1, 2, 1>(csize);
+    default: return max_active_clusters_t<D, 1, 1, 2>(csize);
   }
 }
 
@@ -1736,9 +1693,9 @@ int max_active_clusters_d(int csize, int rows) {
 template <int D, bool FITS, bool MASKED>  // FITS: a split sits in the ring whole
 cudaError_t launch_tc_rep(const AttnArgs& a, const TmaMaps& maps, cudaStream_t stream) {
   if constexpr (FITS) {
-    if (tc_replication(a.R) == 2) return launch_tc_t<D, 1, 2, 2, MASKED>(a, maps, stream);
+    if (tc_replication(a.R) == 2) return launch_tc_t<D, 1, 2, MASKED>(a, maps, stream);
   }
-  return launch_tc_t<D, 1, 1, 2, MASKED, 2>(a, maps, stream);
+  return launch_tc_t<D, 1, 1, MASKED, 2>(a, maps, stream);
 }
 
 template <int D, bool MASKED>
@@ -1747,9 +1704,9 @@ cudaError_t launch_tc_d(const AttnArgs& a, const TmaMaps& maps, cudaStream_t str
   // grid order take (they read a.nh; the others assume one CTA).
   if (a.nh != 1) {
     if (a.R <= 64 || a.R > 128 || a.order_by_length || a.balanced_ctas > 0) return cudaErrorInvalidValue;
-    return launch_tc_o<D, 1, 1, 2, MASKED, kGridOrder, 2>(a, maps, stream);
+    return launch_tc_o<D, 1, 1, MASKED, kGridOrder, 2>(a, maps, stream);
   }
-  if (a.R > 128) return launch_tc_t<D, 2, 1, 2, MASKED>(a, maps, stream);
+  if (a.R > 128) return launch_tc_t<D, 2, 1, MASKED>(a, maps, stream);
   if (ring_holds<D>(a.chunk)) return launch_tc_rep<D, true, MASKED>(a, maps, stream);
   return launch_tc_rep<D, false, MASKED>(a, maps, stream);
 }

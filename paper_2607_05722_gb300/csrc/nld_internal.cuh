@@ -379,28 +379,11 @@ __device__ __forceinline__ void bulk_load(void* sdst, const void* gsrc, uint32_t
                "l"(gsrc), "r"(bytes), "r"(smem_u32(bar))
                : "memory");
 }
-
-// Bulk copy (TMA engine) of `bytes` from this CTA's shared memory to global
-// memory; both addresses 16-byte aligned, bytes a multiple of 16. The issuing
-// thread must call bulk_store_wait_read() before the source is overwritten or
-// the CTA exits.
-__device__ __forceinline__ void bulk_store(void* gdst, const void* ssrc, uint32_t bytes) {
-  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n\t"
-               "cp.async.bulk.commit_group;" ::"l"(gdst), "r"(smem_u32(ssrc)), "r"(bytes)
-               : "memory");
-}
 __device__ __forceinline__ void bulk_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-
-// Tiled TMA stores shared -> global (one box at coordinates {c0, c1[, c2]},
+// Tiled TMA stores shared -> global (one box at coordinates {c0, c1, c2[, c3]},
 // the innermost coordinate a multiple of 16 bytes), in the issuing thread's
 // bulk group: close it with bulk_commit() and wait with bulk_store_wait_read()
 // before the source is overwritten or the CTA exits.
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, const void* src, int c0, int c1) {
-  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
-                   reinterpret_cast<uint64_t>(map)),
-               "r"(smem_u32(src)), "r"(c0), "r"(c1)
-               : "memory");
-}
 __device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, const void* src, int c0, int c1, int c2) {
   asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(
                    reinterpret_cast<uint64_t>(map)),
