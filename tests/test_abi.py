@@ -222,8 +222,8 @@ def test_plan_wide_pieces_as_halves(L, B, Hkv, D, rows, tokens, halves):
     assert (2 * B * Hkv * plan["splits"] <= 152) == halves
 
 
-# clusters of 2..8 CTAs that run at once on 152 SMs
-RESIDENT = [0, 0, 76, 48, 36, 28, 24, 20, 18]
+# clusters of 2..8 CTAs that run at once on the 152 SMs of a GB300
+RESIDENT = [0, 0, 76, 46, 36, 28, 23, 19, 16]
 
 
 def _route(B, Hq, Hkv, D, P, prefix_max, bl, splits=0, flags=0, mask=False, resident=RESIDENT):

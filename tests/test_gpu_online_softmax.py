@@ -56,15 +56,20 @@ def _lib():
     assert nld.nld_device_error(clear=True) == 0, "a kernel flagged a device error"
 
 
-# name, B, Hq, Hkv, D, P, bl, prefix lengths; packed rows G*bl set the
-# kernel: two softmax groups (<= 32 and 65..128 rows), two row copies
-# (33..64) or two M tiles (> 128)
+# name, B, Hq, Hkv, D, P, bl, prefix lengths; packed rows G*bl and the pieces
+# set the kernel: two softmax groups for up to 128 rows, of 33..64 only in pieces
+# longer than the ring (shorter: two row copies, in a test of their own below);
+# more rows as block-slot halves on that kernel where the block length is even
+# and the wave holds them, with two M tiles where it is odd
 SHAPES = [
     ("rows32_cg2_d64", 1, 4, 1, 64, 16, 8, [700]),
     ("rows64_rep2_d128", 1, 32, 8, 128, 16, 16, [1500]),
     ("rows96_rep1_d128", 2, 6, 2, 128, 16, 32, [900, 400]),
     ("rows160_mt2_d128", 1, 10, 2, 128, 16, 32, [1200]),
     ("rows180_mt2_d64", 1, 6, 1, 64, 32, 30, [800]),
+    ("rows145_odd_mt2_d128", 1, 10, 2, 128, 16, 29, [1200]),
+    ("rows248_odd_mt2_d64", 1, 8, 1, 64, 32, 31, [800]),
+    ("rows248_odd_mt2_d128", 1, 8, 1, 128, 32, 31, [800]),
 ]
 
 BF16_8 = np.uint16(0x4100)  # 8.0
@@ -142,7 +147,7 @@ def test_sink_keys_rescale(orc, spec, strength):
     _check_runs(orc, case, (1, 3, 0))
 
 
-@pytest.mark.parametrize("spec", [SHAPES[0], SHAPES[1], SHAPES[3]], ids=[SHAPES[i][0] for i in (0, 1, 3)])
+@pytest.mark.parametrize("spec", [SHAPES[i] for i in (0, 1, 3, 5, 6)], ids=[SHAPES[i][0] for i in (0, 1, 3, 5, 6)])
 def test_sink_keys_cluster_merges(orc, spec):
     """Explicit split counts that run as thread-block clusters: CTAs whose
     log-sum-exps differ by far more than 2^8 merge through shared memory.
@@ -150,6 +155,28 @@ def test_sink_keys_cluster_merges(orc, spec):
     the first to rescale), so only the 2-piece plan must rescale."""
     case = with_sinks(_case(spec, seed=sum(spec[7]) + 43), 32.0)
     _check_runs(orc, case, (2, 4, 8), must_rescale=(2,))
+
+
+@pytest.mark.parametrize("D,splits", [(128, 5), (64, 4)])
+@pytest.mark.parametrize("strength", [32.0, 14.0], ids=["strong", "mild"])
+def test_row_copies_rescale(orc, D, splits, strength):
+    """33..64 rows in pieces that sit in the ring whole (at most 384 tokens at
+    head_dim 128, 512 at 64): the kernel with two copies of each row, whose
+    copies hold maxima of their own. A piece holds several products, so that the
+    sink run falls behind the first."""
+    case = with_sinks(_case(("rows64", 1, 8, 2, D, 16, 16, [1500]), seed=5), strength)
+    dc = DeviceCase(case)
+    assert nld.nld_block_attn_route(dc.params(splits), 16)["chunk"] <= (384 if D == 128 else 512)
+    _check_runs(orc, case, (splits,), must_rescale=(splits,))
+
+
+@pytest.mark.parametrize("spec", [s for s in SHAPES if "odd" in s[0]], ids=[s[0] for s in SHAPES if "odd" in s[0]])
+def test_odd_blocks_run_on_two_tiles(spec):
+    """What the shapes above named odd are for: one CTA with two M tiles."""
+    dc = DeviceCase(_case(spec, seed=1))
+    for splits in (0, 1, 2, 3, 4, 8):
+        route = nld.nld_block_attn_route(dc.params(splits), spec[6])
+        assert route["halves"] == 1 and route["order"] == 0
 
 
 @pytest.mark.parametrize("spec", SHAPES, ids=[s[0] for s in SHAPES])

@@ -622,7 +622,7 @@ SMALL = [
     # 96 packed rows: one M tile without row copies, several tiles per split
     ("d128_g3_bl32_96rows", 2, 6, 2, 128, 16, 32, [450, 190]),
     ("d64_g4_bl24_96rows", 1, 8, 2, 64, 32, 24, [230]),
-    # two M tiles: the rows past 128 copied 2 or 4 times, or not at all
+    # 160..256 rows of an even block length: block-slot halves in these waves
     ("d128_g6_bl30_180rows", 1, 6, 1, 128, 32, 30, [260]),
     ("d64_g5_bl32_160rows", 2, 10, 2, 64, 16, 32, [300, 45]),
     ("d64_g8_bl32_256rows", 1, 16, 2, 64, 16, 32, [100]),
@@ -632,7 +632,6 @@ SMALL = [
     ("d128_g3_bl32_96rows_15tiles", 1, 6, 2, 128, 16, 32, [900]),
     ("d128_g4_bl32_128rows_17tiles", 1, 8, 2, 128, 16, 32, [1060]),
     # more than 128 rows with an odd block length: one CTA with two M tiles
-    # (an even block length splits the slots over two CTAs instead)
     ("d128_g5_bl29_145rows", 1, 10, 2, 128, 16, 29, [300]),
     ("d64_g8_bl31_248rows", 2, 16, 2, 64, 16, 31, [100, 37]),
 ]
@@ -875,11 +874,13 @@ def test_attention_kv_boxes(orc, D, P, splits):
             compare_attn(out, lse, ro, rl, f"kv boxes D={D} P={P} S={splits} mode={mode} flags={flags}")
 
 
-@pytest.mark.parametrize("G,bl,D", [(43, 3, 128), (5, 32, 128), (8, 31, 64), (8, 32, 128), (129, 1, 64)])
+@pytest.mark.parametrize("G,bl,D", [(43, 3, 128), (5, 32, 128), (8, 31, 64), (8, 31, 128), (8, 32, 128), (129, 1, 64),
+                                     (253, 1, 128)])
 def test_attention_two_row_tiles(orc, G, bl, D):
-    """129..256 packed rows (two M tiles of one CTA): one and more score
-    products of one and two K/V tiles, sequence ends inside a tile, one split,
-    streaming splits and a table mask."""
+    """129..256 packed rows, with an odd block length two M tiles of one CTA,
+    with an even one block-slot halves: one and more score products of one and
+    two K/V tiles, sequence ends inside a tile, one split, streaming splits and
+    a table mask."""
     lens = [0, 40, 130, 700]
     case = W.make_block_attn_case("two_tiles", len(lens), G * 2, 2, D, block_len=bl, page_size=16, prefix_lens=lens,
                                   seed=5)
@@ -897,19 +898,88 @@ def test_attention_two_row_tiles(orc, G, bl, D):
     compare_attn(out2, lse2, ro, rl, f"two tiles G={G} bl={bl} table")
 
 
-def test_attention_halves_of_ragged_sequences(orc):
+@pytest.mark.parametrize("G,bl,D,S", [(8, 32, 128, 3), (8, 32, 64, 3), (15, 16, 128, 3), (7, 32, 128, 4)])
+def test_attention_two_row_tiles_even_blocks(orc, G, bl, D, S):
+    """224..256 packed rows of an even block length in more pieces than the wave
+    holds as halves: two M tiles of one CTA, all rows of both tiles in use."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    B = sms // (4 * S) + 1
+    lens = [(37 * b * b) % 701 for b in range(B)]
+    case = W.make_block_attn_case("two_tiles_even", B, G * 2, 2, D, block_len=bl, page_size=16, prefix_lens=lens,
+                                  seed=15)
+    dc = DeviceCase(case)
+    route = nld.nld_block_attn_route(dc.params(S), bl)
+    assert route["halves"] == 1 and route["cluster"] == 1 and route["order"] == 0
+    rows = rows_per_unit(case, 12, 16)
+    kv = case.kv
+    for mode in (DIFF, VER):
+        ro, rl = orc.block_attn_rows(dc.q_bits(mode), kv.k_bits, kv.v_bits, kv.page_table, kv.prefix_lens,
+                                     case.num_q_heads, case.num_kv_heads, bl, mode, case.scale, rows)
+        out, lse = dc.run(mode, num_splits=S)
+        compare_attn(out[rows[:, 0], rows[:, 1], rows[:, 2]], lse[rows[:, 0], rows[:, 2], rows[:, 1]], ro, rl,
+                     f"two tiles, even blocks, G={G} bl={bl} D={D} S={S} mode={mode}")
+
+
+def _causal_table(bl):
+    """The causal block mask as a table: the masked pass is then the verify pass."""
+    return [(2 << i) - 1 & 0xFFFFFFFF for i in range(bl)]
+
+
+def _check_rows(orc, dc, rows, runs, what):
+    """Each (mode, out, lse) of `runs` against the oracle on `rows`."""
+    case, kv, ref = dc.case, dc.case.kv, {}
+    for i, (mode, out, lse) in enumerate(runs):
+        if mode not in ref:
+            ref[mode] = orc.block_attn_rows(dc.q_bits(mode), kv.k_bits, kv.v_bits, kv.page_table,
+                                            dc.prefix.cpu().numpy(), case.num_q_heads, case.num_kv_heads,
+                                            case.block_len, mode, case.scale, rows)
+        compare_attn(out[rows[:, 0], rows[:, 1], rows[:, 2]], lse[rows[:, 0], rows[:, 2], rows[:, 1]], *ref[mode],
+                     f"{what} run {i} mode={mode}")
+
+
+@pytest.mark.parametrize("D,longest", [(64, 2080), (128, 4400)])
+def test_attention_halves_of_ragged_sequences(orc, D, longest):
     """Unsplit sequences of 129..256 rows as cluster pairs, each CTA half of its
     own sequence, longest first: lengths from empty to the longest, with a half
-    of no key for the shortest."""
-    lens = [0, 1, 47, 48, 50, 64, 111, 112, 113, 200, 500, 2047, 2080] + [90 + 53 * i for i in range(26)]
-    case = W.make_block_attn_case("halves", len(lens), 20, 2, 64, block_len=16, page_size=16, prefix_lens=lens, seed=6)
+    of no key for the shortest; both passes and a table mask."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    lens = [0, 1, 47, 48, 50, 64, 111, 112, 113, 200, 500, 2047, longest]
+    lens += [90 + 53 * i for i in range(max(0, sms // 4 + 1 - len(lens)))]  # 2 KV heads: units over half the SMs
+    case = W.make_block_attn_case("halves", len(lens), 20, 2, D, block_len=16, page_size=16, prefix_lens=lens, seed=6)
     dc = DeviceCase(case)
-    assert nld.nld_block_attn_num_splits(dc.params(), 16) == 1  # merged on chip or never split
-    for mode in (W.MODE_DIFFUSION, W.MODE_VERIFY):
-        ro, rl = oracle_full(orc, case, mode)
-        for flags in (0, nld.NLD_ATTN_PREFIX_READY, nld.NLD_ATTN_NO_CLUSTER):
-            out, lse = dc.run(mode, flags=flags)
-            compare_attn(out, lse, ro, rl, f"halves mode={mode} flags={flags}")
+    route = nld.nld_block_attn_route(dc.params(), 16)
+    assert (route["pieces"], route["cluster"], route["order"]) == (2, 2, 1)
+    runs = [(mode, *dc.run(mode, flags=flags)) for mode in (DIFF, VER)
+            for flags in (0, nld.NLD_ATTN_PREFIX_READY, nld.NLD_ATTN_NO_CLUSTER)]
+    runs.append((VER, *run_masked(dc, _causal_table(16), q=dc.q[VER])))
+    _check_rows(orc, dc, rows_per_unit(case, 20, 7), runs, f"halves D={D}")
+
+
+@pytest.mark.parametrize("k,G,D", [(3, 4, 128), (4, 8, 64), (3, 4, 64), (4, 8, 128)])
+def test_masked_longest_first(orc, k, G, D):
+    """A table mask over more units than SMs and ranges above 2048 tokens: the
+    CTAs take the sequences by length (52 rows: two softmax groups, 168: two M
+    tiles), against the oracle's own table and the causal one's verify pass."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    bl, Hkv = 1 + k + k * k, 4
+    B = sms // Hkv + 2
+    lens = [(53 * b * b) % 300 for b in range(B)]
+    lens[B // 2] = 2100
+    case = W.make_block_attn_case("masked_order", B, G * Hkv, Hkv, D, block_len=bl, page_size=16, prefix_lens=lens,
+                                  seed=17)
+    dc = DeviceCase(case)
+    assert nld.nld_block_attn_route(dc.params(), bl, True)["order"] == 1
+    _check_rows(orc, dc, rows_per_unit(case, 4, 18), [(VER, *run_masked(dc, _causal_table(bl), q=dc.q[VER]))],
+                f"masked order k={k} G={G} D={D}")
+    table = nld.nld_quadss_block_mask(k)
+    small = W.BlockAttnCase(case.name, 8, case.num_q_heads, Hkv, D, bl, case.scale, case.q_draft_bits[:8],
+                            case.q_verify_bits[:8],
+                            W.PagedKV(case.kv.k_bits, case.kv.v_bits, case.kv.page_table[:8], case.kv.prefix_lens[:8],
+                                      16, case.kv.num_pages, case.kv.max_pages))
+    ro, rl, _ = orc.block_attn_masked(small.q_draft_bits, case.kv.k_bits, case.kv.v_bits, small.kv.page_table,
+                                      small.kv.prefix_lens, case.num_q_heads, Hkv, bl, table, case.scale)
+    out, lse = run_masked(dc, table)
+    compare_attn(out[:8], lse[:8], ro, rl, f"masked order quadss k={k} G={G} D={D}")
 
 
 MIXED_LENS = {
@@ -954,47 +1024,67 @@ BALANCED_LENS = {
 
 
 @pytest.mark.parametrize("name", sorted(BALANCED_LENS))
-@pytest.mark.parametrize("G,bl,P", [(4, 8, 16), (5, 32, 64)])
-def test_attention_balanced_pieces(orc, name, G, bl, P):
+@pytest.mark.parametrize("G,bl,P,D", [(4, 8, 16, 64), (5, 32, 64, 64), (4, 8, 16, 128), (5, 32, 64, 128)])
+def test_attention_balanced_pieces(orc, name, G, bl, P, D):
     """Several sequences whose pieces are balanced on the device: equal lengths,
-    one that dwarfs the others, a spread and the most sequences it takes;
-    unused split slots hold no keys, also after a call that used them."""
+    one that dwarfs the others, a spread and the most sequences it takes; both
+    passes and a table mask."""
     lens = BALANCED_LENS[name]
     Hkv = 8 if len(lens) <= 9 else 2
-    case = W.make_block_attn_case("balanced", len(lens), G * Hkv, Hkv, 64, block_len=bl, page_size=P, prefix_lens=lens,
+    case = W.make_block_attn_case("balanced", len(lens), G * Hkv, Hkv, D, block_len=bl, page_size=P, prefix_lens=lens,
                                   seed=8)
     dc = DeviceCase(case)
-    slots = nld.nld_block_attn_num_splits(dc.params(flags=nld.NLD_ATTN_NO_CLUSTER), bl)
-    sms = torch.cuda.get_device_properties(0).multi_processor_count
-    assert slots > 1 and slots * len(lens) * Hkv > sms  # the plans whose pieces are balanced
-    rows = sample_rows(case, 400, 3)
-    kv = case.kv
-    for mode in (W.MODE_DIFFUSION, W.MODE_VERIFY):
-        for flags in (nld.NLD_ATTN_NO_CLUSTER, nld.NLD_ATTN_NO_CLUSTER | nld.NLD_ATTN_PREFIX_READY):
-            out, lse = dc.run(mode, flags=flags)
-            ro, rl = orc.block_attn_rows(dc.q_bits(mode), kv.k_bits, kv.v_bits, kv.page_table, kv.prefix_lens,
-                                         case.num_q_heads, case.num_kv_heads, bl, mode, case.scale, rows)
-            o = out[rows[:, 0], rows[:, 1], rows[:, 2]]
-            l = lse[rows[:, 0], rows[:, 2], rows[:, 1]]
-            compare_attn(o, l, ro, rl, f"balanced {name} G={G} mode={mode} flags={flags}")
+    nc = nld.NLD_ATTN_NO_CLUSTER
+    for masked in (False, True):
+        route = nld.nld_block_attn_route(dc.params(flags=nc), bl, masked)
+        assert route["order"] == 2 and route["pieces"] > 1
+    runs = [(mode, *dc.run(mode, flags=flags)) for mode in (DIFF, VER) for flags in (nc, nc | nld.NLD_ATTN_PREFIX_READY)]
+    if nld.nld_block_attn_route(dc.params(), bl, True)["order"] == 2:
+        runs.append((VER, *run_masked(dc, _causal_table(bl), q=dc.q[VER])))
+    _check_rows(orc, dc, sample_rows(case, 400, 3), runs, f"balanced {name} G={G} D={D}")
 
 
-@pytest.mark.parametrize("B,Hkv,G,bl", [(3, 8, 4, 16), (5, 8, 4, 8), (7, 4, 5, 7), (5, 4, 7, 19)])
-def test_attention_automatic_clusters(orc, B, Hkv, G, bl):
-    """Automatic plans that merge on chip in clusters of any size from 2 to 8:
-    6, 3, 5 and 7 resident CTAs a unit, where the device has them."""
-    lens = [2600 - 517 * b for b in range(B)] if B < 6 else [2600 - 371 * b for b in range(B)]
-    case = W.make_block_attn_case("auto_clusters", B, Hkv * G, Hkv, 64, block_len=bl, page_size=32, prefix_lens=lens,
+@pytest.mark.parametrize("G,bl,D", [(4, 8, 128), (5, 32, 64)])
+def test_balanced_pieces_in_a_used_workspace(orc, G, bl, D):
+    """Split slots that a call leaves unused hold no keys, whatever an earlier
+    call left in them: one workspace, long equal lengths first, then ragged and
+    short ones, the page table as it was."""
+    B, Hkv = 9, 8
+    case = W.make_block_attn_case("reused", B, G * Hkv, Hkv, D, block_len=bl, page_size=16, prefix_lens=[5000] * B,
+                                  seed=19)
+    dc = DeviceCase(case)
+    p = dc.params(flags=nld.NLD_ATTN_NO_CLUSTER)
+    assert nld.nld_block_attn_route(p, bl)["order"] == 2
+    ws = nld.alloc_workspace(p, bl)
+    rows = sample_rows(case, 300, 20)
+    for lens in ([5000] * B, [0, 1, 60, 300, 1000, 1700, 2500, 3600, 5000], [100] * B):
+        dc.prefix = torch.tensor(lens, dtype=torch.int32, device="cuda")
+        runs = []
+        for mode in (DIFF, VER):
+            out = torch.empty((B, bl, G * Hkv, D), dtype=torch.bfloat16, device="cuda")
+            lse = torch.empty((B, G * Hkv, bl), dtype=torch.float32, device="cuda")
+            nld.nld_block_attn(p, dc.q[mode], dc.k, dc.v, dc.table, dc.prefix, bl, mode, out, lse, ws)
+            runs.append((mode, out, lse))
+        _check_rows(orc, dc, rows, runs, f"reused workspace G={G} D={D} longest {max(lens)}")
+
+
+@pytest.mark.parametrize("B,Hkv,G,bl,size", [(3, 8, 4, 16, 5), (5, 8, 4, 8, 3), (7, 4, 5, 7, 5), (5, 4, 7, 19, 6),
+                                              (11, 2, 4, 16, 6)])
+@pytest.mark.parametrize("D", [64, 128])
+def test_attention_automatic_clusters(orc, B, Hkv, G, bl, size, D):
+    """Automatic plans that merge on chip in clusters of 3, 5 and 6 CTAs a unit
+    (the sizes that 152 SMs give; clusters of 7 are resident for 19 units, which
+    plan for 8)."""
+    lens = [2600 - 517 * b for b in range(B)] if B < 6 else [max(0, 2600 - 371 * b) for b in range(B)]
+    case = W.make_block_attn_case("auto_clusters", B, Hkv * G, Hkv, D, block_len=bl, page_size=32, prefix_lens=lens,
                                   seed=9)
     dc = DeviceCase(case)
-    rows = sample_rows(case, 300, 4)
-    kv = case.kv
-    for mode in (W.MODE_DIFFUSION, W.MODE_VERIFY):
-        out, lse = dc.run(mode)
-        ro, rl = orc.block_attn_rows(dc.q_bits(mode), kv.k_bits, kv.v_bits, kv.page_table, kv.prefix_lens,
-                                     case.num_q_heads, case.num_kv_heads, bl, mode, case.scale, rows)
-        compare_attn(out[rows[:, 0], rows[:, 1], rows[:, 2]], lse[rows[:, 0], rows[:, 2], rows[:, 1]], ro, rl,
-                     f"auto clusters B={B} mode={mode}")
+    route = nld.nld_block_attn_route(dc.params(), bl)
+    assert route["partials"] == 1 and nld.nld_block_attn_kernels(dc.params(), bl) == 1
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        assert route["cluster"] == size
+    _check_rows(orc, dc, sample_rows(case, 300, 4), [(mode, *dc.run(mode)) for mode in (DIFF, VER)],
+                f"auto clusters B={B} D={D}")
 
 
 def test_attention_split_sweep(orc):
@@ -1006,14 +1096,16 @@ def test_attention_split_sweep(orc):
         compare_attn(out, lse, ro, rl, f"S={S}")
 
 
-_CLUSTER_SPECS = [SMALL[0], SMALL[8], SMALL[10], SMALL[13], SMALL[11]]
+_CLUSTER_SPECS = [SMALL[0], SMALL[8], SMALL[10], SMALL[13], SMALL[11], SMALL[17], SMALL[18]]
 
 
 @pytest.mark.parametrize("spec", _CLUSTER_SPECS, ids=[s[0] for s in _CLUSTER_SPECS])
 def test_attention_cluster_merges(orc, spec):
     """Explicit split counts of 2/4/8 (one thread-block cluster merging
-    through distributed shared memory) and 16 (clusters of 8, two partials):
-    row copies, one and two M tiles, D = 64 and 128, both passes."""
+    through distributed shared memory) and 16 (clusters of 8, two partials), of
+    pieces with row copies and with one M tile, and with two M tiles where the
+    block length is odd (an even one leaves a partial per piece), D = 64 and
+    128, both passes."""
     name, B, Hq, Hkv, D, P, bl, prefix = spec
     case = W.make_block_attn_case(name, B, Hq, Hkv, D, block_len=bl, page_size=P, prefix_lens=prefix,
                                   seed=sum(prefix) + 11 * bl)
