@@ -93,8 +93,8 @@ struct SplitPlan {
   int partials;  // splits / csize
 };
 
-// Longest split that still runs paired score products at both head sizes
-// (the ring holds at least 6 tiles at head_dim 128).
+// Longest split that sits in the ring whole at both head sizes (6 tiles at
+// head_dim 128).
 constexpr long long kPairedChunk = 384;
 
 // A piece of 129..256 rows runs as two CTAs of half the block slots each where
@@ -181,29 +181,29 @@ void plan_splits_for(const nld_attn_params_t* p, int block_len, int sms, Cluster
     if (clusters && want >= 2 && want <= 8) {
       // The largest cluster resident for every unit at once, not below the
       // power of two under `want` (a third of the SMs idle costs more than the
-      // combine): 8B heads, 3
-      // sequences of 4000 tokens as clusters of 6 15.6 us, of 4 16.4; 5 of 3000
-      // of 3 17.1, of 2 20.4. Sizes between the powers of two only for pieces
-      // of two score products or more (28 units of 912 tokens: 5 pieces 10.5
-      // us, 4 pieces 10.1).
+      // combine): 8B heads, 3 sequences of 4000 tokens as clusters of 5 15.6 us,
+      // of 4 16.4; 5 of 3000 of 3 17.1, of 2 20.4. Sizes between the powers of
+      // two only for pieces of two score products or more (28 units of 912
+      // tokens: 5 pieces 10.5 us, 4 pieces 10.1).
       const int floor2 = want >= 8 ? 8 : want >= 4 ? 4 : 2;
-      // With two M tiles a piece's time goes by its products of 128 tokens: the
-      // fewest CTAs with the fewest products (20 units of 721 tokens, 168 rows, 6
-      // pieces of one product 13.4 us, 4 of one and a half 14.7).
       int cs = want;
-      if (rows > 128) {
+      if (rows <= 128) {
+        while (cs >= floor2 && (units > clusters_resident(cs) || (!is_pow2(cs) && max_tokens < 256 * cs))) --cs;
+      } else {
+        // With two M tiles a piece's time goes by its products of 128 tokens:
+        // the fewest CTAs with the fewest products (20 units of 721 tokens, 168
+        // rows, 6 pieces of one product 13.4 us, 4 of one and a half 14.7).
         const auto products = [&](int n) { return (max_tokens + 128ll * n - 1) / (128ll * n); };
         while (cs >= floor2 && units > clusters_resident(cs)) --cs;
         for (int n = cs - 1; n >= floor2; --n)
           if (products(n) <= products(cs)) cs = n;
       }
-      while (rows <= 128 && cs >= floor2 && (units > clusters_resident(cs) || (!is_pow2(cs) && max_tokens < 256 * cs))) --cs;
       if (cs >= floor2) {
         want = cs;
         csize = cs;
       }
     }
-    // Unsplit units of 129..256 rows that fit in one wave: each runs as a
+    // Unsplit long units of 129..256 rows that fit in one wave: each runs as a
     // cluster of two CTAs that take half of its sequence, longest first, and
     // merge on chip in fp32, so that ragged lengths fill the SMs (14B heads, 16
     // sequences of 8192..16384 tokens: one CTA each 230 us, pairs 197). With
@@ -224,9 +224,8 @@ void plan_splits_for(const nld_attn_params_t* p, int block_len, int sms, Cluster
   long long chunk = (max_tokens + want - 1) / want;
   chunk = (chunk + nld::kGroupTok - 1) / nld::kGroupTok * nld::kGroupTok;
   if (automatic && csize == 1 && tc && chunk <= kPairedChunk) {
-    // Splits short enough for paired score products take whole pairs (128
-    // tokens) when that keeps at least 85% of the splits: no half-filled
-    // product or tile in every CTA (8B shape: 19 splits of 224 tokens become
+    // Short splits take whole products (128 tokens) when that keeps at least
+    // 85% of the splits: no half-filled product or tile in every CTA (8B shape: 19 splits of 224 tokens become
     // 17 of 256, measured faster).
     const long long c2 = (chunk + 2 * nld::kTileTok - 1) / (2 * nld::kTileTok) * (2 * nld::kTileTok);
     const long long s2 = (max_tokens + c2 - 1) / c2;
