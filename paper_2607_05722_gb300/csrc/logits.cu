@@ -4,9 +4,9 @@
 //   m = max_v l_v, id = the lowest v with l_v = m,
 //   conf = max_v softmax(l)_v = 1 / sum_v exp(l_v - m).
 // A row is cut into `split` pieces, one CTA each (a thread-block cluster when
-// split > 1). Pieces of at most 4096 vectors of 8 logits (vocabularies up to
-// 262144) are kept in registers: every thread loads its vectors at once and
-// folds them in one pass. Longer pieces stream: in a CTA one producer warp
+// split > 1). Pieces of at most 4096 vectors of 8 logits are kept in
+// registers: every thread loads its vectors at once and folds them in one pass.
+// Longer pieces stream: in a CTA one producer warp
 // streams the piece through a ring of 16 KB stages with bulk copies (TMA
 // engine) and eight warps fold each 8-logit vector into a running (max, sum
 // of exp(l - max), argmax): the vector max comes first, so the rare rescale
@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(kLgThreads)
   }
 }
 
-// Pieces that fit in a CTA's registers (at most THREADS * kLsMaxVecs 8-logit
+// Pieces that fit in a CTA's registers (at most THREADS * VECS 8-logit
 // vectors): no ring. Every thread loads all its vectors at once (one memory
 // round trip); the logits' max is taken on packed bf16 pairs, then one exp
 // per logit against the warp's max; the index of the max is searched only by
@@ -228,7 +228,8 @@ __global__ void __launch_bounds__(kLgThreads)
 // rules as logits_argmax_kernel (ties to the lower index; NaN never wins and
 // makes the sum NaN; nothing above -inf: id 0, conf 0).
 // Bound: few rows, the chain load - exps - three merges; many rows,
-// instruction issue (51% of the cycles, 7.4 instructions a logit) and CTAs
+// instruction issue (53% of the cycles at 512 rows x 131072, 7.3 instructions a
+// logit) and CTAs
 // that hold their slots through the merges, at 16 rows x 131072 3.6 us (a
 // per-logit max and index search: 4.6), at 512 rows 25.9 us = 5.2 TB/s (the
 // streaming kernel, one CTA a row: 34.7, its 512 CTAs being 1.1 waves), at
@@ -643,10 +644,10 @@ __global__ void __launch_bounds__(kEnThreads)
 // terms ca exp(a - max_a) and cb exp(b - max_b) all lie below 0.49 c cannot
 // hold it: two compares of a vector's maxima decide.
 // Bound by the chain load - sums - exchange - best, during which a CTA holds
-// its registers (ncu at 160 row pairs: 41% of issue cycles, waits at CTA
+// its registers (ncu at 160 row pairs: 43% of issue cycles, waits at CTA
 // barriers first): 160 x 100003 25.1 us (reading both rows twice, with two
-// exponentials a logit each time: 54.6), 16 x 131072 5.5 us (12.7), 512 x
-// 131072 74 us (132).
+// exponentials a logit each time: 54.6, both with the logits in L2), 16 x 131072
+// 5.8 us (12.7), 512 x 131072 72 us (132).
 template <int THREADS, int VECS, bool TAIL>
 __global__ void __launch_bounds__(THREADS, VECS <= 4 ? 1024 / THREADS : 1)
     ensemble_argmax_small_kernel(const __nv_bfloat16* __restrict__ ar, const __nv_bfloat16* __restrict__ diff,
